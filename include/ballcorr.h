@@ -308,6 +308,13 @@ bc_status bc_lift_destroy(bc_lift_t lift);
  *                in FP32 contexts with N <= 128 (BC_ERR_UNSUPPORTED otherwise);
  *                a stalled tensor-core wait is reported by bc_sync as
  *                BC_ERR_TIMEOUT.
+ *                With spread 0 and persistent 0 and shapes that fit inside
+ *                one period (no stencil wraps: 2 n |c|_max / P + W + 4 <= n),
+ *                1 stands for a pass of four launches after the knots'
+ *                preparation instead: spreading into row-pair boxes, the z and
+ *                y transforms of each (level, x) plane in shared memory, the x
+ *                pass, the inverse y and z transforms of whole planes
+ *                (fft_schedule does not apply to it).
  *   persistent   0: the x pass (with the deconvolution, ball transforms, level
  *                sum and conjugate product), the inverse y pass and the
  *                inverse z pass run as three launches; 1: one persistent

@@ -102,6 +102,7 @@ struct Workspace {
     DevBuf cnt, cur, rec;     // binned spreading: bin counts (kept zeroed), bin cursors, knot records
     DevBuf sync;              // work-queue and dependency counters of the persistent back-half launch
     bool grid_dirty = false;  // spreading boxes may hold values (an enqueue failed midway)
+    bool fa_line = false;     // the cached spectrum is laid out [m_z][j_y][j_x] (written by k_xw)
     bool boxes_dirty = true;  // support-box accumulators need their reset state
     bool bins_dirty = false;  // bin counts may be non-zero (an enqueue failed midway)
     std::vector<char> last_desc; // descriptors the device copies hold
@@ -152,6 +153,7 @@ struct bc_ctx_s {
     float2 *tw_n = nullptr, *tw_N = nullptr;
     float *consts = nullptr; // [0] = exp(beta) / I0(beta), then the window's piecewise polynomials
     float *xw = nullptr;     // x-pass level weights (Tables::xw) of the correlation
+    float *wl = nullptr;     // the same for k_xw (Tables::wl), where supported_front
     int *modes = nullptr;    // BC_MOMENTS lowest modes of the half spectrum, (m_x, m_y, m_z) each
     int qmax = 0;
     // device status word
@@ -172,7 +174,7 @@ struct bc_ctx_s {
     Workspace ws;                 // pipeline workspaces of direct calls
     DevBuf outbuf, stats, learn, tune; // host-output staging, shape checks, learned-sweep and tuning scratch
     DevBuf score_ft;                   // shape-complementarity weights for (score_r0, score_lambda)
-    DevBuf score_xw;                   // their x-pass level weights
+    DevBuf score_xw, score_wl;         // their x-pass level weights
     double score_r0 = -1.0, score_lambda = 0.0;
     std::set<bc_shape_s *> shapes; // live shapes; orphaned (device memory freed) by bc_destroy
     std::set<bc_mlp_s *> nets;     // live networks; orphaned the same way
@@ -252,6 +254,7 @@ static Tables tables_of(bc_ctx_t c)
     t.qmax = c->qmax;
     t.consts = c->consts;
     t.xw = c->xw;
+    t.wl = c->wl;
     return t;
 }
 
@@ -379,6 +382,10 @@ bc_status bc_create(const bc_params *p, void *cuda_stream, bc_ctx_t *out)
             return bail(e, "build tables");
         if ((e = cudaMalloc(&c->xw, sizeof(float) * xw_floats(g))) != cudaSuccess) return bail(e, "cudaMalloc xw");
         if ((e = launch_build_xw(g, c->deconv, c->ballft, c->xw, c->stream)) != cudaSuccess) return bail(e, "build x weights");
+        if (supported_front(g)) {
+            if ((e = cudaMalloc(&c->wl, sizeof(float) * wl_floats(g))) != cudaSuccess) return bail(e, "cudaMalloc wl");
+            if ((e = launch_build_wl(g, c->deconv, c->ballft, c->wl, c->stream)) != cudaSuccess) return bail(e, "build level weights");
+        }
         if (g.prec == 0 && g.n == 2 * g.N && supported_z_umma(g.N)) {
             const size_t half = (size_t)(g.n / 2) * 32;
             if ((e = cudaMalloc(&c->zdft, sizeof(float) * 2 * half)) != cudaSuccess) return bail(e, "cudaMalloc zdft");
@@ -404,6 +411,7 @@ bc_status bc_destroy(bc_ctx_t c)
         cudaFree(c->tw_n);
         cudaFree(c->tw_N);
         cudaFree(c->xw);
+        cudaFree(c->wl);
         cudaFree(c->err_dev);
         if (c->pin) cudaFreeHost(c->pin);
         cudaFree(c->consts);
@@ -429,7 +437,7 @@ bc_status bc_destroy(bc_ctx_t c)
         if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
         if (c->ev_a) cudaEventDestroy(c->ev_a);
         if (c->ev_b) cudaEventDestroy(c->ev_b);
-        DevBuf *bufs[] = {&c->outbuf, &c->stats, &c->learn, &c->tune, &c->score_ft, &c->score_xw};
+        DevBuf *bufs[] = {&c->outbuf, &c->stats, &c->learn, &c->tune, &c->score_ft, &c->score_xw, &c->score_wl};
         for (DevBuf *b : bufs) b->release();
         c->hstats.release();
         delete c;
@@ -691,6 +699,10 @@ bc_status bc_profile_end(bc_ctx_t c, bc_profile *out)
             out->bytes[2] = cells * 4.0 + zc * 8.0;
         }
         out->bytes[3] = zc * 8.0 + yc * 8.0;
+        if (c->last_mode == 2) { // z and y in one launch
+            out->bytes[2] = 0.0;
+            out->bytes[3] = cells * 4.0 + yc * 8.0;
+        }
         out->bytes[4] = yc * 8.0 + P * half * 8.0;
         out->bytes[5] = 2.0 * P * half * 8.0;
         out->bytes[6] = P * half * 8.0 + P * N * N * N * 4.0;
@@ -718,6 +730,7 @@ bc_status bc_profile_end(bc_ctx_t c, bc_profile *out)
 struct Weights {
     const float *ballft = nullptr; // null: the context's ball transform table
     const float *xw = nullptr;     // x-pass level weights built from ballft
+    const float *wl = nullptr;     // the same for k_xw
     float sign = 1.f;
 };
 
@@ -730,14 +743,28 @@ struct Job {
     int ztc = 0;   // z pass on the tensor cores (mode 0 only)
     int back = 0;  // x, inverse-y and inverse-z passes as one persistent launch
     int overlap = 0; // passes after k_prepare as programmatic dependents of the pass before
+    int front = 0; // the passes of bc_front.cu and bc_line.cu
     bool yz = false; // inverse y and z of whole planes in one launch (batches of many pairs)
     Weights w;
     int nmain = 0, koff = 0, max_knots = 0, max_cap = 0;
     long long goff = 0, zoff = 0, yoff = 0, hpairs = 0;
 };
 
+// Whether passes over these shapes can take the front and back halves of
+// bc_front.cu and bc_line.cu: FP32, N <= 128, the default choices (spread 0,
+// z_transform 1, persistent 0) and every shape well inside one period, so that no
+// stencil wraps.  Passes that share a cached spectrum decide together.
+static bool front_ok(bc_ctx_t c, std::initializer_list<bc_shape_t> shapes)
+{
+    if (c->spread_mode != 0 || !c->z_tc || c->persistent) return false;
+    for (bc_shape_t s : shapes)
+        if (!front_fits(c->g, cap_extent(c, s->rmax))) return false;
+    return true;
+}
+
 static Job plan_job(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, const std::vector<const float *> &quats,
-                    const std::vector<PairDesc> &pairs, bool cache_first, const std::vector<const float *> *qdev)
+                    const std::vector<PairDesc> &pairs, bool cache_first, const std::vector<const float *> *qdev,
+                    bool front_allowed = true)
 {
     const Geometry &g = c->g;
     const int N = g.N, H = g.H, L = g.L;
@@ -750,6 +777,8 @@ static Job plan_job(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, const std
     j.back = c->persistent;
     j.overlap = c->overlap;
     j.nmain = (int)pairs.size() - (cache_first ? 1 : 0);
+    j.front = front_allowed ? 1 : 0;
+    for (bc_shape_t s : shapes) j.front = j.front && front_ok(c, {s});
     j.inst.resize(shapes.size());
     for (size_t i = 0; i < shapes.size(); i++) {
         bc_shape_t s = shapes[i];
@@ -771,12 +800,16 @@ static Job plan_job(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, const std
             d.q[0] = 1.f;
         }
         if (qdev) d.qdev = (*qdev)[i];
+        d.even = j.front;
         j.koff += s->n;
         j.max_knots = std::max(j.max_knots, s->n);
-        j.goff += (long long)L * e * (((e + 31) / 32) * 32) * e; // block-transposed boxes, y padded to 32
+        // row-pair boxes, even y and z extents; 16-byte vector accesses: every instance starts on 128 bytes
+        if (j.front) j.goff += ((long long)L * e * (e + 1) * (e + 1) + 31) & ~31LL;
+        else j.goff += (long long)L * e * (((e + 31) / 32) * 32) * e; // block-transposed boxes, y padded to 32
         j.zoff += (long long)L * e * e * H;
         j.yoff += (long long)L * e * N * H;
     }
+    if (j.front) j.zoff = 0; // the z-transformed planes stay in shared memory
     for (const PairDesc &p : pairs)
         if (p.b >= 0) j.hpairs = std::max(j.hpairs, p.h_off / ((long long)N * N * H) + 1);
     // plane-wise inverse passes once there are enough planes to fill the device
@@ -851,6 +884,7 @@ static bc_status launch_job(bc_ctx_t c, Workspace &ws, const Job &job, const Ins
     if (job.w.ballft) {
         t.ballft = job.w.ballft;
         t.xw = job.w.xw;
+        t.wl = job.w.wl;
     }
     InstPlan *dplan = (InstPlan *)ws.plan.p;
     const PairDesc *pmain = dpairs + (job.cache_first ? 1 : 0);
@@ -864,6 +898,56 @@ static bc_status launch_job(bc_ctx_t c, Workspace &ws, const Job &job, const Ins
     const bool binned = job.mode == 1;
     mark(-1);
     ws.boxes_dirty = true; // until the plan has consumed and reset the accumulators
+    if (job.front) {
+        // profiled, z and y together are stage 3, inverse y and z stage 6
+        ws.grid_dirty = true; // until the z and y pass has consumed the spreading boxes
+        if ((e = launch_prepare(g, dinst, ninst, job.max_knots, (float4 *)ws.ku.p, (int *)ws.boxes.p, dplan, c->err_dev,
+                                nullptr, nullptr, st)) != cudaSuccess)
+            return cuda_fail(e, "prepare");
+        ws.boxes_dirty = false;
+        mark(0);
+        if ((e = launch_spread_rp(g, t, dinst, job.koff, (const float4 *)ws.ku.p, dplan, (float *)ws.grid.p, st)) != cudaSuccess)
+            return cuda_fail(e, "spread");
+        mark(1);
+        mark(2);
+        if ((e = launch_zy(g, t, dinst, ninst, dplan, (float *)ws.grid.p, (float2 *)ws.y1.p, job.max_cap, c->nsm, st)) != cudaSuccess)
+            return cuda_fail(e, "fft z and y");
+        ws.grid_dirty = false;
+        launches += 2 + (job.koff > 0);
+        mark(3);
+        if (job.cache_first) {
+            if ((e = launch_xw(g, t, dinst, dplan, dpairs, 1, (const float2 *)ws.y1.p, nullptr, (float2 *)ws.fa.p,
+                               (float2 *)ws.h.p, job.max_cap, c->err_dev, c->nsm, st)) != cudaSuccess)
+                return cuda_fail(e, "x pass (cache)");
+            launches++;
+        }
+        if (nmain > 0) {
+            if ((e = launch_xw(g, t, dinst, dplan, pmain, nmain, (const float2 *)ws.y1.p, (const float2 *)ws.fa.p, nullptr,
+                               (float2 *)ws.h.p, job.max_cap, c->err_dev, c->nsm, st)) != cudaSuccess)
+                return cuda_fail(e, "x pass");
+            launches++;
+        }
+        mark(4);
+        mark(5);
+        if (nmain > 0) {
+            if ((e = launch_iyz(g, t, pmain, nmain, (const float2 *)ws.h.p, dout, keys, c->nsm, st)) != cudaSuccess)
+                return cuda_fail(e, "inverse y and z");
+            launches++;
+        }
+        mark(6);
+        if (nlaunch) *nlaunch += launches;
+        if (prof) {
+            c->prof_calls++;
+            c->prof_launches += launches;
+            c->last_ninst = ninst;
+            c->last_npairs = nmain;
+            c->last_mode = 2;
+            c->last_back = 0;
+            c->last_yz = 1;
+            c->last_inst = job.inst;
+        }
+        return BC_OK;
+    }
     if (binned) {
         ws.bins_dirty = true; // until the bin scan has consumed and cleared the counts
         if ((e = launch_prepare(g, dinst, ninst, job.max_knots, (float4 *)ws.ku.p, (int *)ws.boxes.p, dplan,
@@ -975,13 +1059,14 @@ static bc_status launch_job(bc_ctx_t c, Workspace &ws, const Job &job, const Ins
 // on the context's own workspace.
 static bc_status enqueue(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, const std::vector<const float *> &quats,
                          const std::vector<PairDesc> &pairs, bool cache_first, float *dout, unsigned long long *keys,
-                         const std::vector<const float *> *qdev = nullptr, Weights w = Weights())
+                         const std::vector<const float *> *qdev = nullptr, Weights w = Weights(), bool front_allowed = true)
 {
     Workspace &ws = c->ws;
-    Job job = plan_job(c, shapes, quats, pairs, cache_first, qdev);
+    Job job = plan_job(c, shapes, quats, pairs, cache_first, qdev, front_allowed);
     job.w = w;
     const long long ninst = (long long)job.inst.size(), npairs = (long long)job.pairs.size();
     if (bc_status s = ensure_ws(c, ws, job.mode, job.koff, ninst, npairs, job.goff, job.zoff, job.yoff, job.hpairs)) return s;
+    if (cache_first) ws.fa_line = job.front != 0;
     const size_t inst_bytes = sizeof(InstDesc) * ninst, pair_bytes = sizeof(PairDesc) * npairs;
     std::vector<char> desc(inst_bytes + pair_bytes);
     std::memcpy(desc.data(), job.inst.data(), inst_bytes);
@@ -1010,7 +1095,7 @@ static bc_status enqueue(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, cons
     const long long sig[] = {(long long)job.inst.size(), (long long)job.pairs.size(), (long long)job.nmain,
                              (long long)job.cache_first, (long long)job.koff, (long long)job.max_knots,
                              (long long)job.mode, (long long)job.sched, (long long)job.ztc, (long long)job.back,
-                             (long long)job.max_cap, (long long)job.overlap};
+                             (long long)job.max_cap, (long long)job.overlap, (long long)job.front};
     add(sig, sizeof(sig));
     const void *ptrs[] = {dout, keys, job.w.ballft, ws.ku.p, ws.plan.p, ws.inst.p, ws.pairs.p, ws.grid.p, ws.z1.p, ws.y1.p,
                           ws.h.p, ws.fa.p, ws.boxes.p, ws.cnt.p, ws.cur.p, ws.rec.p, ws.sync.p, c->stream};
@@ -1072,11 +1157,12 @@ static bc_status sweep_impl(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float 
     if ((e = c->ws.keys.ensure(key_bytes + out_bytes, false, st)) != cudaSuccess) return cuda_fail(e, "keys");
     unsigned long long *keys = (unsigned long long *)c->ws.keys.p;
     if ((e = cudaMemsetAsync(keys, 0, key_bytes, st)) != cudaSuccess) return cuda_fail(e, "clear keys");
+    const bool front = front_ok(c, {A, B});
     {
         std::vector<bc_shape_t> shapes(1, A);
         std::vector<const float *> q(1, nullptr);
         std::vector<PairDesc> pairs(1, PairDesc{0, -1, 0, 0, 0});
-        if (bc_status s = enqueue(c, shapes, q, pairs, true, nullptr, nullptr, nullptr, w)) return s;
+        if (bc_status s = enqueue(c, shapes, q, pairs, true, nullptr, nullptr, nullptr, w, front)) return s;
     }
     for (int r0 = 0; r0 < k; r0 += batch) {
         const int nb = std::min(batch, k - r0);
@@ -1088,7 +1174,7 @@ static bc_status sweep_impl(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float 
             else qd[i] = qdev + 4 * (size_t)(r0 + i);
             pairs[i] = PairDesc{-1, i, (long long)i * N * N * H, 0, (long long)(r0 + i)};
         }
-        if (bc_status s = enqueue(c, shapes, q, pairs, false, nullptr, keys, qhost ? nullptr : &qd, w)) return s;
+        if (bc_status s = enqueue(c, shapes, q, pairs, false, nullptr, keys, qhost ? nullptr : &qd, w, front)) return s;
     }
     float *dpeak = peak;
     int *darg = argmax;
@@ -1182,16 +1268,20 @@ static bc_status score_weights(bc_ctx_t c, double r0, double lambda, const char 
     const size_t before = c->score_ft.bytes;
     if ((e = c->score_ft.ensure(sizeof(float) * n, false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
     if ((e = c->score_xw.ensure(sizeof(float) * xw_floats(c->g), false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
+    if (c->wl && (e = c->score_wl.ensure(sizeof(float) * wl_floats(c->g), false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
     if (c->score_ft.bytes != before || r0 != c->score_r0 || lambda != c->score_lambda) {
         if ((e = launch_build_score_table(c->g, c->period, c->radii_dev, r0, lambda, (float *)c->score_ft.p, c->stream)) != cudaSuccess)
             return cuda_fail(e, who);
         if ((e = launch_build_xw(c->g, c->deconv, (const float *)c->score_ft.p, (float *)c->score_xw.p, c->stream)) != cudaSuccess)
+            return cuda_fail(e, who);
+        if (c->wl && (e = launch_build_wl(c->g, c->deconv, (const float *)c->score_ft.p, (float *)c->score_wl.p, c->stream)) != cudaSuccess)
             return cuda_fail(e, who);
         c->score_r0 = r0;
         c->score_lambda = lambda;
     }
     w->ballft = (const float *)c->score_ft.p;
     w->xw = (const float *)c->score_xw.p;
+    w->wl = (const float *)c->score_wl.p;
     w->sign = -1.f;
     return BC_OK;
 }
@@ -1327,8 +1417,9 @@ bc_status bc_sweep_plan(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *qua
         pl->k = k;
         // plan every pass on the host
         std::vector<Job> jobs;
+        const bool front = front_ok(c, {A, B});
         jobs.push_back(plan_job(c, std::vector<bc_shape_t>(1, A), std::vector<const float *>(1, nullptr),
-                                std::vector<PairDesc>(1, PairDesc{0, -1, 0, 0, 0}), true, nullptr));
+                                std::vector<PairDesc>(1, PairDesc{0, -1, 0, 0, 0}), true, nullptr, front));
         for (int r0 = 0; r0 < k; r0 += batch) {
             const int nb = std::min(batch, k - r0);
             std::vector<const float *> q(nb);
@@ -1337,7 +1428,7 @@ bc_status bc_sweep_plan(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *qua
                 q[i] = quats + 4 * (size_t)(r0 + i);
                 pairs[i] = PairDesc{-1, i, (long long)i * N * N * H, 0, (long long)(r0 + i)};
             }
-            jobs.push_back(plan_job(c, std::vector<bc_shape_t>(nb, B), q, pairs, false, nullptr));
+            jobs.push_back(plan_job(c, std::vector<bc_shape_t>(nb, B), q, pairs, false, nullptr, front));
         }
         long long mk = 0, mi = 0, mp = 0, mg = 0, mz = 0, my = 0, mh = 0;
         std::vector<size_t> doff(jobs.size());
@@ -1444,7 +1535,7 @@ static bc_status shape_moments(bc_ctx_t c, bc_shape_t S, const float *rot, float
     std::vector<const float *> q(1, rot);
     std::vector<PairDesc> pairs(1, PairDesc{0, -1, 0, 0, 0});
     if (bc_status s = enqueue(c, shapes, q, pairs, true, nullptr, nullptr)) return s;
-    cudaError_t e = launch_moments((const float2 *)c->ws.fa.p, c->modes, BC_MOMENTS, c->g.N, c->g.H, out, c->stream);
+    cudaError_t e = launch_moments((const float2 *)c->ws.fa.p, c->modes, BC_MOMENTS, c->g.N, c->g.H, c->ws.fa_line, out, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "moments");
     return BC_OK;
 }
@@ -2022,13 +2113,14 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
         if (bc_status s = enqueue(c, std::vector<bc_shape_t>(1, A), std::vector<const float *>(1, nullptr), pairs, true,
                                   nullptr, nullptr))
             return bail(s);
+        const bool line_a = c->ws.fa_line;
         if ((e = cudaMemcpyAsync(qo->io.p, c->ws.fa.p, spec, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: copy spectrum"));
         if (bc_status s = enqueue(c, std::vector<bc_shape_t>(1, B), std::vector<const float *>(1, quat), pairs, true,
                                   nullptr, nullptr))
             return bail(s);
         if ((e = launch_query_gather((const float2 *)qo->io.p, (const float2 *)c->ws.fa.p, (const int4 *)qo->modes.p,
-                                     mprime, N, (float2 *)qo->ghat.p, st)) != cudaSuccess)
+                                     mprime, N, line_a, c->ws.fa_line, (float2 *)qo->ghat.p, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: gather"));
         if (bc_status s = bc_sync(c)) return bail(s);
         c->queries.insert(qo);

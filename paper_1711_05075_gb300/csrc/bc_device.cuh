@@ -100,6 +100,10 @@ __device__ __forceinline__ void plan_instance(const Geometry &g, const InstDesc 
         pl.b[a] = b;
         pl.pos0[a] = empty ? 0 : ((L0[a] % g.n) + g.n) % g.n;
     }
+    if (inst[i].even) { // row-pair boxes
+        pl.b[1] = (pl.b[1] + 1) & ~1;
+        pl.b[2] = (pl.b[2] + 1) & ~1;
+    }
     if (empty) pl.b[0] = pl.b[1] = pl.b[2] = 0;
     pl.bzp = (pl.b[2] + 3) & ~3;
     plan[i] = pl;

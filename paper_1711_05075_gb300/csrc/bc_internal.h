@@ -23,6 +23,7 @@ struct InstDesc {
     float q[4];         // rotation (w, x, y, z), unit; identity for A
     const float4 *knots; // the shape's knots (x, y, z, level bits)
     const float *qdev;   // when not null: the rotation is read from this device address instead of q
+    int even, pad_;      // 1: the box's y and z extents are rounded up to even (row-pair boxes, bc_front.cu)
 };
 
 // Device-computed support box of one instance in fine-grid cells.
@@ -53,6 +54,7 @@ struct Tables {
     // [l][a = |m_x| in 0..N/2][16]: ballft_l(a^2 + m_y^2 + m_z^2) D(a) D(m_y) D(m_z)
     // (null: the x pass builds them from ballft and deconv)
     const float *xw;
+    const float *wl;      // k_xw's level weights (bc_line.cu)
 };
 
 struct Geometry {
@@ -83,6 +85,24 @@ cudaError_t launch_reset_boxes(int *bb, int ninst, cudaStream_t s);
 // into bin cursors cur (same size; cnt is left zeroed) for launch_bin.
 cudaError_t launch_prepare(const Geometry &g, const InstDesc *inst, int ninst, int max_knots, float4 *ku, int *bb,
                            InstPlan *plan, int *err, int *cnt, int *cur, cudaStream_t s);
+// Front half (bc_front.cu) and back half (bc_line.cu) of a pass whose instances
+// all fit inside the period (front_fits(g, their largest cap_e); FP32, N <= 128):
+// spreading into row-pair boxes, z and y in one launch (boxes left clear), x with
+// warp-private lines, inverse y and z of whole planes.  Their
+// layouts of y1, h and the cached spectrum differ from the other passes'.
+bool supported_front(const Geometry &g);
+bool front_fits(const Geometry &g, int cap);
+cudaError_t launch_spread_rp(const Geometry &g, const Tables &t, const InstDesc *inst, int total_knots, const float4 *ku,
+                             const InstPlan *plan, float *grid, cudaStream_t s);
+cudaError_t launch_zy(const Geometry &g, const Tables &t, const InstDesc *inst, int ninst, const InstPlan *plan,
+                      float *grid, float2 *y1, int cap, int nsm, cudaStream_t s);
+size_t wl_floats(const Geometry &g);
+cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float *ballft, float *wl, cudaStream_t s);
+cudaError_t launch_xw(const Geometry &g, const Tables &t, const InstDesc *inst, const InstPlan *plan,
+                      const PairDesc *pairs, int npairs, const float2 *y1, const float2 *fa_cache, float2 *fa_out,
+                      float2 *h, int cap, int *err, int nsm, cudaStream_t s);
+cudaError_t launch_iyz(const Geometry &g, const Tables &t, const PairDesc *pairs, int npairs, const float2 *h,
+                       float *out, unsigned long long *keys, int nsm, cudaStream_t s);
 // Binned spreading (bc_binned.cu).  cur[b] = first slot of bin b (the
 // instance's knot_off plus the counts of the bins before it in the instance);
 // launch_bin writes one BIN_REC-float record per knot into its bin (cur[b] is
@@ -166,8 +186,9 @@ void ctx_unregister_mlp(bc_ctx_s *c, bc_mlp_s *net);
 void mlp_orphan(bc_mlp_s *net); // bc_mlp.cu
 
 // Single-configuration queries (bc_query.cu).  modes[i] = (m_x, m_y, m_z, w).
-cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, float2 *ghat,
-                                cudaStream_t s);
+// line_a, line_b: the spectrum is laid out [m_z][j_y][j_x] instead of [j_x][j_y][m_z].
+cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, bool line_a,
+                                bool line_b, float2 *ghat, cudaStream_t s);
 cudaError_t launch_query_eval(const float2 *ghat, const int4 *modes, int count, int N, double period, const float *t,
                               int npts, float *g, cudaStream_t s);
 
@@ -179,7 +200,8 @@ cudaError_t launch_compose_quats(const float *sq, const float *q, int n, float *
 // y = alpha y + beta x (device, n)
 cudaError_t launch_axpby(float *y, const float *x, int n, float alpha, float beta, cudaStream_t s);
 // out[i] = |F(m_i)| / F(0) for the modes[i] = (m_x, m_y, m_z), i < count, of a cached half spectrum.
-cudaError_t launch_moments(const float2 *F, const int *modes, int count, int N, int H, float *out, cudaStream_t s);
+cudaError_t launch_moments(const float2 *F, const int *modes, int count, int N, int H, bool line, float *out,
+                           cudaStream_t s);
 // out[r][i] = |f^_S(R_r^T m_i)| / f^_S(0) for the BC_MOMENTS lowest modes m_i and
 // the n rotations R_r of `quats` (device, n x 4), by direct sums over the nk knots
 // (x, y, z, level bits) with the ball transforms ballft[l (qstride) + |m|^2]; a zero

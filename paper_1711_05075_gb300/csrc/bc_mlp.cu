@@ -833,19 +833,21 @@ cudaError_t bc::launch_topk(const float *scores, int n, int k, int *idx, cudaStr
     return cudaGetLastError();
 }
 
-__global__ void k_moments(const float2 *__restrict__ F, const int *__restrict__ modes, int count, int N, int H, float *out)
+__global__ void k_moments(const float2 *__restrict__ F, const int *__restrict__ modes, int count, int N, int H, bool line,
+                          float *out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const int mx = modes[3 * i], my = modes[3 * i + 1], mz = modes[3 * i + 2];
     const int jx = mx < 0 ? mx + N : mx, jy = my < 0 ? my + N : my;
-    const float2 v = F[((long long)jx * N + jy) * H + mz];
+    const float2 v = F[line ? ((long long)mz * N + jy) * N + jx : ((long long)jx * N + jy) * H + mz];
     out[i] = sqrtf(v.x * v.x + v.y * v.y) / F[0].x;
 }
 
-cudaError_t bc::launch_moments(const float2 *F, const int *modes, int count, int N, int H, float *out, cudaStream_t s)
+cudaError_t bc::launch_moments(const float2 *F, const int *modes, int count, int N, int H, bool line, float *out,
+                               cudaStream_t s)
 {
-    k_moments<<<(count + 63) / 64, 64, 0, s>>>(F, modes, count, N, H, out);
+    k_moments<<<(count + 63) / 64, 64, 0, s>>>(F, modes, count, N, H, line, out);
     return cudaGetLastError();
 }
 

@@ -10,28 +10,28 @@
 
 namespace bc {
 
-// g^ at the listed modes from two half spectra F[jx][jy][mz] (jx, jy in FFT
-// order, mz in [0, N/2)); mode i = (m_x, m_y, m_z, w).
+// g^ at the listed modes from two half spectra F[jx][jy][mz] (line: F[mz][jy][jx];
+// jx, jy in FFT order, mz in [0, N/2)); mode i = (m_x, m_y, m_z, w).
 __global__ void k_query_gather(const float2 *__restrict__ fa, const float2 *__restrict__ fb, const int4 *__restrict__ modes,
-                               int count, int N, float2 *ghat)
+                               int count, int N, bool line_a, bool line_b, float2 *ghat)
 {
     const int H = N / 2;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
         const int4 m = modes[i];
         const int jx = m.x < 0 ? m.x + N : m.x, jy = m.y < 0 ? m.y + N : m.y;
-        const long long o = ((long long)jx * N + jy) * H + m.z;
-        const float2 a = fa[o], b = fb[o];
+        const long long o = ((long long)jx * N + jy) * H + m.z, ol = ((long long)m.z * N + jy) * N + jx;
+        const float2 a = fa[line_a ? ol : o], b = fb[line_b ? ol : o];
         ghat[i] = cmulc(a, b);
     }
 }
 
-cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, float2 *ghat,
-                                cudaStream_t s)
+cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, bool line_a,
+                                bool line_b, float2 *ghat, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
     int blocks = (count + 255) / 256;
     if (blocks > 4096) blocks = 4096;
-    k_query_gather<<<blocks, 256, 0, s>>>(fa, fb, modes, count, N, ghat);
+    k_query_gather<<<blocks, 256, 0, s>>>(fa, fb, modes, count, N, line_a, line_b, ghat);
     return cudaGetLastError();
 }
 
