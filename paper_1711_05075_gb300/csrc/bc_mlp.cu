@@ -855,14 +855,31 @@ cudaError_t bc::launch_moments(const float2 *F, const int *modes, int count, int
 // m_{R S}[i] = |f^_S(R^T m_i)| / f^_S(0) (the moments of S turned by R) by direct
 // sums over the knots, f^_S(k) = sum_i h^(rho_{l_i}, |k|) exp(-2 pi i k . c_i / P)
 // (Eq. (fballhat) without spreading: the band-limited spectrum at off-grid
-// frequencies), for many rotations.  exp(-2 pi i m . R c / P) is the product of
-// u_a^{m_a}, u_a = exp(-i pi (2 / P) (R c)_a): three sincospif per knot, then two
-// complex products per mode.  The mode table is compiled in (the 64 lowest modes
-// are the same for every N >= 8: no component exceeds 3); the context checks it
-// against the one it builds.  One block per rotation: two groups of 128 threads
-// take 32 modes each over all knots (thread j of a group the knots j, j + 128,
-// ...), then warp shuffles and a fixed-order combine of the four warps.
-constexpr int MR_THREADS = 256, MR_GROUP = 32;
+// frequencies), for many rotations.  The mode table is compiled in (the 64 lowest
+// modes are the same for every N >= 8: |m|^2 <= 9, so no component exceeds 3 and
+// two or three nonzero ones are at most 2); the context checks it against the one
+// it builds.
+//
+// With c_a, s_a = cos, sin of m_a 2 pi (R c)_a / P, the phase of a mode is
+// prod_a (c_a - i s_a), so the modes (+-m_x, +-m_y, +-m_z) are signed sums of the
+// 2^d real sums over the knots of h^ prod_a (c_a or s_a), d the number of nonzero
+// components.  Those 122 sums are what a thread accumulates: one FMA per sum and
+// knot, the products of two axes shared by the modes of the third -- a mode
+// costs 2 FMAs per knot instead of up to two complex products and two FMAs (4,096
+// rotations of 5,000 knots: 437 -> 223 us, bound by instruction issue; 167
+// registers, three blocks per SM).  One block per rotation, thread j takes the knots j, j + 128, ...; the sums of a
+// warp are reduced by exchanging halves (each of the five steps halves the
+// values a lane holds), the four warps in a fixed order.
+constexpr int MR_THREADS = 128, MR_SHELLS = 10, MR_SUMS = 128;
+// accumulators: [0] h^(rho, 0); axis a, m = 1 .. 3: 1 + 6 a + 2 (m - 1) + (c, s);
+// axes (0, 1), (0, 2), (1, 2), m, m' = 1, 2: 19 + 16 pair + 8 (m - 1) + 4 (m' - 1) + (cc, cs, sc, ss);
+// three axes, triple t: 67 + 8 t + (ccc, ccs, csc, css, scc, scs, ssc, sss)
+constexpr int MR_ONE = 1, MR_TWO = 19, MR_THREE = 67;
+// the triples (m_x, m_y, m_z) of |m|^2 <= 9: 111, 112, 121, 211, 122, 212, 221
+__host__ __device__ constexpr int mr_triple(int mx, int my, int mz)
+{
+    return mx * my * mz == 1 ? 0 : mx * my * mz == 2 ? (mz == 2 ? 1 : my == 2 ? 2 : 3) : mx == 1 ? 4 : my == 1 ? 5 : 6;
+}
 
 // components of mode i offset by 'D' ('A' = -3 .. 'G' = +3), in the order of the table
 __host__ __device__ constexpr int mr_mode(int i, int a)
@@ -872,98 +889,26 @@ __host__ __device__ constexpr int mr_mode(int i, int a)
            'D';
 }
 
-struct Cpx {
-    float x, y;
-};
-__device__ __forceinline__ Cpx cmul(Cpx a, Cpx b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
-// u^m for |m| <= 3 from p[0..3] = u^0 .. u^3 (u on the unit circle: u^-m = conj(u^m))
-__device__ __forceinline__ Cpx cpow(const Cpx (&p)[4], int m)
+__host__ __device__ constexpr bool mr_covered(int i)
 {
-    const Cpx v = p[m < 0 ? -m : m];
-    return m < 0 ? Cpx{v.x, -v.y} : v;
+    const int x = mr_mode(i, 0), y = mr_mode(i, 1), z = mr_mode(i, 2);
+    return x * x + y * y + z * z < MR_SHELLS && x * x + y * y + z * z > 0;
 }
+template <int... I>
+__host__ __device__ constexpr bool mr_all_covered(std::integer_sequence<int, I...>) { return (mr_covered(I) && ...); }
+static_assert(mr_all_covered(std::make_integer_sequence<int, BC_MOMENTS>{}), "the moment modes lie in |m|^2 <= 9");
 
-// the earlier mode -m_i of the table, or -1 (|f^(-m)| = |f^(m)| for a real density,
-// so such a mode is not summed but copied)
-__host__ __device__ constexpr int mr_twin(int i)
+__global__ void __launch_bounds__(MR_THREADS, 3) k_moments_rot(const float4 *__restrict__ knots, int nk,
+                                                               const float *__restrict__ quats,
+                                                               const float *__restrict__ ballft, int qstride, int L,
+                                                               float two_over_P, float *out, int *err)
 {
-    for (int j = 0; j < i; j++)
-        if (mr_mode(j, 0) == -mr_mode(i, 0) && mr_mode(j, 1) == -mr_mode(i, 1) && mr_mode(j, 2) == -mr_mode(i, 2))
-            return j;
-    return -1;
-}
-
-constexpr int MR_SHELLS = 10; // |m|^2 <= 9 over the table
-
-// exp(-2 pi i m . p / P) from the per-axis powers, skipping the zero components
-template <int MX, int MY, int MZ>
-__device__ __forceinline__ Cpx mr_phase(const Cpx (&u)[3][4])
-{
-    if constexpr (MX != 0 && MY != 0 && MZ != 0) return cmul(cmul(cpow(u[0], MX), cpow(u[1], MY)), cpow(u[2], MZ));
-    else if constexpr (MX != 0 && MY != 0) return cmul(cpow(u[0], MX), cpow(u[1], MY));
-    else if constexpr (MX != 0 && MZ != 0) return cmul(cpow(u[0], MX), cpow(u[2], MZ));
-    else if constexpr (MY != 0 && MZ != 0) return cmul(cpow(u[1], MY), cpow(u[2], MZ));
-    else if constexpr (MX != 0) return cpow(u[0], MX);
-    else if constexpr (MY != 0) return cpow(u[1], MY);
-    else return cpow(u[2], MZ);
-}
-
-// acc[2 j], acc[2 j + 1] += h^(rho_l, |m|) exp(-2 pi i m . p / P) for mode m = M (j = M mod 32)
-template <int M>
-__device__ __forceinline__ void mr_term(const Cpx (&u)[3][4], const float *wq, float (&acc)[2 * MR_GROUP])
-{
-    if constexpr (mr_twin(M) < 0) {
-        constexpr int mx = mr_mode(M, 0), my = mr_mode(M, 1), mz = mr_mode(M, 2), j = M % MR_GROUP;
-        const Cpx t = mr_phase<mx, my, mz>(u);
-        const float w = wq[mx * mx + my * my + mz * mz];
-        acc[2 * j] = fmaf(w, t.x, acc[2 * j]);
-        acc[2 * j + 1] = fmaf(w, t.y, acc[2 * j + 1]);
-    }
-}
-
-template <int G, int... J>
-__device__ __forceinline__ void mr_terms(std::integer_sequence<int, J...>, const Cpx (&u)[3][4], const float *wq,
-                                         float (&acc)[2 * MR_GROUP])
-{
-    (mr_term<G * MR_GROUP + J>(u, wq, acc), ...);
-}
-
-template <int G>
-__device__ __forceinline__ void mr_sums(const float4 *__restrict__ kn, int nk, int j0, const float (&R)[9],
-                                        float two_over_P, const float *wq_all, float (&acc)[2 * MR_GROUP], float &a0)
-{
-    for (int i = j0; i < nk; i += MR_THREADS / 2) {
-        const float4 c = kn[i];
-        const int l = __float_as_int(c.w);
-        const float p[3] = {fmaf(R[0], c.x, fmaf(R[1], c.y, R[2] * c.z)), fmaf(R[3], c.x, fmaf(R[4], c.y, R[5] * c.z)),
-                            fmaf(R[6], c.x, fmaf(R[7], c.y, R[8] * c.z))};
-        Cpx u[3][4];
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            float s, co;
-            sincospif(two_over_P * p[a], &s, &co);
-            u[a][0] = {1.f, 0.f};
-            u[a][1] = {co, -s};
-            u[a][2] = cmul(u[a][1], u[a][1]);
-            u[a][3] = cmul(u[a][2], u[a][1]);
-        }
-        const float *wq = wq_all + l * MR_SHELLS; // h^(rho_l, 2 pi sqrt(q) / P), q = |m|^2
-        mr_terms<G>(std::make_integer_sequence<int, MR_GROUP>{}, u, wq, acc);
-        if (G == 0) a0 += wq[0];
-    }
-}
-
-__global__ void __launch_bounds__(MR_THREADS) k_moments_rot(const float4 *__restrict__ knots, int nk,
-                                                            const float *__restrict__ quats,
-                                                            const float *__restrict__ ballft, int qstride, int L,
-                                                            float two_over_P, float *out, int *err)
-{
-    __shared__ float wq[BC_MAX_LEVELS * MR_SHELLS];
-    __shared__ float red[MR_THREADS / 32][2 * MR_GROUP + 1];
+    __shared__ float wq_all[BC_MAX_LEVELS * MR_SHELLS];
+    __shared__ float red[MR_THREADS / 32][MR_SUMS];
     const int r = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int e = threadIdx.x; e < L * MR_SHELLS; e += MR_THREADS) {
         const int l = e / MR_SHELLS, q = e - l * MR_SHELLS;
-        wq[e] = q < qstride ? ballft[(long long)l * qstride + q] : 0.f;
+        wq_all[e] = q < qstride ? ballft[(long long)l * qstride + q] : 0.f;
     }
     float qw = quats[4 * r], qx = quats[4 * r + 1], qy = quats[4 * r + 2], qz = quats[4 * r + 3];
     const float nq = qw * qw + qx * qx + qy * qy + qz * qz;
@@ -978,38 +923,104 @@ __global__ void __launch_bounds__(MR_THREADS) k_moments_rot(const float4 *__rest
                         2.f * (qx * qy + qw * qz), 1.f - 2.f * (qx * qx + qz * qz), 2.f * (qy * qz - qw * qx),
                         2.f * (qx * qz - qw * qy), 2.f * (qy * qz + qw * qx), 1.f - 2.f * (qx * qx + qy * qy)};
     __syncthreads();
-    float acc[2 * MR_GROUP], a0 = 0.f;
+    float acc[MR_SUMS];
 #pragma unroll
-    for (int j = 0; j < 2 * MR_GROUP; j++) acc[j] = 0.f;
-    const int G = threadIdx.x / (MR_THREADS / 2), j0 = threadIdx.x % (MR_THREADS / 2);
-    if (G == 0) mr_sums<0>(knots, nk, j0, R, two_over_P, wq, acc, a0);
-    else mr_sums<1>(knots, nk, j0, R, two_over_P, wq, acc, a0);
+    for (int j = 0; j < MR_SUMS; j++) acc[j] = 0.f;
+    for (int i = threadIdx.x; i < nk; i += MR_THREADS) {
+        const float4 k = knots[i];
+        const float *wq = wq_all + __float_as_int(k.w) * MR_SHELLS; // h^(rho_l, 2 pi sqrt(q) / P), q = |m|^2
+        float c[3][4], s[3][4]; // cos, sin of m theta_a
 #pragma unroll
-    for (int j = 0; j < 2 * MR_GROUP; j++)
-        for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-    for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-    if (lane == 0) {
+        for (int a = 0; a < 3; a++) {
+            const float p = fmaf(R[3 * a], k.x, fmaf(R[3 * a + 1], k.y, R[3 * a + 2] * k.z));
+            sincospif(two_over_P * p, &s[a][1], &c[a][1]);
+            s[a][2] = 2.f * s[a][1] * c[a][1];
+            c[a][2] = fmaf(c[a][1], c[a][1], -s[a][1] * s[a][1]);
+            s[a][3] = fmaf(s[a][2], c[a][1], c[a][2] * s[a][1]);
+            c[a][3] = fmaf(c[a][2], c[a][1], -s[a][2] * s[a][1]);
+        }
+        acc[0] += wq[0];
 #pragma unroll
-        for (int j = 0; j < 2 * MR_GROUP; j++) red[warp][j] = acc[j];
-        red[warp][2 * MR_GROUP] = a0;
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int m = 1; m <= 3; m++) {
+                float *o = acc + MR_ONE + 6 * a + 2 * (m - 1);
+                o[0] = fmaf(wq[m * m], c[a][m], o[0]);
+                o[1] = fmaf(wq[m * m], s[a][m], o[1]);
+            }
+#pragma unroll
+        for (int pr = 0; pr < 3; pr++) {
+            const int a = pr == 2 ? 1 : 0, b = pr == 0 ? 1 : 2;
+#pragma unroll
+            for (int m = 1; m <= 2; m++)
+#pragma unroll
+                for (int n = 1; n <= 2; n++) {
+                    const float cc = c[a][m] * c[b][n], cs = c[a][m] * s[b][n], sc = s[a][m] * c[b][n], ss = s[a][m] * s[b][n];
+                    const float w = wq[m * m + n * n];
+                    float *o = acc + MR_TWO + 16 * pr + 8 * (m - 1) + 4 * (n - 1);
+                    o[0] = fmaf(w, cc, o[0]);
+                    o[1] = fmaf(w, cs, o[1]);
+                    o[2] = fmaf(w, sc, o[2]);
+                    o[3] = fmaf(w, ss, o[3]);
+                    if (pr == 0)
+#pragma unroll
+                        for (int u = 1; u <= 2; u++) {
+                            if (m * m + n * n + u * u > 9) continue; // 222
+                            const float v = wq[m * m + n * n + u * u], wc = v * c[2][u], ws = v * s[2][u];
+                            float *t = acc + MR_THREE + 8 * mr_triple(m, n, u);
+                            t[0] = fmaf(cc, wc, t[0]);
+                            t[1] = fmaf(cc, ws, t[1]);
+                            t[2] = fmaf(cs, wc, t[2]);
+                            t[3] = fmaf(cs, ws, t[3]);
+                            t[4] = fmaf(sc, wc, t[4]);
+                            t[5] = fmaf(sc, ws, t[5]);
+                            t[6] = fmaf(ss, wc, t[6]);
+                            t[7] = fmaf(ss, ws, t[7]);
+                        }
+                }
+        }
     }
+    // lane l ends with the warp's sums 4 l .. 4 l + 3
+#pragma unroll
+    for (int o = 16, half = MR_SUMS / 2; o > 0; o >>= 1, half >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < half; j++) {
+            const float keep = up ? acc[j + half] : acc[j], send = up ? acc[j] : acc[j + half];
+            acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) red[warp][4 * lane + j] = acc[j];
+    __syncthreads();
+    float sum = red[0][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < MR_THREADS / 32; w++) sum += red[w][threadIdx.x];
+    __syncthreads();
+    float *S = red[0];
+    S[threadIdx.x] = sum;
     __syncthreads();
     if (threadIdx.x < BC_MOMENTS) {
-        int i = threadIdx.x;
-        // a mode whose negation comes earlier takes that one's sum (|f^(-m)| = |f^(m)|)
-        for (int t = 0; t < i; t++)
-            if (mr_mode(t, 0) == -mr_mode(i, 0) && mr_mode(t, 1) == -mr_mode(i, 1) && mr_mode(t, 2) == -mr_mode(i, 2)) {
-                i = t;
-                break;
-            }
-        const int g = i / MR_GROUP, j = i - g * MR_GROUP, wpg = MR_THREADS / 64;
-        float re = 0.f, im = 0.f, f0 = 0.f;
-        for (int w = 0; w < wpg; w++) {
-            re += red[g * wpg + w][2 * j];
-            im += red[g * wpg + w][2 * j + 1];
-            f0 += red[w][2 * MR_GROUP];
+        const int i = threadIdx.x, m[3] = {mr_mode(i, 0), mr_mode(i, 1), mr_mode(i, 2)};
+        const int x = abs(m[0]), y = abs(m[1]), z = abs(m[2]);
+        const float gx = m[0] < 0 ? -1.f : 1.f, gy = m[1] < 0 ? -1.f : 1.f, gz = m[2] < 0 ? -1.f : 1.f; // sines' signs
+        float re, im; // |f^| does not depend on the sign of the imaginary part
+        if (x && y && z) {
+            const float *t = S + MR_THREE + 8 * mr_triple(x, y, z);
+            re = t[0] - gy * gz * t[3] - gx * gz * t[5] - gx * gy * t[6];
+            im = gz * t[1] + gy * t[2] + gx * t[4] - gx * gy * gz * t[7];
+        } else if ((x && y) || (x && z) || (y && z)) {
+            const int pr = x && y ? 0 : x ? 1 : 2, a = pr == 2 ? y : x, b = pr == 0 ? y : z;
+            const float ga = pr == 2 ? gy : gx, gb = pr == 0 ? gy : gz;
+            const float *t = S + MR_TWO + 16 * pr + 8 * (a - 1) + 4 * (b - 1);
+            re = t[0] - ga * gb * t[3];
+            im = gb * t[1] + ga * t[2];
+        } else {
+            const float *t = S + MR_ONE + (x ? 0 : y ? 6 : 12) + 2 * (x + y + z - 1);
+            re = t[0];
+            im = t[1];
         }
-        out[(long long)r * BC_MOMENTS + threadIdx.x] = sqrtf(re * re + im * im) / f0;
+        out[(long long)r * BC_MOMENTS + i] = sqrtf(re * re + im * im) / S[0];
     }
 }
 
