@@ -213,10 +213,14 @@ struct bc_query_s {
     bc_ctx_t ctx = nullptr;
     int count = 0;          // m'
     DevBuf modes, ghat, io; // int4 modes, their g^ values, staging for host points and results
+    // the same modes by columns (m_x, m_y), four columns to a group, weighted (launch_query_lines)
+    DevBuf groups;
+    int ngroups = 0, top = 0; // components below top
     void release()
     {
         modes.release();
         ghat.release();
+        groups.release();
         io.release();
     }
 };
@@ -2075,6 +2079,47 @@ static std::vector<std::array<int, 4>> query_modes(int N, int mprime)
     return out;
 }
 
+// The modes by columns (m_x, m_y), longest first, in the records of
+// launch_query_lines: their heads, and for each of a record's 8-byte places the
+// mode whose weighted g^ belongs there (weight 0 where there is none).
+static void query_columns(const std::vector<std::array<int, 4>> &modes, int N, std::vector<QlGroup> *heads,
+                          std::vector<std::array<int, 4>> *places, int *top)
+{
+    const int h = N / 2, per = (int)(sizeof(QlGroup) / sizeof(float2));
+    std::vector<int> len((size_t)N * N, 0); // by column: highest m_z + 1
+    *top = 1;
+    for (const auto &m : modes) {
+        int &n = len[(size_t)(m[0] + h) * N + m[1] + h];
+        n = std::max(n, m[2] + 1);
+        *top = std::max({*top, std::abs(m[0]) + 1, std::abs(m[1]) + 1, m[2] + 1});
+    }
+    std::vector<int> order;
+    for (int i = 0; i < N * N; i++)
+        if (len[i]) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return len[a] > len[b]; });
+    std::vector<int> first((size_t)N * N, 0); // place of the column's m_z = 0
+    for (size_t q = 0; q < order.size(); q += 4) {
+        const int rows = len[order[q]], g0 = (int)heads->size();
+        for (int z0 = 0; z0 < rows; z0 += QL_ROWS) {
+            QlGroup g;
+            std::memset(&g, 0, sizeof(g));
+            g.rows = std::min(QL_ROWS, rows - z0);
+            g.z0 = z0;
+            for (size_t c = 0; c < 4 && q + c < order.size(); c++) {
+                g.mx[c] = (short)(order[q + c] / N - h);
+                g.my[c] = (short)(order[q + c] % N - h);
+            }
+            heads->push_back(g);
+        }
+        for (size_t c = 0; c < 4 && q + c < order.size(); c++) first[order[q + c]] = g0 * per + QL_HEAD + (int)c;
+    }
+    places->assign(heads->size() * (size_t)per, std::array<int, 4>{0, 0, 0, 0});
+    for (const auto &m : modes) {
+        const size_t at = first[(size_t)(m[0] + h) * N + m[1] + h] + (size_t)(m[2] / QL_ROWS) * per + 4 * (size_t)(m[2] % QL_ROWS);
+        (*places)[at] = m;
+    }
+}
+
 extern "C" {
 
 bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *quat, int mprime, bc_query_t *out)
@@ -2091,11 +2136,17 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
             return fail(BC_ERR_ARG, "bc_query_create: m' must be in [1, ((N-1)^3 + 1) / 2]");
         const std::vector<std::array<int, 4>> modes = query_modes(N, mprime);
         if ((int)modes.size() != mprime) return fail(BC_ERR_INTERNAL, "bc_query_create: mode enumeration");
+        std::vector<QlGroup> heads;
+        std::vector<std::array<int, 4>> places;
+        int top = 1;
+        query_columns(modes, N, &heads, &places, &top);
         cudaStream_t st = c->stream;
         cudaError_t e;
         qo = new bc_query_s();
         qo->ctx = c;
         qo->count = mprime;
+        qo->ngroups = (int)heads.size();
+        qo->top = top;
         const size_t spec = sizeof(float2) * (size_t)N * N * c->g.H;
         auto bail = [&](bc_status s) {
             qo->release();
@@ -2104,10 +2155,19 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
         };
         if ((e = qo->modes.ensure(sizeof(int4) * mprime, false, st)) != cudaSuccess ||
             (e = qo->ghat.ensure(sizeof(float2) * mprime, false, st)) != cudaSuccess ||
-            (e = qo->io.ensure(spec, false, st)) != cudaSuccess)
+            (e = qo->io.ensure(spec, false, st)) != cudaSuccess ||
+            (e = qo->groups.ensure(sizeof(QlGroup) * heads.size(), false, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: buffers"));
         if ((e = cudaMemcpyAsync(qo->modes.p, modes.data(), sizeof(int4) * mprime, cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: modes"));
+        DevBuf lm; // the columns' modes, needed only here
+        struct Drop {
+            DevBuf &b;
+            ~Drop() { b.release(); }
+        } drop{lm};
+        if ((e = lm.ensure(sizeof(int4) * places.size(), false, st)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(lm.p, places.data(), sizeof(int4) * places.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+            return bail(cuda_fail(e, "bc_query_create: columns"));
         // f^_A into the workspace cache, kept in io; then f^_RB into the cache
         std::vector<PairDesc> pairs(1, PairDesc{0, -1, 0, 0, 0});
         if (bc_status s = enqueue(c, std::vector<bc_shape_t>(1, A), std::vector<const float *>(1, nullptr), pairs, true,
@@ -2120,7 +2180,11 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
                                   nullptr, nullptr))
             return bail(s);
         if ((e = launch_query_gather((const float2 *)qo->io.p, (const float2 *)c->ws.fa.p, (const int4 *)qo->modes.p,
-                                     mprime, N, line_a, c->ws.fa_line, (float2 *)qo->ghat.p, st)) != cudaSuccess)
+                                     mprime, N, line_a, c->ws.fa_line, false, (float2 *)qo->ghat.p, st)) != cudaSuccess ||
+            (e = launch_query_gather((const float2 *)qo->io.p, (const float2 *)c->ws.fa.p, (const int4 *)lm.p, (int)places.size(),
+                                     N, line_a, c->ws.fa_line, true, (float2 *)qo->groups.p, st)) != cudaSuccess ||
+            (e = cudaMemcpy2DAsync(qo->groups.p, sizeof(QlGroup), heads.data(), sizeof(QlGroup), QL_HEAD * sizeof(float2),
+                                   heads.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: gather"));
         if (bc_status s = bc_sync(c)) return bail(s);
         c->queries.insert(qo);
@@ -2155,8 +2219,16 @@ bc_status bc_query_eval(bc_query_t q, const float *t, int npts, float *g, int on
             dt = stage;
             dg = stage + 3 * (size_t)npts;
         }
-        if ((e = launch_query_eval((const float2 *)q->ghat.p, (const int4 *)q->modes.p, q->count, c->g.N, c->period, dt,
-                                   npts, dg, st)) != cudaSuccess)
+        // k_query_eval takes a block per point, eight resident per SM: up to that many
+        // points it runs in one wave and spreads the modes over every SM (4,096 modes:
+        // 8.5 to 12.4 us for 1 to 1,024 points); beyond, it grows with the points (20 us
+        // at 2,048, 31 at 4,096, 121 at 20,000) and k_query_lines (14.4, 14.4, 45 us) is
+        // the faster one, at any number of modes (64 .. 100,000 measured)
+        e = npts > 8 * c->nsm
+                ? launch_query_lines((const QlGroup *)q->groups.p, q->ngroups, q->top, c->period, dt, npts, dg, st)
+                : launch_query_eval((const float2 *)q->ghat.p, (const int4 *)q->modes.p, q->count, c->g.N, c->period, dt, npts,
+                                    dg, st);
+        if (e != cudaSuccess)
             return cuda_fail(e, "bc_query_eval: launch");
         if (!on_device) {
             if ((e = cudaMemcpyAsync(g, dg, sizeof(float) * (size_t)npts, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
