@@ -702,6 +702,179 @@ __global__ void k_axpby(float *y, const float *__restrict__ x, int n, float alph
     if (i < n) y[i] = alpha * y[i] + beta * x[i];
 }
 
+// ------------------------------------------------------------------ fused forward pass
+// Both hidden layers and the output of 128 rows in one block (hidden <= FW_MAXH):
+//   h1 = relu(W1 x + b1), h2 = relu(W2 h1 + b2), y = w3 . h2 + b3.
+// The weights come as BF16 blocks already in the tensor core's swizzled layout
+// (k_pack_weights, once per parameter change) by bulk copies: W1's three K blocks
+// of 64 and the first of W2 at the start, W2's other blocks into W1's place once
+// the first product is done.  The rows of X are rounded to BF16 by the threads; h1
+// goes from tensor memory through the bias and the ReLU straight into the second
+// product's operand tile.  With STORE the layers are also written out (FP32) for
+// the gradients.  Same operands, same order of accumulation as k_gemm_umma.
+constexpr int FW_MAXH = 256, FW_SLOTS = 4;
+
+int fw_hp(int H) { return (H + 63) & ~63; }
+int fw_smem(int H) { return 1024 + 4 * GU_A_BYTES + FW_SLOTS * H * 128 + 128 * 4 + 128; }
+
+// W1p[3][H][64], W2p[hp / 64][H][64] BF16, rows of 128 bytes swizzled as st_chunk does, zero beyond K
+__global__ void k_pack_weights(const float *__restrict__ W1, const float *__restrict__ W2, int H, int hp, uint8_t *W1p,
+                               uint8_t *W2p)
+{
+    const int n1 = 3 * H * 8, n2 = hp / 64 * H * 8;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 + n2; e += gridDim.x * blockDim.x) {
+        const bool first = e < n1;
+        const int q = first ? e : e - n1, j = q & 7, r = (q >> 3) % H, kb = (q >> 3) / H;
+        const int K = first ? KIN : H, k0 = 64 * kb + 8 * j;
+        const float *src = (first ? W1 : W2) + (long long)r * K;
+        float x[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) x[k] = k0 + k < K ? src[k0 + k] : 0.f;
+        st_chunk((first ? W1p : W2p) + (size_t)kb * H * 128, r, j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+    }
+}
+
+template <bool STORE>
+__global__ void __launch_bounds__(GU_THREADS, 1)
+k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, const uint8_t *__restrict__ W1p,
+              const uint8_t *__restrict__ W2p, const float *__restrict__ b1, const float *__restrict__ b2,
+              const float *__restrict__ w3, const float *__restrict__ b3, float *h1, float *h2, float *y, int *err)
+{
+    extern __shared__ uint8_t gu_raw[];
+    const uint32_t raw = smem_addr(gu_raw), base = (raw + 1023u) & ~1023u;
+    uint8_t *ga = gu_raw + (base - raw); // operand rows: four K blocks of 128 rows
+    const uint32_t slot0 = base + 4 * GU_A_BYTES, sbytes = (uint32_t)H * 128;
+    float *ys = reinterpret_cast<float *>(ga + 4 * GU_A_BYTES + FW_SLOTS * sbytes);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(ys + 128);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 6);
+    volatile int *stop = reinterpret_cast<volatile int *>(tslot + 1);
+    const uint32_t WB = smem_addr(bars), MD = WB + 8 * FW_SLOTS; // weights in slot k; product 1, 2 done
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m0 = blockIdx.x * 128, kb2 = hp / 64;
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < FW_SLOTS + 2; k++) mbar_init(WB + 8 * k, 1);
+        *stop = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int k = 0; k < FW_SLOTS; k++) {
+            mbar_expect_tx(WB + 8 * k, sbytes);
+            bulk_g2s(slot0 + k * sbytes, k < 3 ? W1p + (size_t)k * sbytes : W2p, sbytes, WB + 8 * k);
+        }
+    }
+    if (warp == 0) {
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)), "r"(tcols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int kb = 0; kb < 3; kb++) gu_tile(ga + kb * GU_A_BYTES, X, KPAD, 1, m0, 128, n, 64 * kb, KIN, -1);
+    fence_proxy_async_smem(); // the tile stores are visible to the tensor core's reads
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot, idesc = umma_idesc_bf16(H), d2 = tmem + (uint32_t)(tcols / 2);
+    bool ok = true, loads2 = false, mma2 = false;
+    if (threadIdx.x == 0) {
+        for (int kb = 0; kb < 3 && ok; kb++) {
+            ok = umma_wait(WB + 8 * kb, 0, stop, err, GU_ERR);
+            if (!ok) break;
+            const uint32_t a = base + kb * GU_A_BYTES, b = slot0 + kb * sbytes;
+            for (int k = 0; k < (kb < 2 ? 4 : 1); k++) // K = 16 per MMA: 144 of the 192 columns
+                umma_bf16(tmem, umma_desc_sw128(a + 32 * k), umma_desc_sw128(b + 32 * k), idesc, kb + k > 0);
+        }
+        umma_commit(MD);
+    }
+    ok = __syncthreads_and(umma_wait(MD, 0, stop, err, GU_ERR) && ok);
+    if (ok) {
+        tc_fence_after();
+        if (threadIdx.x == 0 && kb2 > 1) { // W1 is used: W2's other blocks take its slots
+            for (int k = 0; k < kb2 - 1; k++) {
+                mbar_expect_tx(WB + 8 * k, sbytes);
+                bulk_g2s(slot0 + k * sbytes, W2p + (size_t)(k + 1) * sbytes, sbytes, WB + 8 * k);
+            }
+        }
+        loads2 = true;
+        const int q = warp & 3, half = warp >> 2, r = 32 * q + lane, row = m0 + r;
+        for (int c0 = 16 * half; c0 < hp; c0 += 32) {
+            float x[16];
+            if (c0 < H) {
+                uint32_t v[16];
+                tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; j++) x[j] = fmaxf(__uint_as_float(v[j]) + __ldg(b1 + c0 + j), 0.f);
+                if (STORE && row < n) {
+                    float4 *o = reinterpret_cast<float4 *>(h1 + (long long)row * H + c0);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) o[k] = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; j++) x[j] = 0.f;
+            }
+            uint8_t *t = ga + (c0 >> 6) * GU_A_BYTES;
+            const int j0 = (c0 & 63) >> 3;
+            st_chunk(t, r, j0, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+            st_chunk(t, r, j0 + 1, x[8], x[9], x[10], x[11], x[12], x[13], x[14], x[15]);
+        }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (threadIdx.x == 0) {
+            for (int kb = 0; kb < kb2 && ok; kb++) {
+                const int sl = kb == 0 ? 3 : kb - 1;
+                ok = umma_wait(WB + 8 * sl, kb == 0 ? 0 : 1, stop, err, GU_ERR);
+                if (!ok) break;
+                const uint32_t a = base + kb * GU_A_BYTES, b = slot0 + sl * sbytes;
+                for (int k = 0; k < min(4, (H - 64 * kb) / 16); k++)
+                    umma_bf16(d2, umma_desc_sw128(a + 32 * k), umma_desc_sw128(b + 32 * k), idesc, kb + k > 0);
+            }
+            umma_commit(MD + 8);
+        }
+        mma2 = true;
+        ok = __syncthreads_and(umma_wait(MD + 8, 0, stop, err, GU_ERR) && ok);
+        if (ok) {
+            tc_fence_after();
+            float s = 0.f;
+            for (int c0 = 16 * half; c0 < H; c0 += 32) {
+                uint32_t v[16];
+                float x[16];
+                tmem_ld16(d2 + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    x[j] = fmaxf(__uint_as_float(v[j]) + __ldg(b2 + c0 + j), 0.f);
+                    if (!STORE) s = fmaf(rbf(x[j]), rbf(__ldg(w3 + c0 + j)), s);
+                }
+                if (STORE && row < n) {
+                    float4 *o = reinterpret_cast<float4 *>(h2 + (long long)row * H + c0);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) o[k] = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+                }
+            }
+            if (!STORE) { // the training pass takes y from its own head (k_head_train)
+                if (half == 1) ys[r] = s;
+                __syncthreads();
+                if (half == 0 && row < n) y[row] = s + ys[r] + b3[0];
+            }
+        }
+    }
+    if (!ok && threadIdx.x == 0) {
+        // a wait expired: copies and MMAs in flight finish (bounded) before the memory goes
+        auto drain = [&](uint32_t bar, uint32_t par) {
+            const uint64_t t0 = global_ns();
+            while (!mbar_test(bar, par) && global_ns() - t0 < UMMA_WAIT_NS) {
+            }
+        };
+        for (int k = 0; k < FW_SLOTS; k++) drain(WB + 8 * k, loads2 && k < kb2 - 1 ? 1 : 0);
+        drain(MD, 0);
+        if (mma2) drain(MD + 8, 0);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
+    }
+}
+
 } // namespace
 
 // ------------------------------------------------------------------ network object
@@ -719,6 +892,8 @@ struct bc_mlp_s {
     float *xb = nullptr, *tb = nullptr; // a gathered training batch (bc_mlp_train)
     int xb_cap = 0;
     float *loss = nullptr;
+    uint8_t *wp = nullptr;        // BF16 weights in the fused forward pass's layout (hidden <= FW_MAXH)
+    bool packed = false;          // they hold the current parameters
     int rotated_moments = 0;      // the ligand features are the moments of the rotated ligand (bc_mlp_set_features)
 };
 
@@ -766,9 +941,32 @@ bc_status ensure_batch(bc_mlp_t net, int n)
     return BC_OK;
 }
 
+// The fused forward pass: the layers into net->h1, net->h2 (store), else y.  It needs
+// X on a 16-byte boundary only for speed; H a multiple of 16 up to FW_MAXH.
+bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, bool store, cudaStream_t s)
+{
+    const int H = net->H, hp = fw_hp(H);
+    const Offsets &o = net->off;
+    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128;
+    if (!net->packed) {
+        k_pack_weights<<<(3 * H * 8 + hp / 64 * H * 8 + 255) / 256, 256, 0, s>>>(net->p + o.W1, net->p + o.W2, H, hp, W1p, W2p);
+        MCK(cudaGetLastError());
+        net->packed = true;
+    }
+    int tcols = 32; // two accumulators of H columns
+    while (tcols < 2 * H) tcols <<= 1;
+    const int smem = fw_smem(H);
+    auto kernel = store ? k_mlp_forward<true> : k_mlp_forward<false>;
+    kernel<<<(n + 127) / 128, GU_THREADS, smem, s>>>(X, n, H, hp, tcols, W1p, W2p, net->p + o.b1, net->p + o.b2, net->p + o.w3,
+                                                     net->p + o.b3, net->h1, net->h2, y, ctx_err(net->ctx));
+    MCK(cudaGetLastError());
+    return BC_OK;
+}
+
 // the hidden layers into net->h1, net->h2
 bc_status hidden_layers(bc_mlp_t net, const float *X, int n, cudaStream_t s)
 {
+    if (net->wp) return fused_forward(net, X, n, nullptr, true, s);
     const int H = net->H;
     const Offsets &o = net->off;
     GemmArgs a1{X, KPAD, 1, net->p + o.W1, 1, KIN, net->h1, H, 1, n, H, KPAD, net->p + o.b1, 1};
@@ -786,6 +984,7 @@ bc_status hidden_layers(bc_mlp_t net, const float *X, int n, cudaStream_t s)
 // forward pass into net->h1, net->h2, y
 bc_status forward(bc_mlp_t net, const float *X, int n, float *y, cudaStream_t s)
 {
+    if (net->wp) return fused_forward(net, X, n, y, false, s);
     if (bc_status st = hidden_layers(net, X, n, s)) return st;
     const Offsets &o = net->off;
     k_head<<<(n + 7) / 8, 256, 0, s>>>(net->h2, net->p + o.w3, net->p + o.b3, n, net->H, y);
@@ -1069,6 +1268,9 @@ void bc::mlp_orphan(bc_mlp_s *net)
         if (b) cudaFree(b);
     net->p = net->m = net->v = net->g = net->h1 = net->h2 = net->y = net->gy = net->dh2 = net->dh1 = net->loss = nullptr;
     net->part = net->xb = net->tb = nullptr;
+    if (net->wp) cudaFree(net->wp);
+    net->wp = nullptr;
+    net->packed = false;
     net->cap = net->xb_cap = 0;
     net->part_floats = 0;
     net->ctx = nullptr;
@@ -1095,6 +1297,14 @@ bc_status bc_mlp_create(bc_ctx_t ctx, int hidden, const float *init, bc_mlp_t *o
             (e = cudaMalloc(&net->loss, sizeof(float))) != cudaSuccess) {
             bc_mlp_destroy(net);
             return mcuda(e, "bc_mlp_create: cudaMalloc");
+        }
+        if (hidden <= FW_MAXH) {
+            if ((e = cudaMalloc(&net->wp, (size_t)(3 + fw_hp(hidden) / 64) * hidden * 128)) != cudaSuccess ||
+                (e = cudaFuncSetAttribute(k_mlp_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess ||
+                (e = cudaFuncSetAttribute(k_mlp_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess) {
+                bc_mlp_destroy(net);
+                return mcuda(e, "bc_mlp_create: fused forward pass");
+            }
         }
         if ((e = cudaMemcpyAsync(net->p, init, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(net->m, 0, bytes, s)) != cudaSuccess || (e = cudaMemsetAsync(net->v, 0, bytes, s)) != cudaSuccess ||
@@ -1200,6 +1410,7 @@ bc_status bc_mlp_train_step(bc_mlp_t net, const float *X, const float *t, int n,
         k_adam<<<(unsigned)((total + 255) / 256), 256, 0, ctx_stream(net->ctx)>>>(net->p, net->m, net->v, net->g, total, lr,
                                                                                  b1, b2, eps, c1, c2);
         MCK(cudaGetLastError());
+        net->packed = false;
         return BC_OK;
     } catch (...) {
         return mfail(BC_ERR_INTERNAL, "bc_mlp_train_step: unexpected exception");
@@ -1276,6 +1487,7 @@ bc_status bc_mlp_train(bc_mlp_t net, const float *X, const float *t, int n, int 
                 k_adam<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(net->p, net->m, net->v, net->g, total, lr_e, b1,
                                                                       b2, eps, c1, c2);
                 MCK(cudaGetLastError());
+                net->packed = false;
             }
         }
         if (loss) {
@@ -1300,6 +1512,7 @@ bc_status bc_mlp_state(bc_mlp_t net, float *params, float *m, float *v, long lon
         if (!host[i]) continue;
         if (get) MCK(cudaMemcpyAsync(host[i], dev[i], bytes, cudaMemcpyDeviceToHost, s));
         else MCK(cudaMemcpyAsync(dev[i], host[i], bytes, cudaMemcpyHostToDevice, s));
+        if (!get && i == 0) net->packed = false;
     }
     MCK(cudaStreamSynchronize(s));
     if (step) {
