@@ -384,10 +384,12 @@ bc_status bc_create(const bc_params *p, void *cuda_stream, bc_ctx_t *out)
             return bail(e, "copy radii");
         if ((e = launch_build_tables(g, beta, p->period, c->radii_dev, c->deconv, c->ballft, c->tw_n, c->tw_N, c->consts, c->stream)) != cudaSuccess)
             return bail(e, "build tables");
-        if ((e = cudaMalloc(&c->xw, sizeof(float) * xw_floats(g))) != cudaSuccess) return bail(e, "cudaMalloc xw");
+        const size_t xwf = (xw_floats(g) + 63) & ~size_t(63); // one allocation for both forms of the level weights
+        if ((e = cudaMalloc(&c->xw, sizeof(float) * (xwf + (supported_front(g) ? wl_floats(g) : 0)))) != cudaSuccess)
+            return bail(e, "cudaMalloc xw");
         if ((e = launch_build_xw(g, c->deconv, c->ballft, c->xw, c->stream)) != cudaSuccess) return bail(e, "build x weights");
         if (supported_front(g)) {
-            if ((e = cudaMalloc(&c->wl, sizeof(float) * wl_floats(g))) != cudaSuccess) return bail(e, "cudaMalloc wl");
+            c->wl = c->xw + xwf;
             if ((e = launch_build_wl(g, c->deconv, c->ballft, c->wl, c->stream)) != cudaSuccess) return bail(e, "build level weights");
         }
         if (g.prec == 0 && g.n == 2 * g.N && supported_z_umma(g.N)) {
@@ -415,7 +417,6 @@ bc_status bc_destroy(bc_ctx_t c)
         cudaFree(c->tw_n);
         cudaFree(c->tw_N);
         cudaFree(c->xw);
-        cudaFree(c->wl);
         cudaFree(c->err_dev);
         if (c->pin) cudaFreeHost(c->pin);
         cudaFree(c->consts);

@@ -710,42 +710,51 @@ __global__ void k_axpby(float *y, const float *__restrict__ x, int n, float alph
 // of 64 and the first of W2 at the start, W2's other blocks into W1's place once
 // the first product is done.  The rows of X are rounded to BF16 by the threads; h1
 // goes from tensor memory through the bias and the ReLU straight into the second
-// product's operand tile.  With STORE the layers are also written out (FP32) for
-// the gradients.  Same operands, same order of accumulation as k_gemm_umma.
+// product's operand tile.  Same operands, same order of accumulation as
+// k_gemm_umma.  16,384 rows at 256 hidden: 47 us in three launches -> 12.3 us,
+// most of it the latency of its chain (weights, two products, two epilogues).
 constexpr int FW_MAXH = 256, FW_SLOTS = 4;
 
 int fw_hp(int H) { return (H + 63) & ~63; }
-int fw_smem(int H) { return 1024 + 4 * GU_A_BYTES + FW_SLOTS * H * 128 + 128 * 4 + 128; }
+int fw_smem(int H) { return 1024 + 4 * GU_A_BYTES + FW_SLOTS * H * 128 + 4 * (128 + 3 * FW_MAXH) + 128; }
 
-// W1p[3][H][64], W2p[hp / 64][H][64] BF16, rows of 128 bytes swizzled as st_chunk does, zero beyond K
+// W1p[3][H][64], W2p[hp / 64][H][64] and, when wanted, W2T (row h_in, column h_out) BF16, rows of 128
+// bytes swizzled as st_chunk does, zero beyond K
 __global__ void k_pack_weights(const float *__restrict__ W1, const float *__restrict__ W2, int H, int hp, uint8_t *W1p,
-                               uint8_t *W2p)
+                               uint8_t *W2p, uint8_t *W2T)
 {
-    const int n1 = 3 * H * 8, n2 = hp / 64 * H * 8;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 + n2; e += gridDim.x * blockDim.x) {
-        const bool first = e < n1;
-        const int q = first ? e : e - n1, j = q & 7, r = (q >> 3) % H, kb = (q >> 3) / H;
-        const int K = first ? KIN : H, k0 = 64 * kb + 8 * j;
-        const float *src = (first ? W1 : W2) + (long long)r * K;
+    const int n1 = 3 * H * 8, n2 = hp / 64 * H * 8, n3 = W2T ? n2 : 0;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 + n2 + n3; e += gridDim.x * blockDim.x) {
         float x[8];
+        if (e < n1 + n2) {
+            const bool first = e < n1;
+            const int q = first ? e : e - n1, j = q & 7, r = (q >> 3) % H, kb = (q >> 3) / H;
+            const int K = first ? KIN : H, k0 = 64 * kb + 8 * j;
+            const float *src = (first ? W1 : W2) + (long long)r * K;
 #pragma unroll
-        for (int k = 0; k < 8; k++) x[k] = k0 + k < K ? src[k0 + k] : 0.f;
-        st_chunk((first ? W1p : W2p) + (size_t)kb * H * 128, r, j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+            for (int k = 0; k < 8; k++) x[k] = k0 + k < K ? src[k0 + k] : 0.f;
+            st_chunk((first ? W1p : W2p) + (size_t)kb * H * 128, r, j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+        } else { // neighbouring threads: neighbouring h_in
+            const int q = e - n1 - n2, r = q % H, j = (q / H) & 7, kb = q / H / 8, k0 = 64 * kb + 8 * j;
+#pragma unroll
+            for (int k = 0; k < 8; k++) x[k] = k0 + k < H ? W2[(long long)(k0 + k) * H + r] : 0.f;
+            st_chunk(W2T + (size_t)kb * H * 128, r, j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+        }
     }
 }
 
-template <bool STORE>
 __global__ void __launch_bounds__(GU_THREADS, 1)
 k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, const uint8_t *__restrict__ W1p,
               const uint8_t *__restrict__ W2p, const float *__restrict__ b1, const float *__restrict__ b2,
-              const float *__restrict__ w3, const float *__restrict__ b3, float *h1, float *h2, float *y, int *err)
+              const float *__restrict__ w3, const float *__restrict__ b3, float *y, int *err)
 {
     extern __shared__ uint8_t gu_raw[];
     const uint32_t raw = smem_addr(gu_raw), base = (raw + 1023u) & ~1023u;
     uint8_t *ga = gu_raw + (base - raw); // operand rows: four K blocks of 128 rows
     const uint32_t slot0 = base + 4 * GU_A_BYTES, sbytes = (uint32_t)H * 128;
     float *ys = reinterpret_cast<float *>(ga + 4 * GU_A_BYTES + FW_SLOTS * sbytes);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(ys + 128);
+    float *b1s = ys + 128, *b2s = b1s + FW_MAXH, *w3s = b2s + FW_MAXH; // biases, w3 rounded to BF16
+    uint64_t *bars = reinterpret_cast<uint64_t *>(w3s + FW_MAXH);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 6);
     volatile int *stop = reinterpret_cast<volatile int *>(tslot + 1);
     const uint32_t WB = smem_addr(bars), MD = WB + 8 * FW_SLOTS; // weights in slot k; product 1, 2 done
@@ -765,6 +774,12 @@ k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, cons
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int c = threadIdx.x; c < H; c += GU_THREADS) {
+        b1s[c] = b1[c];
+        b2s[c] = b2[c];
+        w3s[c] = rbf(w3[c]);
+    }
+#pragma unroll 1
     for (int kb = 0; kb < 3; kb++) gu_tile(ga + kb * GU_A_BYTES, X, KPAD, 1, m0, 128, n, 64 * kb, KIN, -1);
     fence_proxy_async_smem(); // the tile stores are visible to the tensor core's reads
     tc_fence_before();
@@ -793,18 +808,14 @@ k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, cons
         }
         loads2 = true;
         const int q = warp & 3, half = warp >> 2, r = 32 * q + lane, row = m0 + r;
+#pragma unroll 1
         for (int c0 = 16 * half; c0 < hp; c0 += 32) {
             float x[16];
             if (c0 < H) {
                 uint32_t v[16];
                 tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
 #pragma unroll
-                for (int j = 0; j < 16; j++) x[j] = fmaxf(__uint_as_float(v[j]) + __ldg(b1 + c0 + j), 0.f);
-                if (STORE && row < n) {
-                    float4 *o = reinterpret_cast<float4 *>(h1 + (long long)row * H + c0);
-#pragma unroll
-                    for (int k = 0; k < 4; k++) o[k] = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
-                }
+                for (int j = 0; j < 16; j++) x[j] = fmaxf(__uint_as_float(v[j]) + b1s[c0 + j], 0.f);
             } else {
 #pragma unroll
                 for (int j = 0; j < 16; j++) x[j] = 0.f;
@@ -834,26 +845,19 @@ k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, cons
         if (ok) {
             tc_fence_after();
             float s = 0.f;
+#pragma unroll 1
             for (int c0 = 16 * half; c0 < H; c0 += 32) {
                 uint32_t v[16];
-                float x[16];
                 tmem_ld16(d2 + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
 #pragma unroll
                 for (int j = 0; j < 16; j++) {
-                    x[j] = fmaxf(__uint_as_float(v[j]) + __ldg(b2 + c0 + j), 0.f);
-                    if (!STORE) s = fmaf(rbf(x[j]), rbf(__ldg(w3 + c0 + j)), s);
-                }
-                if (STORE && row < n) {
-                    float4 *o = reinterpret_cast<float4 *>(h2 + (long long)row * H + c0);
-#pragma unroll
-                    for (int k = 0; k < 4; k++) o[k] = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+                    const float x = fmaxf(__uint_as_float(v[j]) + b2s[c0 + j], 0.f);
+                    s = fmaf(rbf(x), w3s[c0 + j], s);
                 }
             }
-            if (!STORE) { // the training pass takes y from its own head (k_head_train)
-                if (half == 1) ys[r] = s;
-                __syncthreads();
-                if (half == 0 && row < n) y[row] = s + ys[r] + b3[0];
-            }
+            if (half == 1) ys[r] = s;
+            __syncthreads();
+            if (half == 0 && row < n) y[row] = s + ys[r] + b3[0];
         }
     }
     if (!ok && threadIdx.x == 0) {
@@ -875,6 +879,417 @@ k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, cons
     }
 }
 
+// ------------------------------------------------------------------ fused training pass
+// Forward pass, loss and every gradient of 128 rows in one block (hidden <=
+// FW_MAXH), the sums over the batch left as one partial per block, added in block
+// order by k_train_sums:
+//   products (tcgen05, BF16 operands, FP32 in tensor memory):
+//     1  h1 pre = X W1^T            columns [0, H)
+//     2  h2 pre = h1 W2^T           columns [T, T + H), T = half of the tensor memory taken
+//     3  dW2^T  = h1^T dh2          both accumulators: rows h_in 0 .. 127 and 128 .. 255
+//     4  dh1 pre = dh2 W2           columns [0, H)
+//     5  [dW1 | db1]^T = [X | 1]^T dh1   rows 0 .. 127 at column T, 128 .. 143 at column 0
+//   3 and 5 sum over the rows, so they read the same operand tiles transposed
+//   (the tiles' 128-byte rows are 64 consecutive columns of one batch row: the
+//   MN-major form of the same swizzle, K groups of 8 rows 1024 bytes apart, the
+//   next 64 columns 16 KB on).  Transposed, the lanes of a warp hold consecutive
+//   weights of one output unit and every store is one 128-byte run (a lane per
+//   output unit: 64 us instead of 53 for the whole pass).
+// Tiles: X | 1 (3 K blocks), h1 and later dh1 (4), dh2 (4), 16 KB each; the weights'
+// K blocks come by bulk copies into a 32 KB slot of their own and into the tiles
+// that are not in use: W1, then W2 around the dh2 tile, W2^T around the h1 tile
+// (its ReLU mask is kept as bits).  Before it took five products and five other
+// launches with every operand through FP32 device memory: 117.6 us for 8,192 rows,
+// H = 256, now 40.  What is left is the latency of one block's chain (five products,
+// five epilogues) on 64 of the 152 SMs.
+constexpr int TR_TILES = 11; // 16 KB tiles: X 0-2, h 3-6, d 7-10
+constexpr int TR_MAX_ROWS = 1 << 15; // partials of 400 KB per 128 rows at H = 256
+
+int tr_smem(int H)
+{
+    return 1024 + TR_TILES * GU_A_BYTES + H * 128 + 4 * (2 * 128 + 8 * 2 * 128 + 8 + 3 * FW_MAXH) + 2 * 8 * GU_THREADS + 128;
+}
+// a block's partial: dW2 [H][H], [dW1 | db1] [H][144], db2 [H], dw3 [H], db3, loss (padded to 16 floats)
+__host__ __device__ constexpr long long tr_part(int H) { return (long long)H * H + 144LL * H + 2 * H + 16; }
+
+// descriptor of a tile read transposed: 64-column blocks GU_A_BYTES apart, groups of 8 rows 1024 bytes apart
+__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t saddr)
+{
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(GU_A_BYTES >> 4) << 16; // leading byte offset
+    d |= (uint64_t)(1024 >> 4) << 32;       // stride byte offset
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+// 16 columns' sums over the warp's 32 lanes: lane l returns the sum of column l / 2 mod 16
+__device__ __forceinline__ float warp_colsum16(float (&x)[16], int lane)
+{
+#pragma unroll
+    for (int o = 16, half = 8; o > 1; o >>= 1, half >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < half; j++) {
+            const float keep = up ? x[j + half] : x[j], send = up ? x[j] : x[j + half];
+            x[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+
+__global__ void __launch_bounds__(GU_THREADS, 1)
+k_mlp_train(const float *__restrict__ X, const float *__restrict__ t, int n, int H, int hp, int tcols,
+            const uint8_t *__restrict__ W1p, const uint8_t *__restrict__ W2p, const uint8_t *__restrict__ W2T,
+            const float *__restrict__ b1, const float *__restrict__ b2, const float *__restrict__ w3,
+            const float *__restrict__ b3, float *y, float *part, int *err)
+{
+    extern __shared__ uint8_t gu_raw[];
+    const uint32_t raw = smem_addr(gu_raw), base = (raw + 1023u) & ~1023u;
+    uint8_t *ga = gu_raw + (base - raw);
+    uint8_t *hT = ga + 3 * GU_A_BYTES, *dT = ga + 7 * GU_A_BYTES;
+    const uint32_t xa = base, ha = base + 3 * GU_A_BYTES, da = base + 7 * GU_A_BYTES, s0 = base + TR_TILES * GU_A_BYTES;
+    const uint32_t sbytes = (uint32_t)H * 128;
+    float *ys = reinterpret_cast<float *>(ga + TR_TILES * GU_A_BYTES + sbytes); // y halves [2][128]
+    float *cs = ys + 2 * 128;                                                   // column sums [warp][dw3, db2][128]
+    float *rs = cs + 8 * 2 * 128;                                               // row sums [4][db3, loss]
+    float *b1s = rs + 8, *b2s = b1s + FW_MAXH, *w3s = b2s + FW_MAXH;            // biases, w3 rounded to BF16
+    // h1 > 0 at the thread's columns 16 half + 32 i + j: bit j of ms[256 i + thread]
+    uint16_t *ms = reinterpret_cast<uint16_t *>(w3s + FW_MAXH);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(ms + 8 * GU_THREADS);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 8);
+    volatile int *stop = reinterpret_cast<volatile int *>(tslot + 1);
+    // weights landed in slot 0, 1, 2 (their phase counts the loads); a product's MMAs done; slot 0 read
+    const uint32_t WB = smem_addr(bars), MD = WB + 24, SF = WB + 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m0 = blockIdx.x * 128, kb2 = hp / 64;
+    const int q = warp & 3, half = warp >> 2, r = 32 * q + lane, row = m0 + r;
+    const bool in = row < n;
+    float *P = part + (long long)blockIdx.x * tr_part(H);
+    const uint32_t slot1[3] = {s0, da, da + sbytes}, slot2[3] = {s0, ha, ha + sbytes}; // two blocks fit a 64 KB tile group
+    uint32_t loads[3] = {0, 0, 0}; // thread 0: loads issued per slot
+    bool copies = false;
+    auto load = [&](int sl, uint32_t dst, const uint8_t *src) {
+        mbar_expect_tx(WB + 8 * sl, sbytes);
+        bulk_g2s(dst, src, sbytes, WB + 8 * sl);
+        loads[sl]++;
+        copies = true;
+    };
+    auto landed = [&](int sl) { return umma_wait(WB + 8 * sl, (loads[sl] - 1) & 1, stop, err, GU_ERR); };
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < 3; k++) mbar_init(WB + 8 * k, 1);
+        mbar_init(MD, 1);
+        mbar_init(SF, 1);
+        *stop = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int k = 0; k < 3; k++) load(k, slot1[k], W1p + (size_t)k * sbytes);
+    }
+    if (warp == 0) {
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)), "r"(tcols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int c = threadIdx.x; c < H; c += GU_THREADS) {
+        b1s[c] = b1[c];
+        b2s[c] = b2[c];
+        w3s[c] = rbf(w3[c]);
+    }
+#pragma unroll 1
+    for (int kb = 0; kb < 3; kb++) gu_tile(ga + kb * GU_A_BYTES, X, KPAD, 1, m0, 128, n, 64 * kb, KIN, -1);
+    __syncthreads();
+    // column 132 of the tile: 1 (W1's column 132 is zero there), for db1
+    if (threadIdx.x < 128 && m0 + (int)threadIdx.x < n) {
+        const int rr = threadIdx.x, k = KIN - 128; // value 4 of chunk 0 of the third block
+        *reinterpret_cast<__nv_bfloat16 *>(ga + 2 * GU_A_BYTES + rr * 128 + (((k >> 3) ^ (rr & 7)) << 4) + 2 * (k & 7)) =
+            __float2bfloat16_rn(1.f);
+    }
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot, T = (uint32_t)(tcols / 2), lanes = (uint32_t)(32 * q) << 16;
+    const uint32_t idesc = umma_idesc_bf16(H), mn = (1u << 15) | (1u << 16); // both operands MN-major
+    uint32_t md = 0; // products waited for
+    bool ok = true, issued = false;
+    // waits (all threads) for the product thread 0 just committed
+    auto product_done = [&]() {
+        issued = true;
+        ok = __syncthreads_and(umma_wait(MD, md & 1, stop, err, GU_ERR) && ok);
+        md++;
+        tc_fence_after();
+        return ok;
+    };
+    // the threads' tile stores and tensor-memory reads precede the next product
+    auto publish = [&]() {
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    };
+    // thread 0: D[128 rows][H] = A tiles (K-major) x weight blocks; block 3 follows block 0 in slot 0
+    uint32_t sf = 0; // times slot 0 was handed on
+    auto weight_product = [&](uint32_t d, uint32_t a, const uint32_t *slots, const uint8_t *src, int nkb, int K) {
+        for (int kb = 0; kb < nkb && ok; kb++) {
+            const int sl = kb % 3;
+            if (kb == 3) {
+                ok = umma_wait(SF, sf & 1, stop, err, GU_ERR);
+                sf++;
+                if (ok) load(0, slots[0], src + (size_t)3 * sbytes);
+            }
+            ok = ok && landed(sl);
+            if (!ok) break;
+            const int steps = min(4, (K - 64 * kb + 15) / 16);
+            for (int k = 0; k < steps; k++)
+                umma_bf16(d, umma_desc_sw128(a + kb * GU_A_BYTES + 32 * k), umma_desc_sw128(slots[sl] + 32 * k), idesc, kb + k > 0);
+            if (kb == 0 && nkb > 3) umma_commit(SF);
+        }
+    };
+    // the epilogue loops stay rolled: each runs once per block, and unrolled code waited on
+    // instruction fetches (3.6 of the stall cycles per issued instruction)
+    do {
+        // ---- 1: h1
+        if (threadIdx.x == 0) {
+            weight_product(tmem, xa, slot1, W1p, 3, 144);
+            umma_commit(MD);
+        }
+        if (!product_done()) break;
+        if (threadIdx.x == 0)
+            for (int k = 0; k < min(3, kb2); k++) load(k, slot1[k], W2p + (size_t)k * sbytes);
+#pragma unroll 1
+        for (int i = 0; i < 8; i++) {
+            const int c0 = 16 * half + 32 * i;
+            if (c0 < hp) {
+                float x[16];
+                if (c0 < H) {
+                    uint32_t v[16], mask = 0;
+                    tmem_ld16(tmem + lanes + (uint32_t)c0, v);
+#pragma unroll
+                    for (int j = 0; j < 16; j++) {
+                        x[j] = fmaxf(__uint_as_float(v[j]) + b1s[c0 + j], 0.f);
+                        if (x[j] > 0.f) mask |= 1u << j;
+                    }
+                    ms[GU_THREADS * i + threadIdx.x] = (uint16_t)mask;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; j++) x[j] = 0.f;
+                }
+                uint8_t *h = hT + (c0 >> 6) * GU_A_BYTES;
+                const int j0 = (c0 & 63) >> 3;
+                st_chunk(h, r, j0, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+                st_chunk(h, r, j0 + 1, x[8], x[9], x[10], x[11], x[12], x[13], x[14], x[15]);
+            }
+        }
+        publish();
+        // ---- 2: h2, y, dh2
+        if (threadIdx.x == 0) {
+            weight_product(tmem + T, ha, slot1, W2p, kb2, H);
+            umma_commit(MD);
+        }
+        if (!product_done()) break;
+        if (threadIdx.x == 0) load(0, s0, W2T);
+        float s = 0.f;
+#pragma unroll 1
+        for (int c0 = 16 * half; c0 < H; c0 += 32) {
+            uint32_t v[16];
+            tmem_ld16(tmem + T + lanes + (uint32_t)c0, v);
+#pragma unroll
+            for (int j = 0; j < 16; j++) s = fmaf(rbf(fmaxf(__uint_as_float(v[j]) + b2s[c0 + j], 0.f)), w3s[c0 + j], s);
+        }
+        ys[half * 128 + r] = s;
+        __syncthreads();
+        const float yr = ys[r] + ys[128 + r] + b3[0];
+        const float dy = in ? yr - t[row] : 0.f, gy = 2.f * dy / (float)n;
+        if (half == 0 && in) y[row] = yr;
+        if (half == 0) {
+            float a = gy, b = dy * dy;
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                b += __shfl_xor_sync(0xffffffffu, b, o);
+            }
+            if (lane == 0) {
+                rs[2 * q] = a;
+                rs[2 * q + 1] = b;
+            }
+        }
+#pragma unroll 1
+        for (int i = 0; i < 8; i++) {
+            const int c0 = 16 * half + 32 * i;
+            if (c0 >= hp) continue;
+            float dw[16], db[16];
+            if (c0 < H) {
+                uint32_t v[16];
+                tmem_ld16(tmem + T + lanes + (uint32_t)c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const float x = fmaxf(__uint_as_float(v[j]) + b2s[c0 + j], 0.f);
+                    dw[j] = gy * rbf(x);
+                    db[j] = x > 0.f ? rbf(gy * w3s[c0 + j]) : 0.f;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; j++) dw[j] = db[j] = 0.f;
+            }
+            uint8_t *h = dT + (c0 >> 6) * GU_A_BYTES;
+            const int j0 = (c0 & 63) >> 3;
+            st_chunk(h, r, j0, db[0], db[1], db[2], db[3], db[4], db[5], db[6], db[7]);
+            st_chunk(h, r, j0 + 1, db[8], db[9], db[10], db[11], db[12], db[13], db[14], db[15]);
+            const float sw = warp_colsum16(dw, lane), sb = warp_colsum16(db, lane);
+            if ((lane & 1) == 0) { // the warp's columns 16 i .. 16 i + 15 of its half
+                cs[(2 * warp) * 128 + 16 * i + (lane >> 1)] = sw;
+                cs[(2 * warp + 1) * 128 + 16 * i + (lane >> 1)] = sb;
+            }
+        }
+        publish();
+        // ---- 3: dW2
+        const int halves = H > 128 ? 2 : 1;
+        if (threadIdx.x == 0) {
+            for (int m = 0; m < halves; m++)
+                for (int k = 0; k < 8; k++)
+                    umma_bf16(tmem + (m ? T : 0), umma_desc_mn(ha + 2 * m * GU_A_BYTES + 2048 * k), umma_desc_mn(da + 2048 * k),
+                              idesc | mn, k > 0);
+            umma_commit(MD);
+        }
+        {   // meanwhile the column and row sums of the four row quarters
+            float *pc = P + (long long)H * H + 144LL * H;
+            for (int c = threadIdx.x; c < H; c += GU_THREADS) {
+                const int hf = (c >> 4) & 1, at = 16 * (c >> 5) + (c & 15);
+                float w = 0.f, b = 0.f;
+                for (int k = 0; k < 4; k++) {
+                    w += cs[2 * (4 * hf + k) * 128 + at];
+                    b += cs[(2 * (4 * hf + k) + 1) * 128 + at];
+                }
+                pc[c] = b;
+                pc[H + c] = w;
+            }
+            if (threadIdx.x == 0) {
+                pc[2 * H] = rs[0] + rs[2] + rs[4] + rs[6];
+                pc[2 * H + 1] = rs[1] + rs[3] + rs[5] + rs[7];
+            }
+        }
+        if (!product_done()) break;
+        if (threadIdx.x == 0)
+            for (int k = 1; k < min(3, kb2); k++) load(k, slot2[k], W2T + (size_t)k * sbytes);
+        for (int m = 0; m < halves; m++) {
+            const int hi = 128 * m + r;
+#pragma unroll 1
+            for (int c0 = 16 * half; c0 < H; c0 += 32) {
+                uint32_t v[16];
+                tmem_ld16(tmem + (m ? T : 0) + lanes + (uint32_t)c0, v);
+                if (hi < H) {
+#pragma unroll
+                    for (int k = 0; k < 16; k++) P[(c0 + k) * H + hi] = __uint_as_float(v[k]);
+                }
+            }
+        }
+        publish();
+        // ---- 4: dh1
+        if (threadIdx.x == 0) {
+            weight_product(tmem, da, slot2, W2T, kb2, H);
+            umma_commit(MD);
+        }
+        if (!product_done()) break;
+#pragma unroll 1
+        for (int i = 0; i < 8; i++) {
+            const int c0 = 16 * half + 32 * i;
+            if (c0 >= hp) continue;
+            float x[16];
+            if (c0 < H) {
+                uint32_t v[16];
+                const uint32_t mask = ms[GU_THREADS * i + threadIdx.x];
+                tmem_ld16(tmem + lanes + (uint32_t)c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; j++) x[j] = (mask >> j) & 1 ? __uint_as_float(v[j]) : 0.f;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; j++) x[j] = 0.f;
+            }
+            uint8_t *h = hT + (c0 >> 6) * GU_A_BYTES;
+            const int j0 = (c0 & 63) >> 3;
+            st_chunk(h, r, j0, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+            st_chunk(h, r, j0 + 1, x[8], x[9], x[10], x[11], x[12], x[13], x[14], x[15]);
+        }
+        publish();
+        // ---- 5: [dW1 | db1]
+        if (threadIdx.x == 0) {
+            for (int m = 0; m < 2; m++) // rows 144 .. 255 are whatever lies beyond the X tiles: not stored
+                for (int k = 0; k < 8; k++)
+                    umma_bf16(tmem + (m ? 0 : T), umma_desc_mn(xa + 2 * m * GU_A_BYTES + 2048 * k), umma_desc_mn(ha + 2048 * k),
+                              idesc | mn, k > 0);
+            umma_commit(MD);
+        }
+        if (!product_done()) break;
+        for (int m = 0; m < (q == 0 ? 2 : 1); m++) {
+            const int k0 = 128 * m + r;
+#pragma unroll 1
+            for (int c0 = 16 * half; c0 < H; c0 += 32) {
+                uint32_t v[16];
+                tmem_ld16(tmem + (m ? 0 : T) + lanes + (uint32_t)c0, v);
+                if (k0 < 144) {
+                    float *o = P + H * H + k0;
+#pragma unroll
+                    for (int k = 0; k < 16; k++) o[(c0 + k) * 144] = __uint_as_float(v[k]);
+                }
+            }
+        }
+    } while (false);
+    if (!ok && threadIdx.x == 0) {
+        // a wait expired: copies and MMAs in flight finish (bounded) before the memory goes
+        auto drain = [&](uint32_t bar, uint32_t par) {
+            const uint64_t t0 = global_ns();
+            while (!mbar_test(bar, par) && global_ns() - t0 < UMMA_WAIT_NS) {
+            }
+        };
+        if (copies)
+            for (int k = 0; k < 3; k++)
+                if (loads[k]) drain(WB + 8 * k, (loads[k] - 1) & 1);
+        if (issued) drain(MD, (md - 1) & 1);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
+    }
+}
+
+// grads (parameter layout) and the loss from the blocks' partials: a warp takes every
+// fourth block's 32 consecutive values in order, the four warps' sums are added in order
+constexpr int TS_SLICES = 4;
+
+__global__ void __launch_bounds__(32 * TS_SLICES)
+k_train_sums(const float *__restrict__ part, int nb, int H, long long stride, Offsets o, int n, float *g, float *loss)
+{
+    __shared__ float red[TS_SLICES][32];
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const long long w1 = (long long)H * H, v = w1 + 144LL * H, total = v + 2 * H + 2;
+    const long long e = (long long)blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (e < total) {
+#pragma unroll 8
+        for (int b = slice; b < nb; b += TS_SLICES) s += part[b * stride + e];
+    }
+    red[slice][lane] = s;
+    __syncthreads();
+    if (slice || e >= total) return;
+#pragma unroll
+    for (int k = 1; k < TS_SLICES; k++) s += red[k][lane];
+    if (e < w1) {
+        g[o.W2 + e] = s;
+    } else if (e < v) {
+        const int r = (int)((e - w1) / 144), c = (int)((e - w1) % 144);
+        if (c < KIN) g[o.W1 + (long long)r * KIN + c] = s;
+        else if (c == KIN) g[o.b1 + r] = s;
+    } else if (e < v + H) {
+        g[o.b2 + (e - v)] = s;
+    } else if (e < v + 2 * H) {
+        g[o.w3 + (e - v - H)] = s;
+    } else if (e == v + 2 * H) {
+        g[o.b3] = s;
+    } else if (loss) {
+        *loss = s / (float)n;
+    }
+}
+
 } // namespace
 
 // ------------------------------------------------------------------ network object
@@ -885,7 +1300,7 @@ struct bc_mlp_s {
     float *p = nullptr, *m = nullptr, *v = nullptr, *g = nullptr; // params, Adam moments, gradients
     long long step = 0;
     // activations for the current batch capacity
-    int cap = 0;
+    int cap = 0, ycap = 0;
     float *h1 = nullptr, *h2 = nullptr, *y = nullptr, *gy = nullptr, *dh2 = nullptr, *dh1 = nullptr;
     float *part = nullptr;        // split-K and column-sum partials
     long long part_floats = 0;
@@ -893,7 +1308,7 @@ struct bc_mlp_s {
     int xb_cap = 0;
     float *loss = nullptr;
     uint8_t *wp = nullptr;        // BF16 weights in the fused forward pass's layout (hidden <= FW_MAXH)
-    bool packed = false;          // they hold the current parameters
+    int packed = 0;               // which hold the current parameters: 1 W1 and W2, 2 W2 transposed too
     int rotated_moments = 0;      // the ligand features are the moments of the rotated ligand (bc_mlp_set_features)
 };
 
@@ -917,48 +1332,85 @@ bc_status mcuda(cudaError_t e, const char *where)
         if (e_ != cudaSuccess) return mcuda(e_, #call);                                                  \
     } while (0)
 
+template <typename T>
+cudaError_t regrow(T *&p, size_t count)
+{
+    if (p) cudaFree(p);
+    p = nullptr;
+    return cudaMalloc(&p, sizeof(T) * count);
+}
+
+// Buffers of a training pass of n rows: the fused one keeps its layers on chip and
+// needs y and the partials only.
 bc_status ensure_batch(bc_mlp_t net, int n)
 {
-    if (n <= net->cap) return BC_OK;
-    float *bufs[] = {net->h1, net->h2, net->y, net->gy, net->dh2, net->dh1};
-    for (float *b : bufs)
-        if (b) cudaFree(b);
-    const int cap = n + n / 4 + 64;
-    const size_t H = net->H;
-    MCK(cudaMalloc(&net->h1, sizeof(float) * cap * H));
-    MCK(cudaMalloc(&net->h2, sizeof(float) * cap * H));
-    MCK(cudaMalloc(&net->dh2, sizeof(float) * cap * H));
-    MCK(cudaMalloc(&net->dh1, sizeof(float) * cap * H));
-    MCK(cudaMalloc(&net->y, sizeof(float) * cap));
-    MCK(cudaMalloc(&net->gy, sizeof(float) * cap));
-    if (net->part) cudaFree(net->part);
-    // up to 32 split-K slices of the largest weight gradient (H x (H + 1) or H x 133,
-    // the last column the bias gradient), and the training head's block sums
-    net->part_floats = std::max(32LL * (long long)H * (std::max<long long>((long long)H, KIN) + 1),
-                                (long long)HT_MAX_BLOCKS * (2LL * (long long)H + 1));
-    MCK(cudaMalloc(&net->part, sizeof(float) * net->part_floats));
-    net->cap = cap;
+    const size_t H = net->H, cap = (size_t)n + n / 4 + 64;
+    const bool fused = net->wp && n <= TR_MAX_ROWS;
+    if (n > net->ycap) {
+        net->ycap = 0;
+        MCK(regrow(net->y, cap));
+        net->ycap = (int)cap;
+    }
+    // the fused pass's partials; or up to 32 split-K slices of the largest weight
+    // gradient (H x (H + 1) or H x 133, the last column the bias gradient), and the
+    // training head's block sums
+    const long long need = fused ? (long long)((n + 127) / 128) * tr_part((int)H)
+                                 : std::max(32LL * (long long)H * (std::max<long long>((long long)H, KIN) + 1),
+                                            (long long)HT_MAX_BLOCKS * (2LL * (long long)H + 1));
+    if (need > net->part_floats) {
+        net->part_floats = 0;
+        MCK(regrow(net->part, (size_t)need));
+        net->part_floats = need;
+    }
+    if (fused || n <= net->cap) return BC_OK;
+    net->cap = 0;
+    for (float **b : {&net->h1, &net->h2, &net->dh2, &net->dh1}) MCK(regrow(*b, cap * H));
+    MCK(regrow(net->gy, cap));
+    net->cap = (int)cap;
     return BC_OK;
 }
 
-// The fused forward pass: the layers into net->h1, net->h2 (store), else y.  It needs
-// X on a 16-byte boundary only for speed; H a multiple of 16 up to FW_MAXH.
-bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, bool store, cudaStream_t s)
+// The BF16 weight blocks of the fused passes, once per parameter change.
+bc_status pack_weights(bc_mlp_t net, int want, cudaStream_t s)
 {
+    if (net->packed >= want) return BC_OK;
+    const int H = net->H, hp = fw_hp(H);
+    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128, *W2T = W2p + (size_t)hp / 64 * H * 128;
+    const int items = (3 + (want > 1 ? 2 : 1) * hp / 64) * H * 8;
+    k_pack_weights<<<(items + 255) / 256, 256, 0, s>>>(net->p + net->off.W1, net->p + net->off.W2, H, hp, W1p, W2p,
+                                                       want > 1 ? W2T : nullptr);
+    MCK(cudaGetLastError());
+    net->packed = want;
+    return BC_OK;
+}
+
+// The fused forward pass: y of n rows.
+bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, cudaStream_t s)
+{
+    if (bc_status st = pack_weights(net, 1, s)) return st;
     const int H = net->H, hp = fw_hp(H);
     const Offsets &o = net->off;
     uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128;
-    if (!net->packed) {
-        k_pack_weights<<<(3 * H * 8 + hp / 64 * H * 8 + 255) / 256, 256, 0, s>>>(net->p + o.W1, net->p + o.W2, H, hp, W1p, W2p);
-        MCK(cudaGetLastError());
-        net->packed = true;
-    }
     int tcols = 32; // two accumulators of H columns
     while (tcols < 2 * H) tcols <<= 1;
-    const int smem = fw_smem(H);
-    auto kernel = store ? k_mlp_forward<true> : k_mlp_forward<false>;
-    kernel<<<(n + 127) / 128, GU_THREADS, smem, s>>>(X, n, H, hp, tcols, W1p, W2p, net->p + o.b1, net->p + o.b2, net->p + o.w3,
-                                                     net->p + o.b3, net->h1, net->h2, y, ctx_err(net->ctx));
+    k_mlp_forward<<<(n + 127) / 128, GU_THREADS, fw_smem(H), s>>>(X, n, H, hp, tcols, W1p, W2p, net->p + o.b1, net->p + o.b2,
+                                                                  net->p + o.w3, net->p + o.b3, y, ctx_err(net->ctx));
+    MCK(cudaGetLastError());
+    return BC_OK;
+}
+
+// The fused training pass: y, the gradients into g and the loss (may be null).
+bc_status fused_train(bc_mlp_t net, const float *X, const float *t, int n, float *g, float *loss, cudaStream_t s)
+{
+    if (bc_status st = pack_weights(net, 2, s)) return st;
+    const int H = net->H, hp = fw_hp(H), blocks = (n + 127) / 128;
+    const Offsets &o = net->off;
+    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128, *W2T = W2p + (size_t)hp / 64 * H * 128;
+    k_mlp_train<<<blocks, GU_THREADS, tr_smem(H), s>>>(X, t, n, H, hp, 512, W1p, W2p, W2T, net->p + o.b1, net->p + o.b2,
+                                                       net->p + o.w3, net->p + o.b3, net->y, net->part, ctx_err(net->ctx));
+    MCK(cudaGetLastError());
+    const long long total = (long long)H * H + 144LL * H + 2 * H + 2;
+    k_train_sums<<<(unsigned)((total + 31) / 32), 32 * TS_SLICES, 0, s>>>(net->part, blocks, H, tr_part(H), o, n, g, loss);
     MCK(cudaGetLastError());
     return BC_OK;
 }
@@ -966,7 +1418,6 @@ bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, bool stor
 // the hidden layers into net->h1, net->h2
 bc_status hidden_layers(bc_mlp_t net, const float *X, int n, cudaStream_t s)
 {
-    if (net->wp) return fused_forward(net, X, n, nullptr, true, s);
     const int H = net->H;
     const Offsets &o = net->off;
     GemmArgs a1{X, KPAD, 1, net->p + o.W1, 1, KIN, net->h1, H, 1, n, H, KPAD, net->p + o.b1, 1};
@@ -984,7 +1435,7 @@ bc_status hidden_layers(bc_mlp_t net, const float *X, int n, cudaStream_t s)
 // forward pass into net->h1, net->h2, y
 bc_status forward(bc_mlp_t net, const float *X, int n, float *y, cudaStream_t s)
 {
-    if (net->wp) return fused_forward(net, X, n, y, false, s);
+    if (net->wp) return fused_forward(net, X, n, y, s);
     if (bc_status st = hidden_layers(net, X, n, s)) return st;
     const Offsets &o = net->off;
     k_head<<<(n + 7) / 8, 256, 0, s>>>(net->h2, net->p + o.w3, net->p + o.b3, n, net->H, y);
@@ -992,9 +1443,11 @@ bc_status forward(bc_mlp_t net, const float *X, int n, float *y, cudaStream_t s)
     return BC_OK;
 }
 
-// forward pass (net->y) and the gradients of the mean squared error into net->g
-bc_status forward_backward(bc_mlp_t net, const float *X, const float *t, int n, cudaStream_t s)
+// forward pass (net->y), the gradients of the mean squared error into net->g -- or,
+// where given, into `grads` -- and the error itself into loss (may be null)
+bc_status forward_backward(bc_mlp_t net, const float *X, const float *t, int n, float *grads, float *loss, cudaStream_t s)
 {
+    if (net->wp && n <= TR_MAX_ROWS) return fused_train(net, X, t, n, grads ? grads : net->g, loss, s);
     if (bc_status st = hidden_layers(net, X, n, s)) return st;
     const int H = net->H;
     const Offsets &o = net->off;
@@ -1015,6 +1468,11 @@ bc_status forward_backward(bc_mlp_t net, const float *X, const float *t, int n, 
     w1.err = ctx_err(net->ctx);
     w1.bone = KIN;
     MCK(gemm_splitk(w1, net->part, net->part_floats, s, net->g + o.b1));
+    if (loss) {
+        k_loss<<<1, 256, 0, s>>>(net->y, t, n, loss);
+        MCK(cudaGetLastError());
+    }
+    if (grads) MCK(cudaMemcpyAsync(grads, net->g, sizeof(float) * (size_t)net->off.total, cudaMemcpyDeviceToDevice, s));
     return BC_OK;
 }
 
@@ -1262,16 +1720,15 @@ cudaError_t bc::launch_axpby(float *y, const float *x, int n, float alpha, float
 
 void bc::mlp_orphan(bc_mlp_s *net)
 {
-    float *bufs[] = {net->p,  net->m,   net->v,    net->g,  net->h1, net->h2,  net->y,
-                     net->gy, net->dh2, net->dh1, net->loss, net->part, net->xb, net->tb};
+    // p heads the allocation that also holds m, v, g, loss and wp
+    float *bufs[] = {net->p, net->h1, net->h2, net->y, net->gy, net->dh2, net->dh1, net->part, net->xb, net->tb};
     for (float *b : bufs)
         if (b) cudaFree(b);
     net->p = net->m = net->v = net->g = net->h1 = net->h2 = net->y = net->gy = net->dh2 = net->dh1 = net->loss = nullptr;
     net->part = net->xb = net->tb = nullptr;
-    if (net->wp) cudaFree(net->wp);
     net->wp = nullptr;
-    net->packed = false;
-    net->cap = net->xb_cap = 0;
+    net->packed = 0;
+    net->cap = net->ycap = net->xb_cap = 0;
     net->part_floats = 0;
     net->ctx = nullptr;
 }
@@ -1292,18 +1749,23 @@ bc_status bc_mlp_create(bc_ctx_t ctx, int hidden, const float *init, bc_mlp_t *o
         const size_t bytes = sizeof(float) * (size_t)net->off.total;
         cudaStream_t s = ctx_stream(ctx);
         cudaError_t e;
-        if ((e = cudaMalloc(&net->p, bytes)) != cudaSuccess || (e = cudaMalloc(&net->m, bytes)) != cudaSuccess ||
-            (e = cudaMalloc(&net->v, bytes)) != cudaSuccess || (e = cudaMalloc(&net->g, bytes)) != cudaSuccess ||
-            (e = cudaMalloc(&net->loss, sizeof(float))) != cudaSuccess) {
+        // one allocation: parameters, Adam moments, gradients, the loss word, BF16 weight blocks
+        const size_t row = (size_t)((net->off.total + 63) & ~63LL), fused = hidden <= FW_MAXH;
+        const size_t wbytes = fused ? (size_t)(3 + 2 * (fw_hp(hidden) / 64)) * hidden * 128 : 0;
+        if ((e = cudaMalloc(&net->p, sizeof(float) * (4 * row + 64) + wbytes)) != cudaSuccess) {
             bc_mlp_destroy(net);
             return mcuda(e, "bc_mlp_create: cudaMalloc");
         }
-        if (hidden <= FW_MAXH) {
-            if ((e = cudaMalloc(&net->wp, (size_t)(3 + fw_hp(hidden) / 64) * hidden * 128)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(k_mlp_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(k_mlp_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess) {
+        net->m = net->p + row;
+        net->v = net->m + row;
+        net->g = net->v + row;
+        net->loss = net->g + row;
+        if (fused) {
+            net->wp = reinterpret_cast<uint8_t *>(net->loss + 64);
+            if ((e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess ||
+                (e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, tr_smem(FW_MAXH))) != cudaSuccess) {
                 bc_mlp_destroy(net);
-                return mcuda(e, "bc_mlp_create: fused forward pass");
+                return mcuda(e, "bc_mlp_create: fused passes");
             }
         }
         if ((e = cudaMemcpyAsync(net->p, init, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
@@ -1371,7 +1833,8 @@ bc_status bc_mlp_predict(bc_mlp_t net, const float *X, int n, float *y)
     try {
         if (!net || !X || !y || n < 1) return mfail(BC_ERR_ARG, "bc_mlp_predict: bad arguments");
         if (!net->ctx) return mfail(BC_ERR_ARG, "bc_mlp_predict: the network's context was destroyed");
-        if (bc_status st = ensure_batch(net, n)) return st;
+        if (!net->wp) // the fused pass needs no buffers
+            if (bc_status st = ensure_batch(net, n)) return st;
         return forward(net, X, n, y, ctx_stream(net->ctx));
     } catch (...) {
         return mfail(BC_ERR_INTERNAL, "bc_mlp_predict: unexpected exception");
@@ -1385,12 +1848,7 @@ bc_status bc_mlp_grads(bc_mlp_t net, const float *X, const float *t, int n, floa
         if (!net->ctx) return mfail(BC_ERR_ARG, "bc_mlp_grads: the network's context was destroyed");
         if (bc_status st = ensure_batch(net, n)) return st;
         cudaStream_t s = ctx_stream(net->ctx);
-        if (bc_status st = forward_backward(net, X, t, n, s)) return st;
-        if (loss) {
-            k_loss<<<1, 256, 0, s>>>(net->y, t, n, loss);
-            MCK(cudaGetLastError());
-        }
-        if (grads) MCK(cudaMemcpyAsync(grads, net->g, sizeof(float) * (size_t)net->off.total, cudaMemcpyDeviceToDevice, s));
+        if (bc_status st = forward_backward(net, X, t, n, grads, loss, s)) return st;
         return BC_OK;
     } catch (...) {
         return mfail(BC_ERR_INTERNAL, "bc_mlp_grads: unexpected exception");
@@ -1410,7 +1868,7 @@ bc_status bc_mlp_train_step(bc_mlp_t net, const float *X, const float *t, int n,
         k_adam<<<(unsigned)((total + 255) / 256), 256, 0, ctx_stream(net->ctx)>>>(net->p, net->m, net->v, net->g, total, lr,
                                                                                  b1, b2, eps, c1, c2);
         MCK(cudaGetLastError());
-        net->packed = false;
+        net->packed = 0;
         return BC_OK;
     } catch (...) {
         return mfail(BC_ERR_INTERNAL, "bc_mlp_train_step: unexpected exception");
@@ -1480,14 +1938,14 @@ bc_status bc_mlp_train(bc_mlp_t net, const float *X, const float *t, int n, int 
                                                                                  net->xb, net->tb);
                 }
                 MCK(cudaGetLastError());
-                if (bc_status r = forward_backward(net, net->xb, net->tb, batch, s)) return r;
+                if (bc_status r = forward_backward(net, net->xb, net->tb, batch, nullptr, nullptr, s)) return r;
                 net->step++;
                 const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
                 const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
                 k_adam<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(net->p, net->m, net->v, net->g, total, lr_e, b1,
                                                                       b2, eps, c1, c2);
                 MCK(cudaGetLastError());
-                net->packed = false;
+                net->packed = 0;
             }
         }
         if (loss) {
@@ -1512,7 +1970,7 @@ bc_status bc_mlp_state(bc_mlp_t net, float *params, float *m, float *v, long lon
         if (!host[i]) continue;
         if (get) MCK(cudaMemcpyAsync(host[i], dev[i], bytes, cudaMemcpyDeviceToHost, s));
         else MCK(cudaMemcpyAsync(dev[i], host[i], bytes, cudaMemcpyHostToDevice, s));
-        if (!get && i == 0) net->packed = false;
+        if (!get && i == 0) net->packed = 0;
     }
     MCK(cudaStreamSynchronize(s));
     if (step) {
