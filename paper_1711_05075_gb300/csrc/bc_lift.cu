@@ -613,7 +613,7 @@ bc_status bc_lift_create(const bc_lift_params *p, void *cuda_stream, bc_lift_t *
         const int N = lf->N, Nr = lf->Nr, W = 8;
         const double a = W / 2.0 * 1.5;
         const double beta = (double)(float)(M_PI * std::sqrt(a * a - 0.8));
-        const size_t fl = (size_t)N + Nr + CONSTS_FLOATS + 2 * (size_t)N + 2 * (size_t)Nr + 8;
+        const size_t fl = (size_t)N + Nr + CONSTS_FLOATS + 2 * (size_t)N + 2 * (size_t)Nr + 8 + LIFT4_BOX_BYTES / sizeof(float);
         const size_t bytes = sizeof(float) * fl + sizeof(float2) * (2 * (size_t)N + 2 * (size_t)Nr + N + Nr) + 256;
         if ((e = cudaMalloc(&lf->t4_mem, bytes)) != cudaSuccess) return bail(e, "cudaMalloc NUFFT tables");
         float2 *tw = (float2 *)lf->t4_mem; // n + n_r twiddles, then N + N_r scratch ones
@@ -624,8 +624,9 @@ bc_status bc_lift_create(const bc_lift_params *p, void *cuda_stream, bc_lift_t *
         lf->t4.deconv_s = f;
         lf->t4.deconv_r = f + N;
         lf->t4.consts = f + N + Nr;
-        lf->t4.dbox = (int *)(lf->t4.consts + CONSTS_FLOATS);
-        if ((e = cudaMallocHost(&lf->t4.hbox, 8 * sizeof(int))) != cudaSuccess) return bail(e, "cudaMallocHost box");
+        lf->t4.dbox = (int *)(((uintptr_t)(lf->t4.consts + CONSTS_FLOATS) + 15) & ~(uintptr_t)15);
+        if ((e = cudaMallocHost(&lf->t4.hbox, LIFT4_BOX_BYTES)) != cudaSuccess) return bail(e, "cudaMallocHost box");
+        if ((e = cudaMalloc(&lf->t4.wts, lift4_weight_bytes(N, Nr))) != cudaSuccess) return bail(e, "cudaMalloc mode weights");
         Geometry gs{}, gr{};
         gs.N = N, gs.n = 2 * N, gs.W = W, gs.L = 0;
         gr.N = Nr, gr.n = 2 * Nr, gr.W = W, gr.L = 0;
@@ -634,6 +635,7 @@ bc_status bc_lift_create(const bc_lift_params *p, void *cuda_stream, bc_lift_t *
             (e = launch_build_tables(gr, beta, lf->period_r, nullptr, lf->t4.deconv_r, nullptr, lf->t4.tw_r, twNr,
                                      lf->t4.consts, lf->stream)) != cudaSuccess)
             return bail(e, "bc_lift_create: NUFFT tables");
+        if ((e = lift4_build_weights(lf->t4, N, Nr, lf->cone, lf->stream)) != cudaSuccess) return bail(e, "bc_lift_create: mode weights");
     }
     if ((e = cudaStreamSynchronize(lf->stream)) != cudaSuccess) return bail(e, "bc_lift_create: sync");
     cudaFree(g);
@@ -649,6 +651,7 @@ bc_status bc_lift_destroy(bc_lift_t lf)
     if (lf->cone) cudaFree(lf->cone);
     if (lf->tw) cudaFree(lf->tw);
     if (lf->t4_mem) cudaFree(lf->t4_mem);
+    if (lf->t4.wts) cudaFree(lf->t4.wts);
     if (lf->t4.hbox) cudaFreeHost(lf->t4.hbox);
     if (lf->ws) cudaFree(lf->ws);
     if (lf->pin) cudaFreeHost(lf->pin);
@@ -746,6 +749,7 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
         return lift_cuda(e, "bc_lift_correlate: descriptors");
     if ((e = cudaMemsetAsync(derr, 0, sizeof(int), st)) != cudaSuccess) return lift_cuda(e, "bc_lift_correlate: error word");
     const float scale = (float)(1.0 / (lf->period * lf->period * lf->period * lf->period_r));
+    bool line = false; // h is already inverse transformed along x (lift4_pair)
     if (lf->contraction == 3) {
         // both spectra by the 4D NUFFT, their r transforms fused with the collapse
         const double qw = quat[0] * inv, qx = quat[1] * inv, qy = quat[2] * inv, qz = quat[3] * inv;
@@ -753,7 +757,7 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
                              2 * (qx * qy + qw * qz), 1 - 2 * (qx * qx + qz * qz), 2 * (qy * qz - qw * qx),
                              2 * (qx * qz - qw * qy), 2 * (qy * qz + qw * qx), 1 - 2 * (qx * qx + qy * qy)};
         if ((e = lift4_pair(lf->t4, N, Nr, kA, nA, kB, nB, R, lf->period, lf->period_r, lf->cone, dsl, nslices, scale, E,
-                            h, lf->nsm, st)) != cudaSuccess)
+                            h, &line, derr, lf->nsm, st)) != cudaSuccess)
             return lift_cuda(e, "bc_lift_correlate: 4D NUFFT");
     } else {
     // both spectra are accumulated with atomics: one clear for the pair
@@ -821,6 +825,16 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
     if ((e = launch_lift_collapse(rhoA, rhoB, lf->cone, N, Nr, dsl, nslices, lf->period_r, scale, h, st)) != cudaSuccess)
         return lift_cuda(e, "bc_lift_correlate: collapse");
     }
+    Geometry g{};
+    g.N = N;
+    g.n = 2 * N;
+    g.H = H;
+    Tables t{};
+    t.tw_N = lf->tw;
+    if (line) {
+        if ((e = launch_iyz(g, t, dpairs, nslices, h, dout, nullptr, lf->nsm, st)) != cudaSuccess)
+            return lift_cuda(e, "bc_lift_correlate: inverse y and z");
+    } else {
     switch (N) {
     case 32: k_lift_ifft_x<32><<<lf->nsm, TB, 0, st>>>(h, nslices, lf->tw); break;
     case 64: k_lift_ifft_x<64><<<lf->nsm, TB, 0, st>>>(h, nslices, lf->tw); break;
@@ -828,15 +842,10 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
     default: k_lift_ifft_x<128><<<lf->nsm, TB, 0, st>>>(h, nslices, lf->tw); break;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return lift_cuda(e, "bc_lift_correlate: collapse");
-    Geometry g{};
-    g.N = N;
-    g.n = 2 * N;
-    g.H = H;
-    Tables t{};
-    t.tw_N = lf->tw;
     if ((e = launch_ifft_y(g, t, dpairs, nslices, h, lf->nsm, st)) != cudaSuccess) return lift_cuda(e, "bc_lift_correlate: ifft y");
     if ((e = launch_ifft_z(g, t, dpairs, nslices, h, dout, nullptr, lf->nsm, st)) != cudaSuccess)
         return lift_cuda(e, "bc_lift_correlate: ifft z");
+    }
     if (!on_device) {
         if ((e = cudaMemcpyAsync(out, dout, sizeof(float) * (size_t)N * N * N * nslices, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return lift_cuda(e, "bc_lift_correlate: copy out");

@@ -40,7 +40,10 @@
 // Transforms: the library's shared-memory Stockham FFT (bc_fft.cuh) on tiles of
 // 16 interleaved lines.  The grid and the z planes share the workspace with
 // the y and x planes (each pass's output fits in the space its input left).
+#include <algorithm>
+#include <climits>
 #include <cmath>
+#include <cstring>
 
 #include "bc_device.cuh"
 #include "bc_lift4.h"
@@ -49,54 +52,36 @@ namespace bc {
 
 constexpr int L4_W = 8; // window width of the lifted NUFFT
 
-// Fine-grid coordinate of knot c on axis a (0, 1, 2: rotated x, y, z; 3: r,
-// mirrored for B), half a period on.
-__device__ __forceinline__ double l4_coord(const float4 &c, int a, const double (&R)[9], int mirror, int ns, int nr,
-                                           double inv_p, double inv_pr)
-{
-    double v;
-    if (a < 3) v = (R[3 * a] * c.x + R[3 * a + 1] * c.y + R[3 * a + 2] * c.z) * inv_p + 0.5;
-    else v = (mirror ? -(double)c.w : (double)c.w) * inv_pr + 0.5;
-    return (v - floor(v)) * (a < 3 ? ns : nr);
-}
+using L4Rot = Lift4Rot;
+using L4Box = Lift4Box;
 
-struct L4Rot {
-    double R[9];
-};
-
-// box[a] = min, box[4 + a] = max over the knots of the first stencil cell
-// ceil(u_a - W/2) (box preset to INT_MAX / INT_MIN).
+// box[a] = min, box[4 + a] = min of the negative, over the knots, of the first
+// stencil cell ceil(u_a - W/2) (preset to large values).
 __global__ void k_l4_box(const float4 *__restrict__ knots, int n, L4Rot rot, int mirror, int ns, int nr, double inv_p,
                          double inv_pr, int *box)
 {
-    int lo[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX}, hi[4] = {INT_MIN, INT_MIN, INT_MIN, INT_MIN};
+    int lo[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX}, hi[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 c = knots[i];
 #pragma unroll
         for (int a = 0; a < 4; a++) {
-            const int g0 = (int)ceil(l4_coord(c, a, rot.R, mirror, ns, nr, inv_p, inv_pr) - 0.5 * L4_W);
+            const int g0 = (int)ceil(lift4_coord(c, a, rot.R, mirror, ns, nr, inv_p, inv_pr) - 0.5 * L4_W);
             lo[a] = min(lo[a], g0);
-            hi[a] = max(hi[a], g0);
+            hi[a] = min(hi[a], -g0);
         }
     }
 #pragma unroll
     for (int a = 0; a < 4; a++) {
         for (int off = 16; off > 0; off >>= 1) {
             lo[a] = min(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], off));
-            hi[a] = max(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], off));
+            hi[a] = min(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], off));
         }
         if ((threadIdx.x & 31) == 0 && lo[a] != INT_MAX) {
             atomicMin(box + a, lo[a]);
-            atomicMax(box + 4 + a, hi[a]);
+            atomicMin(box + 4 + a, hi[a]);
         }
     }
 }
-
-// Box of the grid: per axis (x, y, z, r) the first cell lo and the extent b;
-// cell g of the axis is box element (g - lo) mod n.
-struct L4Box {
-    int lo[4], b[4];
-};
 
 // 4W window weights of one knot per warp, then the W^4 stencil into the box
 // grid G[i_r][i_x][i_y][i_z].
@@ -115,7 +100,7 @@ k_l4_spread(const float4 *__restrict__ knots, int n, L4Rot rot, int mirror, int 
     for (int i = blockIdx.x * 8 + wib; i < n; i += gridDim.x * 8) {
         const float4 c = knots[i];
         if (lane < 4 * W) {
-            const double u = l4_coord(c, a, rot.R, mirror, ns, nr, inv_p, inv_pr);
+            const double u = lift4_coord(c, a, rot.R, mirror, ns, nr, inv_p, inv_pr);
             const int g0 = (int)ceil(u - 0.5 * W);
             // offset t's weight is phi(x + W/2 - 1 - t), x = u - g0 - (W/2 - 1) in (0, 1]
             wts[wib][a][t] = kb_poly(kc, (float)(u - g0 - (0.5 * W - 1.0)));
@@ -341,45 +326,19 @@ static cudaError_t l4_mid(const float2 *in, float2 *out, long long nouter, int n
     return cudaGetLastError();
 }
 
-// The x planes X1[j_x][j_y][i_r][m_z] of n knots (box, spreading, z, y and x
-// passes); lo_r and b_r receive the box along r.  Synchronises s once (the
-// support box comes back to the host through the page-locked words hbox).
+// The x planes X1[j_x][j_y][i_r][m_z] of n knots in the box bx (spreading, z, y and x
+// passes), for boxes that take a whole axis.
 static cudaError_t l4_xplanes(const Lift4Tables &t, int N, int Nr, const float4 *knots, int n, const L4Rot &rot,
-                              int mirror, double ip, double ipr, void *ws, float2 *X1, int &lo_r, int &b_r, int nsm,
+                              int mirror, double ip, double ipr, const L4Box &bx, void *ws, float2 *X1, int nsm,
                               cudaStream_t s)
 {
     const int ns = 2 * N, nr = 2 * Nr, H = N / 2;
-    // the support box
     cudaError_t e;
-    if ((e = cudaMemsetAsync(t.dbox, 0x7f, 4 * sizeof(int), s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(t.dbox + 4, 0x80, 4 * sizeof(int), s)) != cudaSuccess)
-        return e;
-    if (n > 0) {
-        const int blocks = (n + 255) / 256 < 4 * nsm ? (n + 255) / 256 : 4 * nsm;
-        k_l4_box<<<blocks, 256, 0, s>>>(knots, n, rot, mirror, ns, nr, ip, ipr, t.dbox);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if ((e = cudaMemcpyAsync(t.hbox, t.dbox, 8 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    L4Box bx;
-    for (int a = 0; a < 4; a++) {
-        const int na = a < 3 ? ns : nr;
-        const long long lo = t.hbox[a], hi = (long long)t.hbox[4 + a] + L4_W - 1;
-        if (n == 0 || hi - lo + 1 >= na) {
-            bx.lo[a] = 0;
-            bx.b[a] = na;
-        } else {
-            bx.lo[a] = (int)lo;
-            bx.b[a] = (int)(hi - lo + 1);
-        }
-    }
     const int bX = bx.b[0], bY = bx.b[1], bZ = bx.b[2], bR = bx.b[3];
     const size_t gfl = (size_t)bR * bX * bY * bZ;
     float *G = (float *)ws;
     float2 *Z1 = (float2 *)((char *)ws + l4_align(sizeof(float) * (size_t)nr * ns * ns * ns));
     float2 *Y1 = (float2 *)G;
-    lo_r = bx.lo[3];
-    b_r = bR;
     if ((e = cudaMemsetAsync(G, 0, sizeof(float) * gfl, s)) != cudaSuccess) return e;
     if (n > 0) {
         const int blocks = (n + 7) / 8 < 65535 ? (n + 7) / 8 : 65535;
@@ -443,8 +402,9 @@ static cudaError_t l4_rc_ns(const float2 *XA, const float2 *XB, int N, int loA, 
 
 cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                        const double (&RB)[9], double period, double period_r, const float2 *cone, const float *slices,
-                       int nslices, float scale, void *ws, float2 *h, int nsm, cudaStream_t s)
+                       int nslices, float scale, void *ws, float2 *h, bool *line, int *err, int nsm, cudaStream_t s)
 {
+    *line = false;
     const int ns = 2 * N, nr = 2 * Nr;
     if (nA == 0 || nB == 0) return cudaMemsetAsync(h, 0, sizeof(float2) * (size_t)N * N * (N / 2) * nslices, s);
     const double ip = 1.0 / period, ipr = 1.0 / period_r;
@@ -455,10 +415,51 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
         ra.R[k] = (k % 4 == 0) ? 1.0 : 0.0; // A unrotated
         rb.R[k] = RB[k];
     }
-    int loA = 0, bA = nr, loB = 0, bB = nr;
+    // both support boxes, one read-back
     cudaError_t e;
-    if ((e = l4_xplanes(t, N, Nr, kA, nA, ra, 0, ip, ipr, ws, XA, loA, bA, nsm, s)) != cudaSuccess) return e;
-    if ((e = l4_xplanes(t, N, Nr, kB, nB, rb, 1, ip, ipr, ws, Z1, loB, bB, nsm, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(t.dbox, 0x7f, 16 * sizeof(int), s)) != cudaSuccess) return e;
+    for (int k = 0; k < 2; k++) {
+        const int n = k ? nB : nA, blocks = std::min((n + 255) / 256, 4 * nsm);
+        k_l4_box<<<blocks, 256, 0, s>>>(k ? kB : kA, n, k ? rb : ra, k, ns, nr, ip, ipr, t.dbox + 8 * k);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if ((e = cudaMemcpyAsync(t.hbox, t.dbox, 16 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    L4Box bx[2], even[2]; // even: row pairs, 16-byte rows
+    bool inside = true;
+    for (int k = 0; k < 2; k++)
+        for (int a = 0; a < 4; a++) {
+            const int na = a < 3 ? ns : nr;
+            const long long lo = t.hbox[8 * k + a], hi = -(long long)t.hbox[8 * k + 4 + a] + L4_W - 1;
+            const bool whole = hi - lo + 1 >= na;
+            bx[k].lo[a] = whole ? 0 : (int)lo;
+            bx[k].b[a] = whole ? na : (int)(hi - lo + 1);
+            even[k].lo[a] = bx[k].lo[a];
+            even[k].b[a] = a == 1 || a == 2 ? (bx[k].b[a] + 1) & ~1 : bx[k].b[a];
+            inside = inside && !whole;
+        }
+    *line = inside && t.wts && lift4_line_fits(N, Nr, bx[0].b[3], bx[1].b[3], nslices);
+    if (*line) {
+        // spectra in turn over the same grid and y planes; A's x planes have their own
+        // place, B's take the grid's
+        InstPlan *hp = (InstPlan *)(t.hbox + 16), *dp = (InstPlan *)(t.dbox + 16);
+        const InstDesc *dd = (const InstDesc *)(dp + 2); // offsets zero
+        static_assert(16 * sizeof(int) + 2 * sizeof(InstPlan) + 2 * sizeof(InstDesc) <= LIFT4_BOX_BYTES, "box words");
+        std::memset(hp, 0, 2 * sizeof(InstPlan) + 2 * sizeof(InstDesc));
+        for (int k = 0; k < 2; k++)
+            for (int a = 0; a < 3; a++) hp[k].b[a] = even[k].b[a];
+        if ((e = cudaMemcpyAsync(dp, hp, 2 * sizeof(InstPlan) + 2 * sizeof(InstDesc), cudaMemcpyHostToDevice, s)) != cudaSuccess)
+            return e;
+        float *G = (float *)ws;
+        float2 *XB = (float2 *)ws;
+        if ((e = lift4_line_spectrum(t, N, Nr, kA, nA, ra, 0, ip, ipr, even[0], dp, dd, G, Z1, XA, err, nsm, s)) != cudaSuccess ||
+            (e = lift4_line_spectrum(t, N, Nr, kB, nB, rb, 1, ip, ipr, even[1], dp + 1, dd + 1, G, Z1, XB, err, nsm, s)) != cudaSuccess)
+            return e;
+        return lift4_line_collapse(t, N, Nr, XA, XB, even[0], even[1], slices, nslices, period_r, scale, h, err, nsm, s);
+    }
+    if ((e = l4_xplanes(t, N, Nr, kA, nA, ra, 0, ip, ipr, bx[0], ws, XA, nsm, s)) != cudaSuccess) return e;
+    if ((e = l4_xplanes(t, N, Nr, kB, nB, rb, 1, ip, ipr, bx[1], ws, Z1, nsm, s)) != cudaSuccess) return e;
+    const int loA = bx[0].lo[3], bA = bx[0].b[3], loB = bx[1].lo[3], bB = bx[1].b[3];
     switch (nr) {
     case 32: return l4_rc_ns<32>(XA, Z1, N, loA, bA, loB, bB, t, cone, slices, nslices, period_r, scale, h, nsm, s);
     case 64: return l4_rc_ns<64>(XA, Z1, N, loA, bA, loB, bB, t, cone, slices, nslices, period_r, scale, h, nsm, s);
