@@ -11,6 +11,10 @@
 namespace bc {
 
 constexpr int TB = 256; // threads per transform block
+// threads of a forward pass: 512-point lines fill one block per SM either way (135 KB of
+// tiles and more), so it takes twice the threads (a correlation at N = 256: 1,193 us, with
+// 256 threads 1,226)
+__host__ __device__ constexpr int tb_of(int NF) { return NF == 512 ? 512 : TB; }
 constexpr int CL = 16;  // interleaved lines per tile (16 complex = 128 bytes per tile row)
 
 // Block loop over the work items of a sequence of instances (or pairs),

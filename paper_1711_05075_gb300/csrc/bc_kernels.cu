@@ -503,10 +503,11 @@ cudaError_t launch_spread(const Geometry &g, const Tables &t, const InstDesc *in
 // Output rows: with Z = FFT(a + i b), A_k = (Z_k + conj Z_{n-k}) / 2,
 // B_k = (Z_k - conj Z_{n-k}) / (2i), for m_z = k in [0, N/2).
 template <int NF, bool SP, int S>
-__global__ void __launch_bounds__(TB, (NF <= 256 ? 2 : 1))
+__global__ void __launch_bounds__(tb_of(NF), (NF <= 256 ? 2 : 1))
 k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const InstPlan *__restrict__ plan,
         float *grid, float2 *z1)
 {
+    constexpr int NT = tb_of(NF);
     constexpr bool three = Radix<NF, S>::r2 > 1;
     extern __shared__ float4 sm4[];
     float2 *tw = reinterpret_cast<float2 *>(sm4);
@@ -518,7 +519,7 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
     pdl_wait(); // earlier passes' outputs are read from here on
     constexpr int H = NF / 4; // kept z modes (N/2, n = 2N)
     const int L = g.L;
-    FirstInputs<NF, Radix<NF, S>::r0, CL, TB> in;
+    FirstInputs<NF, Radix<NF, S>::r0, CL, NT> in;
     RotStart rs;
     for (int i = 0; i < ninst; i++) {
         const InstPlan p = plan[i];
@@ -542,21 +543,21 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             const int l = it / (b0 * nyb), rem = it - l * (b0 * nyb);
             const int ix = rem / nyb, iy0 = (rem - ix * nyb) << 5;
             if constexpr (SP) in.scatter(S0);
-            else rr_first<NF, Radix<NF, S>::r0, false, CL, TB>(in, S0);
+            else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
             __syncthreads(); // every thread has consumed its loads of this item
             {
                 // the item's box rows are one contiguous run of bz x 128 bytes
                 float4 *run = reinterpret_cast<float4 *>(G2 + (long long)it * bz * 16);
-                for (int e = threadIdx.x; e < bz * 8; e += TB) run[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = threadIdx.x; e < bz * 8; e += NT) run[e] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
             if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
             auto sink = [&](int, int, int c, int pos, float2 v) { OUT[pos * CL + c] = v; };
-            if constexpr (SP) sp_all<NF, false, CL, TB, S>(S0, S1, tw, sink);
-            else rr_rest<NF, false, CL, TB, S>(S0, S1, tw, sink);
+            if constexpr (SP) sp_all<NF, false, CL, NT, S>(S0, S1, tw, sink);
+            else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
             __syncthreads();
             // unpack into a staging area [row][k] (row stride H + 1), then write
             // each 8H-byte row of z1 with consecutive threads on consecutive k
-            for (int e = threadIdx.x; e < 32 * H; e += TB) {
+            for (int e = threadIdx.x; e < 32 * H; e += NT) {
                 const int r = e & 31, kk = e >> 5;
                 const int qq = r >> 1;
                 const float2 zk = OUT[kk * CL + qq];
@@ -567,7 +568,7 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             __syncthreads();
             float2 *Z = z1 + d.z1_off + (((long long)l * b0 + ix) * b1 + iy0) * H;
             const int rows = min(32, b1 - iy0);
-            for (int e = threadIdx.x; e < rows * H; e += TB) {
+            for (int e = threadIdx.x; e < rows * H; e += NT) {
                 const int r = e / H, kk = e - r * H;
                 Z[(long long)r * H + kk] = STG[r * (H + 1) + kk];
             }
@@ -593,10 +594,11 @@ struct YStaged {
 };
 
 template <int NF, bool SP, int S>
-__global__ void __launch_bounds__(TB, (NF <= 256 ? 2 : 1))
+__global__ void __launch_bounds__(tb_of(NF), (NF <= 256 ? 2 : 1))
 k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const InstPlan *__restrict__ plan,
         const float2 *__restrict__ z1, float2 *y1)
 {
+    constexpr int NT = tb_of(NF);
     extern __shared__ float4 sm4[];
     float2 *tw = reinterpret_cast<float2 *>(sm4);
     float2 *S0 = tw + NF, *S1 = S0 + NF * CL;
@@ -620,7 +622,7 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             auto fetch = [&](int it, float2 *dst) {
                 const int lx = it / nch, ch = it - lx * nch;
                 const float2 *base = z1 + d.z1_off + (long long)lx * b1 * H + ch * CL;
-                for (int q = threadIdx.x; q < NF * CL / 2; q += TB) {
+                for (int q = threadIdx.x; q < NF * CL / 2; q += NT) {
                     const int pos = q / (CL / 2), cc = (q % (CL / 2)) * 2;
                     int iy = pos - py;
                     if (iy < 0) iy += NF;
@@ -637,7 +639,7 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                 cp_async_commit();
                 cp_async_wait_prev();
                 __syncthreads();
-                il_stage<NF, Radix<NF, S>::r0, 1, false, CL, TB>(B(k), S0, tw);
+                il_stage<NF, Radix<NF, S>::r0, 1, false, CL, NT>(B(k), S0, tw);
                 __syncthreads();
                 const int lx = it / nch, ch = it - lx * nch;
                 float2 *Y = y1 + d.y1_off + (long long)lx * N * H + ch * CL;
@@ -648,13 +650,13 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                     else return;
                     Y[(long long)jy * H + c] = jy == N / 2 ? make_float2(0.f, 0.f) : v;
                 };
-                rr_rest<NF, false, CL, TB, S>(S0, S1, tw, sink);
+                rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
                 __syncthreads();
             }
             rs.rot += items;
         }
     } else {
-        FirstInputs<NF, Radix<NF, S>::r0, CL, TB> in;
+        FirstInputs<NF, Radix<NF, S>::r0, CL, NT> in;
         for (int i = 0; i < ninst; i++) {
             const InstPlan p = plan[i];
             if (p.b[0] == 0) continue;
@@ -675,7 +677,7 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             for (; it < items; it += gridDim.x) {
                 const int lx = it / nch, ch = it - lx * nch;
                 if constexpr (SP) in.scatter(S0);
-                else rr_first<NF, Radix<NF, S>::r0, false, CL, TB>(in, S0);
+                else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
                 __syncthreads();
                 if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
                 float2 *Y = y1 + d.y1_off + (long long)lx * N * H + ch * CL;
@@ -686,8 +688,8 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                     else return;
                     Y[(long long)jy * H + c] = jy == N / 2 ? make_float2(0.f, 0.f) : v;
                 };
-                if constexpr (SP) sp_all<NF, false, CL, TB, S>(S0, S1, tw, sink);
-                else rr_rest<NF, false, CL, TB, S>(S0, S1, tw, sink);
+                if constexpr (SP) sp_all<NF, false, CL, NT, S>(S0, S1, tw, sink);
+                else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
                 __syncthreads();
             }
             rs.rot += items;
@@ -796,7 +798,7 @@ k_fft_y_shift(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int nins
 // (bc_passes.cuh): forward x transform of both spectra with the level sum,
 // conjugate product and inverse x transform.
 template <int NF, int NI, bool SP, int S>
-__global__ void __launch_bounds__(TB, (NF <= 256 ? 2 : 1))
+__global__ void __launch_bounds__(tb_of(NF), (NF <= 256 ? 2 : 1))
 k_fft_x(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *__restrict__ plan,
         const PairDesc *__restrict__ pairs, int npairs, const float2 *__restrict__ y1,
         const float2 *__restrict__ fa_cache, float2 *fa_out, float2 *h, int G)
@@ -815,7 +817,7 @@ k_fft_x(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan
         const PairDesc pr = pairs[pi];
         for (int it = rs.first(); it < items; it += gridDim.x) {
             const int jy = it / nch, ch = it - jy * nch;
-            x_item<NF, NI, SP, S>(g, tb, inst, plan, pr, jy, ch, y1, fa_cache, fa_out, h, G, sm);
+            x_item<NF, NI, SP, S, tb_of(NF)>(g, tb, inst, plan, pr, jy, ch, y1, fa_cache, fa_out, h, G, sm);
         }
         rs.rot += items;
     }
@@ -1083,7 +1085,7 @@ static cudaError_t fft_z_t(const Geometry &g, const Tables &t, const InstDesc *i
     const size_t smem = sizeof(float2) * (NF + 2 * NF * CL);
     cudaError_t e = set_smem(k_fft_z<NF, SP, S>, smem);
     if (e != cudaSuccess) return e;
-    return launch_k(k_fft_z<NF, SP, S>, resident_blocks(k_fft_z<NF, SP, S>, smem, nsm), TB, smem, s, g.pdl != 0, g, t,
+    return launch_k(k_fft_z<NF, SP, S>, resident_blocks(k_fft_z<NF, SP, S>, smem, nsm, tb_of(NF)), tb_of(NF), smem, s, g.pdl != 0, g, t,
                     inst, ninst, plan, grid, z1);
 }
 
@@ -1127,7 +1129,7 @@ static cudaError_t fft_y_t(const Geometry &g, const Tables &t, const InstDesc *i
     const size_t smem = sizeof(float2) * (NF + (YStaged<NF, SP, S>::on ? 3 : 2) * NF * CL);
     cudaError_t e = set_smem(k_fft_y<NF, SP, S>, smem);
     if (e != cudaSuccess) return e;
-    return launch_k(k_fft_y<NF, SP, S>, resident_blocks(k_fft_y<NF, SP, S>, smem, nsm), TB, smem, s, g.pdl != 0, g, t,
+    return launch_k(k_fft_y<NF, SP, S>, resident_blocks(k_fft_y<NF, SP, S>, smem, nsm, tb_of(NF)), tb_of(NF), smem, s, g.pdl != 0, g, t,
                     inst, ninst, plan, z1, y1);
 }
 
@@ -1169,7 +1171,7 @@ static cudaError_t fft_x_t(const Geometry &g, const Tables &t, const InstDesc *i
     const size_t smem = XL::bytes(G);
     cudaError_t e = set_smem(k_fft_x<NF, NI, SP, S>, smem);
     if (e != cudaSuccess) return e;
-    return launch_k(k_fft_x<NF, NI, SP, S>, resident_blocks(k_fft_x<NF, NI, SP, S>, smem, nsm), TB, smem, s,
+    return launch_k(k_fft_x<NF, NI, SP, S>, resident_blocks(k_fft_x<NF, NI, SP, S>, smem, nsm, tb_of(NF)), tb_of(NF), smem, s,
                     g.pdl != 0, g, t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, G);
 }
 

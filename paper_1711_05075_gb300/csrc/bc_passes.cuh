@@ -26,10 +26,10 @@ __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wa
 // (m_x = pos - n), i.e. exactly m_x in [-N/2, N/2); those slots of F hold
 // sum_l T_l(|m|^2) D(m) FFT_x[Y_l](m) for m_y = mode(j_y), m_z = 16 ch + c.
 // Level l + 1 is loaded while level l is transformed.
-template <int NF, int S>
+template <int NF, int S, int NT>
 struct XModes {
     static constexpr int R = LastStage<NF, S>::R, NS = LastStage<NF, S>::NS;
-    static constexpr int IT = (NS * CL + TB - 1) / TB;
+    static constexpr int IT = (NS * CL + NT - 1) / NT;
     static __device__ __forceinline__ constexpr bool kept(int r) { return r < R / 4 || r >= 3 * R / 4; }
 };
 
@@ -40,7 +40,7 @@ struct XModes {
 // m_x = a and m_x = -a; the index a = N/2 addresses m_x = -N/2 in the
 // deconvolution table's FFT order.  Built in shared memory by the whole block,
 // it replaces the table gathers of every level of both spectra.
-template <int NI>
+template <int NI, int NT>
 __device__ __forceinline__ void build_xweights(float *Ts, const Tables &tb, int l0, int nl, int jy, int ch)
 {
     constexpr int A = NI / 2 + 1;
@@ -48,7 +48,7 @@ __device__ __forceinline__ void build_xweights(float *Ts, const Tables &tb, int 
     const float dy = tb.deconv[jy];
     const long long Q = tb.qmax + 1;
     const int tot = nl * A * CL;
-    for (int e = threadIdx.x; e < tot; e += TB) {
+    for (int e = threadIdx.x; e < tot; e += NT) {
         const int c = e % CL, a = (e / CL) % A, lg = e / (CL * A);
         const int mz = ch * CL + c;
         Ts[e] = tb.ballft[(l0 + lg) * Q + a * a + my * my + mz * mz] * (tb.deconv[a] * dy * tb.deconv[mz]);
@@ -58,14 +58,14 @@ __device__ __forceinline__ void build_xweights(float *Ts, const Tables &tb, int 
 // Ts holds the weights of levels [ts_base, ts_base + G) of the current item;
 // a level outside that range rebuilds it (after the barrier that ends the
 // previous level, before the one that publishes the level's first stage).
-template <int NF, int NI, bool SP, int S>
-__device__ __forceinline__ void spectrum_x(float2 (&F)[XModes<NF, S>::IT][XModes<NF, S>::R], const Geometry &g,
+template <int NF, int NI, bool SP, int S, int NT>
+__device__ __forceinline__ void spectrum_x(float2 (&F)[XModes<NF, S, NT>::IT][XModes<NF, S, NT>::R], const Geometry &g,
                                            const Tables &tb, const InstDesc *__restrict__ inst,
                                            const InstPlan *__restrict__ plan, int si, const float2 *__restrict__ y1,
                                            int jy, int ch, const float2 *tw, float2 *S0, float2 *S1, float *Ts, int G,
                                            int &ts_base)
 {
-    using XM = XModes<NF, S>;
+    using XM = XModes<NF, S, NT>;
     constexpr int H = NI / 2, N = NI, A = NI / 2 + 1;
     const int L = g.L;
 #pragma unroll
@@ -84,15 +84,15 @@ __device__ __forceinline__ void spectrum_x(float2 (&F)[XModes<NF, S>::IT][XModes
             return ix < b0 ? base[(long long)ix * N * H + c] : make_float2(0.f, 0.f);
         };
     };
-    FirstInputs<NF, Radix<NF, S>::r0, CL, TB> in;
+    FirstInputs<NF, Radix<NF, S>::r0, CL, NT> in;
     in.load(src(0));
     for (int l = 0; l < L; l++) {
         if (l < ts_base || l >= ts_base + G) {
             ts_base = l;
-            build_xweights<NI>(Ts, tb, l, min(G, L - l), jy, ch);
+            build_xweights<NI, NT>(Ts, tb, l, min(G, L - l), jy, ch);
         }
         if constexpr (SP) in.scatter(S0);
-        else rr_first<NF, Radix<NF, S>::r0, false, CL, TB>(in, S0);
+        else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
         __syncthreads();
         if (l + 1 < L) in.load(src(l + 1));
         const float *Tl = Ts + (l - ts_base) * A * CL;
@@ -102,21 +102,21 @@ __device__ __forceinline__ void spectrum_x(float2 (&F)[XModes<NF, S>::IT][XModes
             const float Mv = Tl[(mx < 0 ? -mx : mx) * CL + c];
             F[it][r] = make_float2(fmaf(Mv, v.x, F[it][r].x), fmaf(Mv, v.y, F[it][r].y));
         };
-        if constexpr (SP) sp_all<NF, false, CL, TB, S>(S0, S1, tw, sink);
-        else rr_rest<NF, false, CL, TB, S>(S0, S1, tw, sink);
+        if constexpr (SP) sp_all<NF, false, CL, NT, S>(S0, S1, tw, sink);
+        else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
         __syncthreads();
     }
 }
 
 // Calls f(it, r, c, jx) for every kept mode slot of the calling thread.
-template <int NF, int NI, int S, class Fn>
+template <int NF, int NI, int S, int NT, class Fn>
 __device__ __forceinline__ void for_kept(Fn f)
 {
-    using XM = XModes<NF, S>;
+    using XM = XModes<NF, S, NT>;
 #pragma unroll
     for (int it = 0; it < XM::IT; it++) {
-        const int idx = (int)threadIdx.x + it * TB;
-        if ((XM::NS * CL) % TB != 0 && idx >= XM::NS * CL) break;
+        const int idx = (int)threadIdx.x + it * NT;
+        if ((XM::NS * CL) % NT != 0 && idx >= XM::NS * CL) break;
         const int c = idx % CL, j = idx / CL;
 #pragma unroll
         for (int r = 0; r < XM::R; r++) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
                                               const float2 *__restrict__ y1, const float2 *__restrict__ fa_cache,
                                               float2 *fa_out, float2 *h, int G, const typename XSmem<NF, NI, SP, S>::Ptr &sm)
 {
-    using XM = XModes<NF, S>;
+    using XM = XModes<NF, S, TB>;
     using XS = XStage<NF, SP, S>;
     constexpr int H = NI / 2, N = NI, A = NI / 2 + 1;
     const int L = g.L;
@@ -254,7 +254,7 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
     };
     zero_f();
     if (!hasA) { // F_A from the cached spectrum (already in place)
-        for_kept<NF, NI, S>([&](int, int, int c, int jx) {
+        for_kept<NF, NI, S, TB>([&](int, int, int c, int jx) {
             sm.FAt[jx * CL + c] = fa_cache[((long long)jx * N + jy) * H + ch * CL + c];
         });
     }
@@ -276,7 +276,7 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
         const int l = ph < L ? ph : ph - L;
         if (l < ts_base || l >= ts_base + G) {
             ts_base = l;
-            build_xweights<NI>(sm.Ts, tb, l, min(G, L - l), jy, ch);
+            build_xweights<NI, TB>(sm.Ts, tb, l, min(G, L - l), jy, ch);
         }
         __syncthreads(); // this phase's rows (every thread's copies) have landed
         xs_first<NF, SP, S>(cur, sm.S0);
@@ -293,7 +293,7 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
         if (l == L - 1) { // this instance's level sum is complete: restore its box origin
             const int px = plan[inst_of(ph)].pos0[0];
             const bool isA = hasA && ph < L;
-            for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) {
+            for_kept<NF, NI, S, TB>([&](int i2, int r, int c, int jx) {
                 const int mx = jx < N / 2 ? jx : jx - N;
                 const float2 v = cmul(F[i2][r], box_phase<NF>(sm.twF, mx, px));
                 if (isA) sm.FAt[jx * CL + c] = v;
@@ -303,12 +303,12 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
         }
     }
     if (!hasB) {
-        for_kept<NF, NI, S>([&](int, int, int c, int jx) {
+        for_kept<NF, NI, S, TB>([&](int, int, int c, int jx) {
             fa_out[((long long)jx * N + jy) * H + ch * CL + c] = sm.FAt[jx * CL + c];
         });
         return;
     }
-    for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) {
+    for_kept<NF, NI, S, TB>([&](int i2, int r, int c, int jx) {
         const int mx = mode_of(jx, N), mz = ch * CL + c;
         float2 v = make_float2(0.f, 0.f);
         if (jx != N / 2 && jy != N / 2) {
@@ -334,20 +334,21 @@ __device__ __forceinline__ void x_item_staged(const Geometry &g, const Tables &t
 // With pr.a < 0, F_A comes from the cached spectrum; with pr.b < 0, F_A is
 // written to `fa_out` and nothing else happens.  All threads call it; it ends
 // with a block barrier except when pr.b < 0.
-template <int NF, int NI, bool SP, int S>
+template <int NF, int NI, bool SP, int S, int NT = TB>
 __device__ __forceinline__ void x_item(const Geometry &g, const Tables &tb, const InstDesc *__restrict__ inst,
                                        const InstPlan *__restrict__ plan, const PairDesc &pr, int jy, int ch,
                                        const float2 *__restrict__ y1, const float2 *__restrict__ fa_cache,
                                        float2 *fa_out, float2 *h, int G, const typename XSmem<NF, NI, SP, S>::Ptr &sm)
 {
     if constexpr (XStage<NF, SP, S>::on) {
+        static_assert(NT == TB, "staged x pass");
         constexpr int MAXR = XStage<NF, SP, S>::MAXR;
         if ((pr.a < 0 || plan[pr.a].b[0] <= MAXR) && (pr.b < 0 || plan[pr.b].b[0] <= MAXR)) {
             x_item_staged<NF, NI, SP, S>(g, tb, inst, plan, pr, jy, ch, y1, fa_cache, fa_out, h, G, sm);
             return;
         }
     }
-    using XM = XModes<NF, S>;
+    using XM = XModes<NF, S, NT>;
     constexpr int H = NI / 2, N = NI;
     const float2 *twF = sm.twF, *twI = sm.twI;
     float2 *S0 = sm.S0, *S1 = sm.S1, *FAt = sm.FAt;
@@ -360,23 +361,23 @@ __device__ __forceinline__ void x_item(const Geometry &g, const Tables &tb, cons
     {
         float2 FA[XM::IT][XM::R];
         if (pr.a < 0) {
-            for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) {
+            for_kept<NF, NI, S, NT>([&](int i2, int r, int c, int jx) {
                 FAt[jx * CL + c] = fa_cache[((long long)jx * N + jy) * H + ch * CL + c];
             });
         } else {
-            spectrum_x<NF, NI, SP, S>(FA, g, tb, inst, plan, pr.a, y1, jy, ch, twF, S0, S1, Ts, G, ts_base);
-            for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) { FAt[jx * CL + c] = FA[i2][r]; });
+            spectrum_x<NF, NI, SP, S, NT>(FA, g, tb, inst, plan, pr.a, y1, jy, ch, twF, S0, S1, Ts, G, ts_base);
+            for_kept<NF, NI, S, NT>([&](int i2, int r, int c, int jx) { FAt[jx * CL + c] = FA[i2][r]; });
         }
     }
     if (pr.b < 0) {
-        for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) {
+        for_kept<NF, NI, S, NT>([&](int i2, int r, int c, int jx) {
             fa_out[((long long)jx * N + jy) * H + ch * CL + c] = FAt[jx * CL + c];
         });
         return;
     }
     float2 FB[XM::IT][XM::R];
-    spectrum_x<NF, NI, SP, S>(FB, g, tb, inst, plan, pr.b, y1, jy, ch, twF, S0, S1, Ts, G, ts_base);
-    for_kept<NF, NI, S>([&](int i2, int r, int c, int jx) {
+    spectrum_x<NF, NI, SP, S, NT>(FB, g, tb, inst, plan, pr.b, y1, jy, ch, twF, S0, S1, Ts, G, ts_base);
+    for_kept<NF, NI, S, NT>([&](int i2, int r, int c, int jx) {
         const int mx = mode_of(jx, N), mz = ch * CL + c;
         float2 v = make_float2(0.f, 0.f);
         if (jx != N / 2 && jy != N / 2) {
@@ -386,9 +387,9 @@ __device__ __forceinline__ void x_item(const Geometry &g, const Tables &tb, cons
         S0[jx * CL + c] = v;
     });
     __syncthreads();
-    const float2 *res = il_fft<NI, true, CL, TB>(S0, S1, twI);
+    const float2 *res = il_fft<NI, true, CL, NT>(S0, S1, twI);
     float2 *Hp = h + pr.h_off + (long long)jy * H + ch * CL + 2 * part;
-    for (int kx = r8; kx < N; kx += TB / 8)
+    for (int kx = r8; kx < N; kx += NT / 8)
         *reinterpret_cast<float4 *>(Hp + (long long)kx * N * H) = *reinterpret_cast<const float4 *>(res + kx * CL + 2 * part);
     __syncthreads();
 }
