@@ -19,6 +19,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace bc {
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
@@ -171,12 +173,35 @@ struct SplitSched {
     static constexpr int S = NF == 256 ? 1 : 0;
 };
 
+// Column order of a tile row.  Natural: value c of row pos at column c.  Swz: at
+// column c ^ f(pos), f from the row's place in the strides of the tensor-core
+// stage that reads the tile (A, 0: none) and of the one that writes it (B, 0:
+// none).  Those stages touch 4 rows A (B) apart with the lanes of one access, 8
+// (read) and 4 (written) columns of each, and whole rows are a multiple of the
+// 32 banks: unswizzled, the 4 rows fall on the same banks (a split correlation
+// at N = 128, L = 4: 579 us, swizzled 527).
+struct Natural {
+    static __device__ __forceinline__ int at(int, int c) { return c; }
+};
+template <int A, int B>
+struct Swz {
+    static __device__ __forceinline__ int at(int pos, int c)
+    {
+        if constexpr (A > 0) c ^= ((pos / A) & 3) << 2;
+        if constexpr (B > 0) {
+            const int x = pos / B;
+            c ^= (x & 1) | ((x & 2) << 2);
+        }
+        return c;
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Interleaved tiles: C lines stored as x[pos * C + c].  Consecutive threads take
 // consecutive lines c of the same butterfly, so every shared-memory access of
 // a stage is a run of C consecutive complex values (no bank conflicts), and a
 // tile row of C values is one 8C-byte run in global memory as well.
-template <int NF, int R, int NS, bool INV, int C, int NT>
+template <int NF, int R, int NS, bool INV, int C, int NT, class In = Natural, class Out = Natural>
 __device__ __forceinline__ void il_stage(const float2 *__restrict__ in, float2 *__restrict__ out,
                                          const float2 *__restrict__ tw)
 {
@@ -192,7 +217,7 @@ __device__ __forceinline__ void il_stage(const float2 *__restrict__ in, float2 *
         float2 v[R];
 #pragma unroll
         for (int r = 0; r < R; r++) {
-            float2 x = in[(j + r * NB) * C + c];
+            float2 x = in[(j + r * NB) * C + In::at(j + r * NB, c)];
             if (NS > 1 && r > 0) {
                 float2 w = tw[r * k * (NF / (NS * R))];
                 if (INV) w.y = -w.y;
@@ -203,7 +228,7 @@ __device__ __forceinline__ void il_stage(const float2 *__restrict__ in, float2 *
         dft_small<R, INV>(v);
         const int base = (j / NS) * NS * R + k;
 #pragma unroll
-        for (int r = 0; r < R; r++) out[(base + r * NS) * C + c] = v[r];
+        for (int r = 0; r < R; r++) out[(base + r * NS) * C + Out::at(base + r * NS, c)] = v[r];
     }
 }
 
@@ -254,7 +279,8 @@ struct FirstInputs {
                 v[it][r] = ((TOT % NT) == 0 || idx < TOT) ? src(c, j + r * NB) : make_float2(0.f, 0.f);
         }
     }
-    // Writes the loaded values to their positions of a tile (tile[pos * C + c]).
+    // Writes the loaded values to their positions of a tile in column order `Out`.
+    template <class Out = Natural>
     __device__ __forceinline__ void scatter(float2 *tile) const
     {
 #pragma unroll
@@ -263,7 +289,7 @@ struct FirstInputs {
             if ((TOT % NT) != 0 && idx >= TOT) break;
             const int c = idx % C, j = idx / C;
 #pragma unroll
-            for (int r = 0; r < R; r++) tile[(j + r * NB) * C + c] = v[it][r];
+            for (int r = 0; r < R; r++) tile[(j + r * NB) * C + Out::at(j + r * NB, c)] = v[it][r];
         }
     }
     // visit(c, pos) for every position load() read.
@@ -398,14 +424,14 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <int NF, int NS, bool INV, int C, int NT>
+template <int NF, int NS, bool INV, int C, int NT, class In, class Out>
 __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 *__restrict__ out,
                                           const float2 *__restrict__ tw)
 {
     constexpr int R = 8, NB = NF / R, TOT = NB * C, GROUPS = TOT / 8;
-    static_assert(TOT % 8 == 0, "groups of 8 butterflies");
+    static_assert(C == 16 && (NT / 32) % 2 == 0, "a group: half a row of butterflies; a warp keeps its half");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
+    const int g = lane >> 2, t = lane & 3, c0 = (warp & 1) * 8;
     // A fragments of F, split into hi and lo
     unsigned ahi[4], alo[4];
     {
@@ -422,11 +448,10 @@ __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 
     }
     float *outf = reinterpret_cast<float *>(out);
     for (int grp = warp; grp < GROUPS; grp += NT / 32) {
-        // inputs r = t and r = t + 4 of butterfly b = 8 grp + g
-        const int b = grp * 8 + g;
-        const int c = b % C, j = b / C, k = j % NS;
-        float2 x0 = in[(j + t * NB) * C + c];
-        float2 x1 = in[(j + (t + 4) * NB) * C + c];
+        // inputs r = t and r = t + 4 of butterfly (j, c)
+        const int c = c0 + g, j = grp >> 1, k = j % NS;
+        float2 x0 = in[(j + t * NB) * C + In::at(j + t * NB, c)];
+        float2 x1 = in[(j + (t + 4) * NB) * C + In::at(j + (t + 4) * NB, c)];
         if (NS > 1) {
             if (t > 0) {
                 float2 w = tw[t * k * (NF / (NS * R))];
@@ -448,28 +473,38 @@ __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 
         mma_bf16(d, ahi, bl0, bl1);
         mma_bf16(d, alo, bh0, bh1);
         // d[0] = C[g][2t], d[1] = C[g][2t+1], d[2] = C[g+8][2t], d[3] = C[g+8][2t+1]
+        const int p = g & 1, lo = (j / NS) * NS * R + k + (g >> 1) * NS, hi = lo + 4 * NS;
 #pragma unroll
         for (int u = 0; u < 2; u++) {
-            const int bb = grp * 8 + 2 * t + u;
-            const int cc = bb % C, jj = bb / C, kk2 = jj % NS;
-            const int base = (jj / NS) * NS * R + kk2;
-            const int p = g & 1, r0 = g >> 1;
-            outf[((base + r0 * NS) * C + cc) * 2 + p] = d[u];
-            outf[((base + (r0 + 4) * NS) * C + cc) * 2 + p] = d[2 + u];
+            const int cc = c0 + 2 * t + u;
+            outf[(lo * C + Out::at(lo, cc)) * 2 + p] = d[u];
+            outf[(hi * C + Out::at(hi, cc)) * 2 + p] = d[2 + u];
         }
     }
 }
 
 // A stage of the split-precision schedule: tensor-core DFT for radix 8, FP32 otherwise.
-template <int NF, int R, int NS, bool INV, int C, int NT>
+template <int NF, int R, int NS, bool INV, int C, int NT, class In, class Out>
 __device__ __forceinline__ void sp_stage(const float2 *in, float2 *out, const float2 *tw)
 {
-    if constexpr (R == 8) tc_stage8<NF, NS, INV, C, NT>(in, out, tw);
-    else il_stage<NF, R, NS, INV, C, NT>(in, out, tw);
+    if constexpr (R == 8) tc_stage8<NF, NS, INV, C, NT, In, Out>(in, out, tw);
+    else il_stage<NF, R, NS, INV, C, NT, In, Out>(in, out, tw);
 }
 
+// Column orders of the tiles of a split-precision transform: its input, after
+// the first, the second and the last stage.
+template <int NF, int S>
+struct SplitTiles {
+    using R = Radix<NF, S>;
+    static constexpr int NB = NF / 8;
+    using Input = Swz<R::r0 == 8 ? NB : 0, 0>;
+    using T1 = Swz<R::r1 == 8 ? NB : 0, R::r0 == 8 ? 1 : 0>;
+    using T2 = Swz<R::r2 == 8 ? NB : 0, R::r1 == 8 ? R::r0 : 0>;
+    using T3 = Swz<0, R::r2 == 8 ? R::r0 * R::r1 : 0>;
+};
+
 // Split-precision transform of a tile whose inputs were scattered into s0 by
-// FirstInputs::scatter (natural order, whatever the loading schedule); then
+// FirstInputs::scatter in the order SplitTiles::Input; then
 // sink(it, r, c, pos, value) in the thread mapping of rr_last for radix
 // schedule S.  All threads call it; the caller adds a barrier before s0/s1 are
 // written again.
@@ -477,16 +512,18 @@ template <int NF, bool INV, int C, int NT, int S, class Sink>
 __device__ __forceinline__ void sp_all(float2 *s0, float2 *s1, const float2 *tw, Sink sink)
 {
     using R = Radix<NF, S>;
-    sp_stage<NF, R::r0, 1, INV, C, NT>(s0, s1, tw);
+    using ST = SplitTiles<NF, S>;
+    sp_stage<NF, R::r0, 1, INV, C, NT, typename ST::Input, typename ST::T1>(s0, s1, tw);
     __syncthreads();
-    sp_stage<NF, R::r1, R::r0, INV, C, NT>(s1, s0, tw);
+    sp_stage<NF, R::r1, R::r0, INV, C, NT, typename ST::T1, typename ST::T2>(s1, s0, tw);
     __syncthreads();
     const float2 *fin = s0;
     if constexpr (R::r2 > 1) {
-        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT>(s0, s1, tw);
+        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT, typename ST::T2, typename ST::T3>(s0, s1, tw);
         __syncthreads();
         fin = s1;
     }
+    using Fin = std::conditional_t<(R::r2 > 1), typename ST::T3, typename ST::T2>;
     constexpr int RL = LastStage<NF, S>::R, NSL = LastStage<NF, S>::NS, TOT = NSL * C, IT = (TOT + NT - 1) / NT;
 #pragma unroll
     for (int it = 0; it < IT; it++) {
@@ -494,7 +531,7 @@ __device__ __forceinline__ void sp_all(float2 *s0, float2 *s1, const float2 *tw,
         if ((TOT % NT) != 0 && idx >= TOT) break;
         const int c = idx % C, j = idx / C;
 #pragma unroll
-        for (int r = 0; r < RL; r++) sink(it, r, c, j + r * NSL, fin[(j + r * NSL) * C + c]);
+        for (int r = 0; r < RL; r++) sink(it, r, c, j + r * NSL, fin[(j + r * NSL) * C + Fin::at(j + r * NSL, c)]);
     }
 }
 

@@ -542,7 +542,7 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
         for (; it < items; it += gridDim.x) {
             const int l = it / (b0 * nyb), rem = it - l * (b0 * nyb);
             const int ix = rem / nyb, iy0 = (rem - ix * nyb) << 5;
-            if constexpr (SP) in.scatter(S0);
+            if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
             else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
             __syncthreads(); // every thread has consumed its loads of this item
             {
@@ -676,7 +676,7 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             if (it < items) in.load(src(it));
             for (; it < items; it += gridDim.x) {
                 const int lx = it / nch, ch = it - lx * nch;
-                if constexpr (SP) in.scatter(S0);
+                if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
                 else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
                 __syncthreads();
                 if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
