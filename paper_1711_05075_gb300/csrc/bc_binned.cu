@@ -269,7 +269,7 @@ k_fft_z_binned(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int nin
                 return make_float2((float)v.x * inv_scale, (float)v.y * inv_scale);
             });
             __syncthreads(); // the tile is in registers; S1 is free for the transform
-            if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
+            if constexpr (SP) sp_first<NF, CL, TB, S>(in, S0, S1);
             else rr_first<NF, Radix<NF, S>::r0, false, CL, TB>(in, S0);
             __syncthreads();
             auto sink = [&](int, int, int c, int pos, float2 v) { OUT[pos * CL + c] = v; };

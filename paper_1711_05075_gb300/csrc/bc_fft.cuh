@@ -179,7 +179,7 @@ struct SplitSched {
 // none).  Those stages touch 4 rows A (B) apart with the lanes of one access, 8
 // (read) and 4 (written) columns of each, and whole rows are a multiple of the
 // 32 banks: unswizzled, the 4 rows fall on the same banks (a split correlation
-// at N = 128, L = 4: 579 us, swizzled 527).
+// at N = 128, L = 4, 20,000 + 20,000 balls: 579 us, swizzled 527).
 struct Natural {
     static __device__ __forceinline__ int at(int, int c) { return c; }
 };
@@ -307,8 +307,8 @@ struct FirstInputs {
     }
 };
 
-// First stage (Ns = 1, no twiddles): registers -> out[pos * C + c].
-template <int NF, int R, bool INV, int C, int NT>
+// First stage (Ns = 1, no twiddles): registers -> out, column order `Out`.
+template <int NF, int R, bool INV, int C, int NT, class Out = Natural>
 __device__ __forceinline__ void rr_first(const FirstInputs<NF, R, C, NT> &in, float2 *__restrict__ out)
 {
     using FI = FirstInputs<NF, R, C, NT>;
@@ -322,7 +322,7 @@ __device__ __forceinline__ void rr_first(const FirstInputs<NF, R, C, NT> &in, fl
         for (int r = 0; r < R; r++) v[r] = in.v[it][r];
         dft_small<R, INV>(v);
 #pragma unroll
-        for (int r = 0; r < R; r++) out[(j * R + r) * C + c] = v[r];
+        for (int r = 0; r < R; r++) out[(j * R + r) * C + Out::at(j * R + r, c)] = v[r];
     }
 }
 
@@ -388,32 +388,45 @@ __device__ __forceinline__ void rr_rest(float2 *s0, float2 *s1, const float2 *tw
 // transforms 8 butterflies.  Both F and the twiddled inputs are split into
 // BF16 hi + lo parts (hi = bf16(v), lo = bf16(v - hi)); the product is formed
 // as F_hi x_hi + F_hi x_lo + F_lo x_hi with FP32 accumulation (the lo x lo term,
-// of relative size 2^-32, is dropped).  Lane (g, t) of a warp loads inputs
+// of relative size 2^-18 at most, is dropped).  Lane (g, t) of a warp loads inputs
 // r = t and r = t + 4 of butterfly g of the group (the B fragment layout) and
 // receives output components g and g + 8 of butterflies 2t and 2t + 1.
-__device__ __forceinline__ float dft8_entry(int m, int k, bool inv)
+//
+// Bound by issued instructions, so the stage spends few beside the products: F is
+// built from one entry, each complex value is split with two conversions, no lane
+// branches, two groups are in flight, a FP32 first stage runs on the registers
+// that hold its inputs, and the z pass unpacks straight from the result tile.
+// Split correlation at N = 128, L = 4, 20,000 + 20,000 balls: 527 us -> 283.
+//
+// The lane's words of F as a pair (hi, lo), of which the entry (r', r) = (g / 2,
+// t) is computed: 4 more on r' or on r turns the angle by pi times t or r', so the
+// other three words are that one with its signs flipped or not.
+template <bool INV>
+__device__ __forceinline__ void dft8_words(int g, int t, unsigned (&hi)[4], unsigned (&lo)[4])
 {
-    // A[m][k], m = 2 r' + p, k = 2 r + q: the 2 x 2 real block of exp(-+i theta), theta = 2 pi r r' / 8
-    const float h = 0.70710678118654752440f;
-    const int e = ((m >> 1) * (k >> 1)) & 7;
-    // cos and sin of e pi / 4
-    const float c = e == 0 ? 1.f : e == 4 ? -1.f : (e == 2 || e == 6) ? 0.f : (e == 1 || e == 7) ? h : -h;
-    const float sv = e == 2 ? 1.f : e == 6 ? -1.f : (e == 0 || e == 4) ? 0.f : (e == 1 || e == 3) ? h : -h;
-    const float s = inv ? -sv : sv;
-    const int p = m & 1, q = k & 1;
-    return p == 0 ? (q == 0 ? c : s) : (q == 0 ? -s : c);
+    // rows p = 0: (cos, sin), p = 1: (-sin, cos) of e pi / 4 (sin negated for the inverse)
+    const int e = ((g >> 1) * t) & 7;
+    const bool odd = e & 1;
+    const unsigned H = odd ? 0x3f35u : 0x3f80u, L = odd ? 0x389eu : 0u; // sqrt(1/2) or 1 as bf16 hi, lo
+    const bool c0 = (e & 3) == 2, s0 = (e & 3) == 0;             // the entries that are zero
+    const unsigned cn = (e + 2) & 4 ? 0x8000u : 0u, sn = ((e & 4) != 0) != INV ? 0x8000u : 0u;
+    const unsigned ch = c0 ? 0u : H ^ cn, cl = c0 || !L ? 0u : L ^ cn;
+    const unsigned sh = s0 ? 0u : H ^ sn, sl = s0 || !L ? 0u : L ^ sn;
+    const bool p = g & 1;
+    const unsigned h = p ? (sh ^ 0x8000u) | ch << 16 : ch | sh << 16;
+    const unsigned l = p ? (sl ^ 0x8000u) | cl << 16 : cl | sl << 16;
+    const unsigned mt = t & 1 ? 0x80008000u : 0u, mr = g & 2 ? 0x80008000u : 0u;
+    hi[0] = h, hi[1] = h ^ mt, hi[2] = h ^ mr, hi[3] = h ^ mt ^ mr;
+    lo[0] = l, lo[1] = l ^ mt, lo[2] = l ^ mr, lo[3] = l ^ mt ^ mr;
 }
 
-__device__ __forceinline__ unsigned bf2(float lo_elem, float hi_elem)
+// (v.x, v.y) as packed bf16 hi and lo parts, x in the lower half
+__device__ __forceinline__ void split_bf16x2(float2 v, unsigned &hi, unsigned &lo)
 {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo_elem, hi_elem); // .x = first (lower 16 bits)
-    return *reinterpret_cast<unsigned *>(&v);
-}
-
-__device__ __forceinline__ void split_bf16(float v, float &hi, float &lo)
-{
-    hi = __bfloat162float(__float2bfloat16_rn(v));
-    lo = v - hi;
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+    hi = *reinterpret_cast<const unsigned *>(&h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(v.x - __uint_as_float(hi << 16), v.y - __uint_as_float(hi & 0xffff0000u));
+    lo = *reinterpret_cast<const unsigned *>(&l);
 }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1)
@@ -429,45 +442,28 @@ __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 
                                           const float2 *__restrict__ tw)
 {
     constexpr int R = 8, NB = NF / R, TOT = NB * C, GROUPS = TOT / 8;
-    static_assert(C == 16 && (NT / 32) % 2 == 0, "a group: half a row of butterflies; a warp keeps its half");
+    static_assert(C == 16 && (NT / 32) % 2 == 0 && GROUPS % (NT / 32) == 0, "a group: half a row of butterflies; a warp keeps its half");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3, c0 = (warp & 1) * 8;
-    // A fragments of F, split into hi and lo
     unsigned ahi[4], alo[4];
-    {
-        const int mm[4] = {g, g + 8, g, g + 8};
-        const int kk[4] = {2 * t, 2 * t, 2 * t + 8, 2 * t + 8};
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            float h0, l0, h1, l1;
-            split_bf16(dft8_entry(mm[i], kk[i], INV), h0, l0);
-            split_bf16(dft8_entry(mm[i], kk[i] + 1, INV), h1, l1);
-            ahi[i] = bf2(h0, h1);
-            alo[i] = bf2(l0, l1);
-        }
-    }
+    dft8_words<INV>(g, t, ahi, alo);
     float *outf = reinterpret_cast<float *>(out);
-    for (int grp = warp; grp < GROUPS; grp += NT / 32) {
+#pragma unroll 2
+    for (int i = 0; i < GROUPS / (NT / 32); i++) {
+        const int grp = warp + i * (NT / 32);
         // inputs r = t and r = t + 4 of butterfly (j, c)
         const int c = c0 + g, j = grp >> 1, k = j % NS;
         float2 x0 = in[(j + t * NB) * C + In::at(j + t * NB, c)];
         float2 x1 = in[(j + (t + 4) * NB) * C + In::at(j + (t + 4) * NB, c)];
-        if (NS > 1) {
-            if (t > 0) {
-                float2 w = tw[t * k * (NF / (NS * R))];
-                if (INV) w.y = -w.y;
-                x0 = cmul(x0, w);
-            }
-            float2 w = tw[(t + 4) * k * (NF / (NS * R))];
-            if (INV) w.y = -w.y;
-            x1 = cmul(x1, w);
+        if (NS > 1) { // (no branch for t = 0: its twiddle is 1)
+            float2 w0 = tw[t * k * (NF / (NS * R))], w1 = tw[(t + 4) * k * (NF / (NS * R))];
+            if (INV) w0.y = -w0.y, w1.y = -w1.y;
+            x0 = cmul(x0, w0);
+            x1 = cmul(x1, w1);
         }
-        float h0, l0, h1, l1, h2, l2, h3, l3;
-        split_bf16(x0.x, h0, l0);
-        split_bf16(x0.y, h1, l1);
-        split_bf16(x1.x, h2, l2);
-        split_bf16(x1.y, h3, l3);
-        const unsigned bh0 = bf2(h0, h1), bh1 = bf2(h2, h3), bl0 = bf2(l0, l1), bl1 = bf2(l2, l3);
+        unsigned bh0, bl0, bh1, bl1;
+        split_bf16x2(x0, bh0, bl0);
+        split_bf16x2(x1, bh1, bl1);
         float d[4] = {0.f, 0.f, 0.f, 0.f};
         mma_bf16(d, ahi, bh0, bh1);
         mma_bf16(d, ahi, bl0, bl1);
@@ -501,29 +497,49 @@ struct SplitTiles {
     using T1 = Swz<R::r1 == 8 ? NB : 0, R::r0 == 8 ? 1 : 0>;
     using T2 = Swz<R::r2 == 8 ? NB : 0, R::r1 == 8 ? R::r0 : 0>;
     using T3 = Swz<0, R::r2 == 8 ? R::r0 * R::r1 : 0>;
+    using Result = std::conditional_t<(R::r2 > 1), T3, T2>;
 };
 
-// Split-precision transform of a tile whose inputs were scattered into s0 by
-// FirstInputs::scatter in the order SplitTiles::Input; then
+// Split-precision transform of C interleaved lines whose inputs, in registers,
+// sp_first has left in s1 as the outputs of an FP32 first stage (radix 3 or 4),
+// or in s0 for a tensor-core one (radix 8).  sp_stages: the stages; returns the
+// tile that holds the result, column order SplitTiles::Result, once the caller
+// has added a barrier.  sp_all: the same, then
 // sink(it, r, c, pos, value) in the thread mapping of rr_last for radix
-// schedule S.  All threads call it; the caller adds a barrier before s0/s1 are
-// written again.
-template <int NF, bool INV, int C, int NT, int S, class Sink>
-__device__ __forceinline__ void sp_all(float2 *s0, float2 *s1, const float2 *tw, Sink sink)
+// schedule S.  All threads call them; the caller adds a barrier after sp_first
+// and before s0/s1 are written again.
+template <int NF, int C, int NT, int S>
+__device__ __forceinline__ void sp_first(const FirstInputs<NF, Radix<NF, S>::r0, C, NT> &in, float2 *s0, float2 *s1)
+{
+    using ST = SplitTiles<NF, S>;
+    if constexpr (Radix<NF, S>::r0 == 8) in.template scatter<typename ST::Input>(s0);
+    else rr_first<NF, Radix<NF, S>::r0, false, C, NT, typename ST::T1>(in, s1);
+}
+
+template <int NF, bool INV, int C, int NT, int S>
+__device__ __forceinline__ float2 *sp_stages(float2 *s0, float2 *s1, const float2 *tw)
 {
     using R = Radix<NF, S>;
     using ST = SplitTiles<NF, S>;
-    sp_stage<NF, R::r0, 1, INV, C, NT, typename ST::Input, typename ST::T1>(s0, s1, tw);
-    __syncthreads();
-    sp_stage<NF, R::r1, R::r0, INV, C, NT, typename ST::T1, typename ST::T2>(s1, s0, tw);
-    __syncthreads();
-    const float2 *fin = s0;
-    if constexpr (R::r2 > 1) {
-        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT, typename ST::T2, typename ST::T3>(s0, s1, tw);
+    if constexpr (R::r0 == 8) {
+        sp_stage<NF, R::r0, 1, INV, C, NT, typename ST::Input, typename ST::T1>(s0, s1, tw);
         __syncthreads();
-        fin = s1;
     }
-    using Fin = std::conditional_t<(R::r2 > 1), typename ST::T3, typename ST::T2>;
+    sp_stage<NF, R::r1, R::r0, INV, C, NT, typename ST::T1, typename ST::T2>(s1, s0, tw);
+    if constexpr (R::r2 > 1) {
+        __syncthreads();
+        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT, typename ST::T2, typename ST::T3>(s0, s1, tw);
+        return s1;
+    }
+    return s0;
+}
+
+template <int NF, bool INV, int C, int NT, int S, class Sink>
+__device__ __forceinline__ void sp_all(float2 *s0, float2 *s1, const float2 *tw, Sink sink)
+{
+    using Fin = typename SplitTiles<NF, S>::Result;
+    const float2 *fin = sp_stages<NF, INV, C, NT, S>(s0, s1, tw);
+    __syncthreads();
     constexpr int RL = LastStage<NF, S>::R, NSL = LastStage<NF, S>::NS, TOT = NSL * C, IT = (TOT + NT - 1) / NT;
 #pragma unroll
     for (int it = 0; it < IT; it++) {

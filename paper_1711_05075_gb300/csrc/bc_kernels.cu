@@ -512,8 +512,10 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
     extern __shared__ float4 sm4[];
     float2 *tw = reinterpret_cast<float2 *>(sm4);
     float2 *S0 = tw + NF, *S1 = S0 + NF * CL;
-    float2 *OUT = three ? S0 : S1; // tile the last stage writes (not the one it reads)
-    float2 *STG = three ? S1 : S0; // staging for the output rows
+    // tile the last stage writes (FP32: not the one it reads; split: the result's own)
+    float2 *OUT = three != SP ? S0 : S1;
+    float2 *STG = three != SP ? S1 : S0; // staging for the output rows
+    using Cols = std::conditional_t<SP, typename SplitTiles<NF, S>::Result, Natural>; // order of OUT's columns
     load_twiddles<NF>(tw, tb.tw_n);
     pdl_signal();
     pdl_wait(); // earlier passes' outputs are read from here on
@@ -542,7 +544,7 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
         for (; it < items; it += gridDim.x) {
             const int l = it / (b0 * nyb), rem = it - l * (b0 * nyb);
             const int ix = rem / nyb, iy0 = (rem - ix * nyb) << 5;
-            if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
+            if constexpr (SP) sp_first<NF, CL, NT, S>(in, S0, S1);
             else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
             __syncthreads(); // every thread has consumed its loads of this item
             {
@@ -551,17 +553,17 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                 for (int e = threadIdx.x; e < bz * 8; e += NT) run[e] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
             if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
-            auto sink = [&](int, int, int c, int pos, float2 v) { OUT[pos * CL + c] = v; };
-            if constexpr (SP) sp_all<NF, false, CL, NT, S>(S0, S1, tw, sink);
-            else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
+            if constexpr (SP) sp_stages<NF, false, CL, NT, S>(S0, S1, tw);
+            else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, [&](int, int, int c, int pos, float2 v) { OUT[pos * CL + c] = v; });
             __syncthreads();
             // unpack into a staging area [row][k] (row stride H + 1), then write
             // each 8H-byte row of z1 with consecutive threads on consecutive k
             for (int e = threadIdx.x; e < 32 * H; e += NT) {
                 const int r = e & 31, kk = e >> 5;
                 const int qq = r >> 1;
-                const float2 zk = OUT[kk * CL + qq];
-                const float2 zn = OUT[(kk == 0 ? 0 : NF - kk) * CL + qq];
+                const int kn = kk == 0 ? 0 : NF - kk;
+                const float2 zk = OUT[kk * CL + Cols::at(kk, qq)];
+                const float2 zn = OUT[kn * CL + Cols::at(kn, qq)];
                 STG[r * (H + 1) + kk] = (r & 1) ? make_float2(0.5f * (zk.y + zn.y), -0.5f * (zk.x - zn.x))
                                                 : make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
             }
@@ -676,7 +678,7 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             if (it < items) in.load(src(it));
             for (; it < items; it += gridDim.x) {
                 const int lx = it / nch, ch = it - lx * nch;
-                if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
+                if constexpr (SP) sp_first<NF, CL, NT, S>(in, S0, S1);
                 else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
                 __syncthreads();
                 if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));

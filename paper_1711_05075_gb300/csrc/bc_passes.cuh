@@ -91,7 +91,7 @@ __device__ __forceinline__ void spectrum_x(float2 (&F)[XModes<NF, S, NT>::IT][XM
             ts_base = l;
             build_xweights<NI, NT>(Ts, tb, l, min(G, L - l), jy, ch);
         }
-        if constexpr (SP) in.template scatter<typename SplitTiles<NF, S>::Input>(S0);
+        if constexpr (SP) sp_first<NF, CL, NT, S>(in, S0, S1);
         else rr_first<NF, Radix<NF, S>::r0, false, CL, NT>(in, S0);
         __syncthreads();
         if (l + 1 < L) in.load(src(l + 1));
