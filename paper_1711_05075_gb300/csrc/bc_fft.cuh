@@ -396,7 +396,7 @@ __device__ __forceinline__ void rr_rest(float2 *s0, float2 *s1, const float2 *tw
 // built from one entry, each complex value is split with two conversions, no lane
 // branches, two groups are in flight, a FP32 first stage runs on the registers
 // that hold its inputs, and the z pass unpacks straight from the result tile.
-// Split correlation at N = 128, L = 4, 20,000 + 20,000 balls: 527 us -> 283.
+// Split correlation at N = 128, L = 4, 20,000 + 20,000 balls: 527 us -> 273.
 //
 // The lane's words of F as a pair (hi, lo), of which the entry (r', r) = (g / 2,
 // t) is computed: 4 more on r' or on r turns the angle by pi times t or r', so the
@@ -437,7 +437,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <int NF, int NS, bool INV, int C, int NT, class In, class Out>
+template <int NF, int NS, bool INV, int C, int NT, int U, class In, class Out>
 __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 *__restrict__ out,
                                           const float2 *__restrict__ tw)
 {
@@ -448,7 +448,7 @@ __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 
     unsigned ahi[4], alo[4];
     dft8_words<INV>(g, t, ahi, alo);
     float *outf = reinterpret_cast<float *>(out);
-#pragma unroll 2
+#pragma unroll U
     for (int i = 0; i < GROUPS / (NT / 32); i++) {
         const int grp = warp + i * (NT / 32);
         // inputs r = t and r = t + 4 of butterfly (j, c)
@@ -480,10 +480,10 @@ __device__ __forceinline__ void tc_stage8(const float2 *__restrict__ in, float2 
 }
 
 // A stage of the split-precision schedule: tensor-core DFT for radix 8, FP32 otherwise.
-template <int NF, int R, int NS, bool INV, int C, int NT, class In, class Out>
+template <int NF, int R, int NS, bool INV, int C, int NT, int U, class In, class Out>
 __device__ __forceinline__ void sp_stage(const float2 *in, float2 *out, const float2 *tw)
 {
-    if constexpr (R == 8) tc_stage8<NF, NS, INV, C, NT, In, Out>(in, out, tw);
+    if constexpr (R == 8) tc_stage8<NF, NS, INV, C, NT, U, In, Out>(in, out, tw);
     else il_stage<NF, R, NS, INV, C, NT, In, Out>(in, out, tw);
 }
 
@@ -499,6 +499,12 @@ struct SplitTiles {
     using T3 = Swz<0, R::r2 == 8 ? R::r0 * R::r1 : 0>;
     using Result = std::conditional_t<(R::r2 > 1), T3, T2>;
 };
+
+// Groups that a warp has in flight in a tensor-core stage: all eight at 256 points,
+// where their addresses and twiddles become constants of the loop (a split
+// correlation at N = 128: 283 us with two, 273 with all in the z and y passes);
+// elsewhere, and in the x pass, all of them spill.
+__host__ __device__ constexpr int split_unroll(int NF) { return NF == 256 ? 8 : 2; }
 
 // Split-precision transform of C interleaved lines whose inputs, in registers,
 // sp_first has left in s1 as the outputs of an FP32 first stage (radix 3 or 4),
@@ -516,29 +522,29 @@ __device__ __forceinline__ void sp_first(const FirstInputs<NF, Radix<NF, S>::r0,
     else rr_first<NF, Radix<NF, S>::r0, false, C, NT, typename ST::T1>(in, s1);
 }
 
-template <int NF, bool INV, int C, int NT, int S>
+template <int NF, bool INV, int C, int NT, int S, int U = split_unroll(NF)>
 __device__ __forceinline__ float2 *sp_stages(float2 *s0, float2 *s1, const float2 *tw)
 {
     using R = Radix<NF, S>;
     using ST = SplitTiles<NF, S>;
     if constexpr (R::r0 == 8) {
-        sp_stage<NF, R::r0, 1, INV, C, NT, typename ST::Input, typename ST::T1>(s0, s1, tw);
+        sp_stage<NF, R::r0, 1, INV, C, NT, U, typename ST::Input, typename ST::T1>(s0, s1, tw);
         __syncthreads();
     }
-    sp_stage<NF, R::r1, R::r0, INV, C, NT, typename ST::T1, typename ST::T2>(s1, s0, tw);
+    sp_stage<NF, R::r1, R::r0, INV, C, NT, U, typename ST::T1, typename ST::T2>(s1, s0, tw);
     if constexpr (R::r2 > 1) {
         __syncthreads();
-        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT, typename ST::T2, typename ST::T3>(s0, s1, tw);
+        sp_stage<NF, R::r2, R::r0 * R::r1, INV, C, NT, U, typename ST::T2, typename ST::T3>(s0, s1, tw);
         return s1;
     }
     return s0;
 }
 
-template <int NF, bool INV, int C, int NT, int S, class Sink>
+template <int NF, bool INV, int C, int NT, int S, int U = split_unroll(NF), class Sink>
 __device__ __forceinline__ void sp_all(float2 *s0, float2 *s1, const float2 *tw, Sink sink)
 {
     using Fin = typename SplitTiles<NF, S>::Result;
-    const float2 *fin = sp_stages<NF, INV, C, NT, S>(s0, s1, tw);
+    const float2 *fin = sp_stages<NF, INV, C, NT, S, U>(s0, s1, tw);
     __syncthreads();
     constexpr int RL = LastStage<NF, S>::R, NSL = LastStage<NF, S>::NS, TOT = NSL * C, IT = (TOT + NT - 1) / NT;
 #pragma unroll
