@@ -364,6 +364,15 @@ struct LastStage {
     static constexpr int NS = NF / R;
 };
 
+// Outputs of the last stage that a pass keeps: modes [-NF/4, NF/4), the first and
+// last quarter of r.  Known when compiled, so the others are not computed.
+template <int NF, int S>
+__device__ __forceinline__ constexpr bool kept_out(int r)
+{
+    static_assert(LastStage<NF, S>::R % 4 == 0, "last stage");
+    return r < LastStage<NF, S>::R / 4 || r >= LastStage<NF, S>::R / 4 * 3;
+}
+
 // The middle (three-stage schedules) and last stages after rr_first has
 // written tile s0; s1 is scratch for three-stage schedules.  All threads call
 // it; the caller adds a barrier before s0/s1 are written again.

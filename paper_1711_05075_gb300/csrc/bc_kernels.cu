@@ -554,7 +554,9 @@ k_fft_z(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
             }
             if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
             if constexpr (SP) sp_stages<NF, false, CL, NT, S>(S0, S1, tw);
-            else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, [&](int, int, int c, int pos, float2 v) { OUT[pos * CL + c] = v; });
+            else rr_rest<NF, false, CL, NT, S>(S0, S1, tw, [&](int, int r, int c, int pos, float2 v) {
+                if (kept_out<NF, S>(r)) OUT[pos * CL + c] = v;
+            });
             __syncthreads();
             // unpack into a staging area [row][k] (row stride H + 1), then write
             // each 8H-byte row of z1 with consecutive threads on consecutive k
@@ -645,11 +647,9 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                 __syncthreads();
                 const int lx = it / nch, ch = it - lx * nch;
                 float2 *Y = y1 + d.y1_off + (long long)lx * N * H + ch * CL;
-                auto sink = [&](int, int, int c, int pos, float2 v) {
-                    int jy;
-                    if (pos < N / 2) jy = pos;
-                    else if (pos >= NF - N / 2) jy = pos - NF + N;
-                    else return;
+                auto sink = [&](int, int r, int c, int pos, float2 v) {
+                    if (!kept_out<NF, S>(r)) return;
+                    const int jy = pos < N / 2 ? pos : pos - NF + N;
                     Y[(long long)jy * H + c] = jy == N / 2 ? make_float2(0.f, 0.f) : v;
                 };
                 rr_rest<NF, false, CL, NT, S>(S0, S1, tw, sink);
@@ -683,11 +683,9 @@ k_fft_y(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, con
                 __syncthreads();
                 if (it + (int)gridDim.x < items) in.load(src(it + gridDim.x));
                 float2 *Y = y1 + d.y1_off + (long long)lx * N * H + ch * CL;
-                auto sink = [&](int, int, int c, int pos, float2 v) {
-                    int jy;
-                    if (pos < N / 2) jy = pos;
-                    else if (pos >= NF - N / 2) jy = pos - NF + N;
-                    else return;
+                auto sink = [&](int, int r, int c, int pos, float2 v) {
+                    if (!kept_out<NF, S>(r)) return;
+                    const int jy = pos < N / 2 ? pos : pos - NF + N;
                     Y[(long long)jy * H + c] = jy == N / 2 ? make_float2(0.f, 0.f) : v;
                 };
                 if constexpr (SP) sp_all<NF, false, CL, NT, S>(S0, S1, tw, sink);
