@@ -56,7 +56,7 @@ NCU_TRAFFIC = {
 }
 
 
-KERNEL_SOURCES = ("bc_kernels.cu", "bc_back.cu", "bc_binned.cu", "bc_query.cu", "bc_zumma.cu", "bc_fft.cuh",
+KERNEL_SOURCES = ("bc_front.cu", "bc_line.cu", "bc_wfft.cuh", "bc_kernels.cu", "bc_back.cu", "bc_binned.cu", "bc_query.cu", "bc_zumma.cu", "bc_fft.cuh",
                   "bc_device.cuh", "bc_passes.cuh", "bc_umma.cuh", "bc_internal.h")
 
 
@@ -393,11 +393,13 @@ def run_ours(args, rank, world, local_rank):
     dom_ms = dom["ms"] / calls
     achieved = dom["bytes"] / (dom_ms * 1e-3) / 1e9 if dom_ms > 0 else 0.0
     binned = tuning["spread"] == 1
-    kname = {"prepare": "k_prepare", "spread": "k_bin" if binned else "k_spread",
+    # shapes inside one period: z and y in one launch, counted under fft_y
+    line = not binned and next(x for x in stages if x["name"] == "fft_z")["bytes"] == 0
+    kname = {"prepare": "k_prepare", "spread": "k_bin" if binned else ("k_spread_rp" if line else "k_spread"),
              "fft_z": "k_fft_z_binned" if binned else ("k_fft_z_umma" if tuning.get("z_transform") else "k_fft_z"),
-             "fft_y": "k_fft_y",
-             "fft_x": "k_back" if tuning.get("persistent") else "k_fft_x", "ifft_y": "k_ifft_y",
-             "ifft_z": "k_ifft_z"}[dom["name"]]
+             "fft_y": "k_zy" if line else "k_fft_y",
+             "fft_x": "k_back" if tuning.get("persistent") else ("k_xw" if line else "k_fft_x"), "ifft_y": "k_ifft_y",
+             "ifft_z": "k_iyz" if line else "k_ifft_z"}[dom["name"]]
     tr = NCU_TRAFFIC.get(kname)
     traffic = tr["bytes"] if tr and tr.get("kernel_hash") == kernel_source_hash() else None
     stage_share = {s["name"]: round(s["ms"] / max(sum(x["ms"] for x in stages), 1e-12), 4) for s in stages}

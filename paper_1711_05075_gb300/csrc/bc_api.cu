@@ -623,7 +623,7 @@ bc_status bc_sync(bc_ctx_t c)
         CK(cudaMemset(c->err_dev, 0, sizeof(int)));
         if (herr & 4) return fail(BC_ERR_ARG, "a device-resident rotation had zero norm");
         if (herr & 8)
-            return fail(BC_ERR_TIMEOUT, "the tensor-core z transform stalled (a bounded wait expired); results are incomplete");
+            return fail(BC_ERR_TIMEOUT, "a transform pass stalled (a bounded wait expired); results are incomplete");
         if (herr & 16)
             return fail(BC_ERR_TIMEOUT, "a dependency wait of the persistent launch expired; results are incomplete");
         if (herr & 32)

@@ -24,6 +24,10 @@
 //   k_ifft_z    complex-to-real inverse along z (two rows per complex transform)
 //               giving g on the N^3 translation grid.
 //
+// Shapes that fit inside one period (N <= 128, FP32, default tuning) take a
+// shorter sequence after k_prepare: k_spread_rp and k_zy (bc_front.cu), k_xw and
+// k_iyz (bc_line.cu).
+//
 // The transform passes work on shared-memory tiles of 16 interleaved lines
 // (bc_fft.cuh) loaded and stored with 16-byte accesses.
 //

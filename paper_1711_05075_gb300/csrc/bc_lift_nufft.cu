@@ -37,6 +37,8 @@
 // half-period shift multiplies each spectrum by (-1)^(m_x + m_y + m_z + m_r),
 // which cancels in the product of the two spectra.  Box element i of an axis
 // sits at line position (lo + i) mod n; positions outside the box are zero.
+// Boxes narrower than the period on every axis take the passes of bc_lift_line.cu
+// after k_l4_box; the others these.
 // Transforms: the library's shared-memory Stockham FFT (bc_fft.cuh) on tiles of
 // 16 interleaved lines.  The grid and the z planes share the workspace with
 // the y and x planes (each pass's output fits in the space its input left).

@@ -49,6 +49,10 @@ cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float 
 // exchange.  With pr.a < 0 the spectrum of A comes from fa (layout
 // [m_z][j_y][j_x]); with pr.b < 0 it is written there and nothing else happens.
 // Output h[k_x][m_z][j_y].  Every wait is bounded (bit 8 of the error word).
+// Bound by instructions and latency (issue 57%, 128 registers).  20,000 + 20,000
+// balls, N = 128, L = 4: 37.3 us (k_fft_x 38.7 us); the walk's state in every thread's
+// registers instead of shared memory 44.5 us.  Items of 8 lines, not 16: the same time
+// at that size, more items for small grids.
 constexpr int XW_STAGES = 3, XW_ERR = 8, XW_RW = 6;
 
 template <int NF, int LW>
@@ -297,6 +301,7 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
 // one 16-byte load; finished rows leave through the warp's exchange tile so that
 // each store covers whole rows.  With `keys` the block folds its largest value
 // (lowest index on ties) into the pair's peak key.
+// N = 128: 9.5 us, against 6.1 + 10.4 us of k_ifft_y and k_ifft_z.
 template <int NI>
 struct IYZ {
     static constexpr int R0 = NI / 8, H = NI / 2, LW = 4;   // lines of a warp per step
@@ -429,10 +434,13 @@ static cudaError_t xw_t(const Geometry &g, const Tables &t, const InstDesc *inst
                         const PairDesc *pairs, int npairs, const float2 *y1, const float2 *fa_cache, float2 *fa_out,
                         float2 *h, int cap, int *err, int nsm, cudaStream_t s)
 {
-    // where every item is resident at once at four warps each, idle lanes cost nothing
-    // and the shorter steps of two lines per warp shorten the pass
+    // where every item has an SM to itself, idle lanes cost nothing and the shorter steps
+    // of two lines per warp shorten the pass.  Up to four items per SM (256 or 448
+    // items) the fewer warps are the faster ones: a score at N = 64 with 5 rotations 69.9
+    // us with two lines per warp, 67.7 with four; 7 rotations at N = 32 32.5 and 31.0;
+    // only a single pair at N = 64 (256 items) gains from two: 38.7 against 39.2
     if constexpr (LW > 2)
-        if ((long long)npairs * WF<NF>::H * (WF<NF>::N / XL) <= 4LL * nsm)
+        if ((long long)npairs * WF<NF>::H * (WF<NF>::N / XL) <= nsm)
             return xw_t<NF, 2>(g, t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, cap, err, nsm, s);
     using X = XW<NF, LW>;
     const size_t smem = X::smem(cap);

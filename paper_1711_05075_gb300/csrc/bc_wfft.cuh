@@ -1,5 +1,6 @@
 // Warp-synchronous 1D FFTs in two radix stages (FP32), for the passes that keep
-// every line of a transform inside one warp (bc_front.cu, bc_xw.cu, bc_iyz.cu).
+// every line of a transform inside one warp (bc_front.cu, bc_line.cu,
+// bc_lift_line.cu).
 //
 // Forward, length NF = R0 . 16 (64 = 4.16, 128 = 8.16, 192 = 12.16, 256 =
 // 16.16): 16 first-stage butterflies of radix R0 on the inputs j + 16 r, then
