@@ -102,7 +102,7 @@ constexpr int ZY_WARPS = 8;
 template <int NF, int LW>
 __global__ void __launch_bounds__(ZY_WARPS * 32, 2)
 k_zy(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const InstPlan *__restrict__ plan,
-     float *grid, float2 *y1, int PS)
+     float *grid, float2 *y1, int PS, bool clear)
 {
     using F = WF<NF, LW>;
     constexpr int R0 = F::R0, H = F::H, N = F::N;
@@ -155,10 +155,10 @@ k_zy(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const 
                 __syncwarp();
             }
             __syncthreads();
-            // the plane is read: clear it (one contiguous run; a store beside each load
+            // the plane is read: clear it, if asked (one contiguous run; a store beside each load
             // of the same cell took 148 us instead of 47)
             float4 *G4 = reinterpret_cast<float4 *>(G2);
-            for (int e = threadIdx.x; e < np * bz / 2; e += ZY_WARPS * 32) G4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int e = threadIdx.x; clear && e < np * bz / 2; e += ZY_WARPS * 32) G4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
             const int l = it / b0, ix = it - l * b0;
             float2 *Y = y1 + d.y1_off + ((long long)l * H * (N / XL) * b0 + ix) * XL;
             for (int k0 = warp * LW; k0 < H; k0 += ZY_WARPS * LW) {
@@ -235,29 +235,29 @@ cudaError_t launch_spread_rp(const Geometry &g, const Tables &t, const InstDesc 
 
 template <int NF, int LW = wf_full(NF)>
 static cudaError_t zy_t(const Geometry &g, const Tables &t, const InstDesc *inst, int ninst, const InstPlan *plan,
-                        float *grid, float2 *y1, int cap, int nsm, cudaStream_t s)
+                        float *grid, float2 *y1, int cap, int nsm, cudaStream_t s, bool clear)
 {
     // where every plane may be resident at once, idle lanes cost nothing and the shorter
     // steps of two lines per warp shorten the pass (128 + 128 balls at N = 32, whole
     // correlation: 22.4 us, with eight lines 23.5)
     if constexpr (LW > 2)
         if ((long long)ninst * g.L * cap <= 2LL * nsm)
-            return zy_t<NF, 2>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s);
+            return zy_t<NF, 2>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
     const size_t smem = zy_smem<NF, LW>(cap);
     cudaError_t e = set_smem(k_zy<NF, LW>, smem);
     if (e != cudaSuccess) return e;
     return launch_k(k_zy<NF, LW>, resident_blocks(k_zy<NF, LW>, smem, nsm, ZY_WARPS * 32), ZY_WARPS * 32, smem, s,
-                    g.pdl != 0, g, t, inst, ninst, plan, grid, y1, zy_ps(cap));
+                    g.pdl != 0, g, t, inst, ninst, plan, grid, y1, zy_ps(cap), clear);
 }
 
 cudaError_t launch_zy(const Geometry &g, const Tables &t, const InstDesc *inst, int ninst, const InstPlan *plan,
-                      float *grid, float2 *y1, int cap, int nsm, cudaStream_t s)
+                      float *grid, float2 *y1, int cap, int nsm, cudaStream_t s, bool clear)
 {
     switch (g.n) {
-    case 64: return zy_t<64>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s);
-    case 128: return zy_t<128>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s);
-    case 192: return zy_t<192>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s);
-    case 256: return zy_t<256>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s);
+    case 64: return zy_t<64>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
+    case 128: return zy_t<128>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
+    case 192: return zy_t<192>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
+    case 256: return zy_t<256>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
     default: return cudaErrorInvalidValue;
     }
 }

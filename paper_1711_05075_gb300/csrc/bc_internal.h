@@ -95,7 +95,7 @@ bool front_fits(const Geometry &g, int cap);
 cudaError_t launch_spread_rp(const Geometry &g, const Tables &t, const InstDesc *inst, int total_knots, const float4 *ku,
                              const InstPlan *plan, float *grid, cudaStream_t s);
 cudaError_t launch_zy(const Geometry &g, const Tables &t, const InstDesc *inst, int ninst, const InstPlan *plan,
-                      float *grid, float2 *y1, int cap, int nsm, cudaStream_t s);
+                      float *grid, float2 *y1, int cap, int nsm, cudaStream_t s, bool clear = true);
 size_t wl_floats(const Geometry &g);
 cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float *ballft, float *wl, cudaStream_t s);
 cudaError_t launch_xw(const Geometry &g, const Tables &t, const InstDesc *inst, const InstPlan *plan,

@@ -744,6 +744,14 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
         ppairs[s] = PairDesc{0, 0, (long long)(s * plane), (long long)s * N * N * N, 0};
     }
     *perr = 0;
+    const double qw = quat[0] * inv, qx = quat[1] * inv, qy = quat[2] * inv, qz = quat[3] * inv;
+    const double R[9] = {1 - 2 * (qy * qy + qz * qz), 2 * (qx * qy - qw * qz), 2 * (qx * qz + qw * qy),
+                         2 * (qx * qy + qw * qz), 1 - 2 * (qx * qx + qz * qz), 2 * (qy * qz - qw * qx),
+                         2 * (qx * qz - qw * qy), 2 * (qy * qz + qw * qx), 1 - 2 * (qx * qx + qy * qy)};
+    // the boxes go first: the host waits for them, the copies that follow need not be waited for
+    if (lf->contraction == 3 && (e = lift4_boxes(lf->t4, N, Nr, kA, nA, kB, nB, R, lf->period, lf->period_r, lf->nsm, st)) !=
+                                    cudaSuccess)
+        return lift_cuda(e, "bc_lift_correlate: support boxes");
     if ((e = cudaMemcpyAsync(dsl, psl, sizeof(float) * nslices, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(dpairs, ppairs, sizeof(PairDesc) * nslices, cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return lift_cuda(e, "bc_lift_correlate: descriptors");
@@ -752,10 +760,6 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
     bool line = false; // h is already inverse transformed along x (lift4_pair)
     if (lf->contraction == 3) {
         // both spectra by the 4D NUFFT, their r transforms fused with the collapse
-        const double qw = quat[0] * inv, qx = quat[1] * inv, qy = quat[2] * inv, qz = quat[3] * inv;
-        const double R[9] = {1 - 2 * (qy * qy + qz * qz), 2 * (qx * qy - qw * qz), 2 * (qx * qz + qw * qy),
-                             2 * (qx * qy + qw * qz), 1 - 2 * (qx * qx + qz * qz), 2 * (qy * qz - qw * qx),
-                             2 * (qx * qz - qw * qy), 2 * (qy * qz + qw * qx), 1 - 2 * (qx * qx + qy * qy)};
         if ((e = lift4_pair(lf->t4, N, Nr, kA, nA, kB, nB, R, lf->period, lf->period_r, lf->cone, dsl, nslices, scale, E,
                             h, &line, derr, lf->nsm, st)) != cudaSuccess)
             return lift_cuda(e, "bc_lift_correlate: 4D NUFFT");

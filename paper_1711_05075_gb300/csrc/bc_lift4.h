@@ -55,6 +55,9 @@ size_t lift4_ws_bytes(int N, int Nr);
 // lift4_ws_bytes(N, Nr) bytes.  Synchronises s once (to size the support boxes).
 // With *line set on return h is [s][k_x][m_z][j_y] instead, the inverse transform
 // along x done (what launch_iyz takes); *err gets bit 8 if a bounded wait expired.
+// lift4_boxes first: it enqueues the search for the two shapes' support boxes.
+cudaError_t lift4_boxes(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
+                        const double (&RB)[9], double period, double period_r, int nsm, cudaStream_t s);
 cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                        const double (&RB)[9], double period, double period_r, const float2 *cone, const float *slices,
                        int nslices, float scale, void *ws, float2 *h, bool *line, int *err, int nsm, cudaStream_t s);
@@ -63,10 +66,12 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
 size_t lift4_weight_bytes(int N, int Nr);
 cudaError_t lift4_build_weights(const Lift4Tables &t, int N, int Nr, const float2 *cone, cudaStream_t s);
 bool lift4_line_fits(int N, int Nr, int bA, int bB, int nslices);
-// x planes X1[m_z][j_y][i_r][j_x] of n knots; G: the box grid (cleared here), y1: scratch
+inline size_t lift4_cells(const Lift4Box &b) { return (size_t)b.b[3] * b.b[0] * b.b[1] * b.b[2]; }
+// x planes X1[m_z][j_y][i_r][j_x] of n knots; G: the box grid, whose first `clean` cells are
+// zero (with none, the passes leave the box's cells zero behind them; else they don't); y1: scratch
 cudaError_t lift4_line_spectrum(const Lift4Tables &t, int N, int Nr, const float4 *knots, int n, const Lift4Rot &rot,
                                 int mirror, double ip, double ipr, const Lift4Box &bx, const InstPlan *dplan,
-                                const InstDesc *dinst, float *G, float2 *y1, float2 *X1, int *err, int nsm, cudaStream_t s);
+                                const InstDesc *dinst, float *G, size_t clean, float2 *y1, float2 *X1, int *err, int nsm, cudaStream_t s);
 cudaError_t lift4_line_collapse(const Lift4Tables &t, int N, int Nr, const float2 *XA, const float2 *XB, const Lift4Box &ba,
                                 const Lift4Box &bb, const float *slices, int nslices, double period_r, float scale, float2 *h,
                                 int *err, int nsm, cudaStream_t s);

@@ -412,11 +412,11 @@ bool lift4_line_fits(int N, int Nr, int bA, int bB, int nslices)
 
 cudaError_t lift4_line_spectrum(const Lift4Tables &t, int N, int Nr, const float4 *knots, int n, const Lift4Rot &rot,
                                 int mirror, double ip, double ipr, const Lift4Box &bx, const InstPlan *dplan,
-                                const InstDesc *dinst, float *G, float2 *y1, float2 *X1, int *err, int nsm, cudaStream_t s)
+                                const InstDesc *dinst, float *G, size_t clean, float2 *y1, float2 *X1, int *err, int nsm, cudaStream_t s)
 {
-    const size_t cells = (size_t)bx.b[3] * bx.b[0] * bx.b[1] * bx.b[2];
+    const size_t cells = lift4_cells(bx);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(G, 0, sizeof(float) * cells, s)) != cudaSuccess) return e;
+    if (cells > clean && (e = cudaMemsetAsync(G + clean, 0, sizeof(float) * (cells - clean), s)) != cudaSuccess) return e;
     k_lx_spread<<<std::min((n + 7) / 8, 65535), 256, 0, s>>>(knots, n, rot, mirror, 2 * N, 2 * Nr, ip, ipr, bx, t.consts, G);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     Geometry g{};
@@ -425,7 +425,7 @@ cudaError_t lift4_line_spectrum(const Lift4Tables &t, int N, int Nr, const float
     g.L = bx.b[3];
     Tables tb{};
     tb.tw_n = t.tw_s;
-    if ((e = launch_zy(g, tb, dinst, 1, dplan, G, y1, bx.b[1], nsm, s)) != cudaSuccess) return e;
+    if ((e = launch_zy(g, tb, dinst, 1, dplan, G, y1, bx.b[1], nsm, s, clean == 0)) != cudaSuccess) return e;
     switch (N) {
     case 32: return lx_x<64>(y1, bx.b[0], bx.b[3], t.tw_s, X1, err, nsm, s);
     case 64: return lx_x<128>(y1, bx.b[0], bx.b[3], t.tw_s, X1, err, nsm, s);

@@ -58,10 +58,19 @@ using L4Rot = Lift4Rot;
 using L4Box = Lift4Box;
 
 // box[a] = min, box[4 + a] = min of the negative, over the knots, of the first
-// stencil cell ceil(u_a - W/2) (preset to large values).
-__global__ void k_l4_box(const float4 *__restrict__ knots, int n, L4Rot rot, int mirror, int ns, int nr, double inv_p,
-                         double inv_pr, int *box)
+// stencil cell ceil(u_a - W/2) (preset to large values).  Grid: (blocks over knots,
+// shape); shape 1 is mirrored in r.
+struct L4Shape {
+    const float4 *knots;
+    int n;
+    L4Rot rot;
+};
+__global__ void k_l4_box(L4Shape A, L4Shape B, int ns, int nr, double inv_p, double inv_pr, int *box)
 {
+    const int mirror = blockIdx.y, n = mirror ? B.n : A.n;
+    const float4 *knots = mirror ? B.knots : A.knots;
+    const L4Rot &rot = mirror ? B.rot : A.rot;
+    box += 8 * mirror;
     int lo[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX}, hi[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 c = knots[i];
@@ -402,6 +411,23 @@ static cudaError_t l4_rc_ns(const float2 *XA, const float2 *XB, int N, int loA, 
     return l4_rc<NF, 16>(XA, XB, N, loA, bA, loB, bB, t, cone, slices, nslices, period_r, scale, h, nsm, s);
 }
 
+cudaError_t lift4_boxes(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
+                        const double (&RB)[9], double period, double period_r, int nsm, cudaStream_t s)
+{
+    if (nA == 0 || nB == 0) return cudaSuccess;
+    L4Shape A{kA, nA, {}}, B{kB, nB, {}};
+    for (int k = 0; k < 9; k++) {
+        A.rot.R[k] = (k % 4 == 0) ? 1.0 : 0.0; // A unrotated
+        B.rot.R[k] = RB[k];
+    }
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(t.dbox, 0x7f, 16 * sizeof(int), s)) != cudaSuccess) return e;
+    const int blocks = std::min((std::max(nA, nB) + 255) / 256, 4 * nsm);
+    k_l4_box<<<dim3(blocks, 2), 256, 0, s>>>(A, B, 2 * N, 2 * Nr, 1.0 / period, 1.0 / period_r, t.dbox);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaMemcpyAsync(t.hbox, t.dbox, 16 * sizeof(int), cudaMemcpyDeviceToHost, s);
+}
+
 cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                        const double (&RB)[9], double period, double period_r, const float2 *cone, const float *slices,
                        int nslices, float scale, void *ws, float2 *h, bool *line, int *err, int nsm, cudaStream_t s)
@@ -417,16 +443,8 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
         ra.R[k] = (k % 4 == 0) ? 1.0 : 0.0; // A unrotated
         rb.R[k] = RB[k];
     }
-    // both support boxes, one read-back
     cudaError_t e;
-    if ((e = cudaMemsetAsync(t.dbox, 0x7f, 16 * sizeof(int), s)) != cudaSuccess) return e;
-    for (int k = 0; k < 2; k++) {
-        const int n = k ? nB : nA, blocks = std::min((n + 255) / 256, 4 * nsm);
-        k_l4_box<<<blocks, 256, 0, s>>>(k ? kB : kA, n, k ? rb : ra, k, ns, nr, ip, ipr, t.dbox + 8 * k);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if ((e = cudaMemcpyAsync(t.hbox, t.dbox, 16 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e; // lift4_boxes has the boxes read back
     L4Box bx[2], even[2]; // even: row pairs, 16-byte rows
     bool inside = true;
     for (int k = 0; k < 2; k++)
@@ -443,7 +461,8 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
     *line = inside && t.wts && lift4_line_fits(N, Nr, bx[0].b[3], bx[1].b[3], nslices);
     if (*line) {
         // spectra in turn over the same grid and y planes; A's x planes have their own
-        // place, B's take the grid's
+        // place, B's take the grid's, which only A's passes have to leave clear (B's 250 MB
+        // of zeroing and clearing at N = 128, N_r = 32 go)
         InstPlan *hp = (InstPlan *)(t.hbox + 16), *dp = (InstPlan *)(t.dbox + 16);
         const InstDesc *dd = (const InstDesc *)(dp + 2); // offsets zero
         static_assert(16 * sizeof(int) + 2 * sizeof(InstPlan) + 2 * sizeof(InstDesc) <= LIFT4_BOX_BYTES, "box words");
@@ -454,8 +473,9 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
             return e;
         float *G = (float *)ws;
         float2 *XB = (float2 *)ws;
-        if ((e = lift4_line_spectrum(t, N, Nr, kA, nA, ra, 0, ip, ipr, even[0], dp, dd, G, Z1, XA, err, nsm, s)) != cudaSuccess ||
-            (e = lift4_line_spectrum(t, N, Nr, kB, nB, rb, 1, ip, ipr, even[1], dp + 1, dd + 1, G, Z1, XB, err, nsm, s)) != cudaSuccess)
+        if ((e = lift4_line_spectrum(t, N, Nr, kA, nA, ra, 0, ip, ipr, even[0], dp, dd, G, 0, Z1, XA, err, nsm, s)) != cudaSuccess ||
+            (e = lift4_line_spectrum(t, N, Nr, kB, nB, rb, 1, ip, ipr, even[1], dp + 1, dd + 1, G, lift4_cells(even[0]), Z1, XB, err,
+                                     nsm, s)) != cudaSuccess)
             return e;
         return lift4_line_collapse(t, N, Nr, XA, XB, even[0], even[1], slices, nslices, period_r, scale, h, err, nsm, s);
     }
