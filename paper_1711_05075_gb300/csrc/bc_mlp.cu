@@ -597,20 +597,6 @@ __global__ void k_loss(const float *__restrict__ y, const float *__restrict__ t,
     if (threadIdx.x == 0) *loss = part[0] / (float)n;
 }
 
-// Adam with bias correction on every parameter
-__global__ void k_adam(float *p, float *m, float *v, const float *__restrict__ g, long long total, float lr, float b1,
-                       float b2, float eps, float c1, float c2)
-{
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const float gg = g[e];
-    const float mm = b1 * m[e] + (1.f - b1) * gg;
-    const float vv = b2 * v[e] + (1.f - b2) * gg * gg;
-    m[e] = mm;
-    v[e] = vv;
-    p[e] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
-}
-
 // x[r] = [q_r / |q_r| with w >= 0; fa; fb; zeros to KPAD]; err |= 4 on a zero quaternion
 // Row r: [q_r / |q_r| (w >= 0); fa; fb + r ldb] (ldb = 0: the same fb for every row).
 __global__ void k_features(const float *__restrict__ q, int n, const float *__restrict__ fa,
@@ -706,7 +692,7 @@ __global__ void k_axpby(float *y, const float *__restrict__ x, int n, float alph
 // Both hidden layers and the output of 128 rows in one block (hidden <= FW_MAXH):
 //   h1 = relu(W1 x + b1), h2 = relu(W2 h1 + b2), y = w3 . h2 + b3.
 // The weights come as BF16 blocks already in the tensor core's swizzled layout
-// (k_pack_weights, once per parameter change) by bulk copies: W1's three K blocks
+// (k_pack_weights, then kept by k_adam) by bulk copies: W1's three K blocks
 // of 64 and the first of W2 at the start, W2's other blocks into W1's place once
 // the first product is done.  The rows of X are rounded to BF16 by the threads; h1
 // goes from tensor memory through the bias and the ReLU straight into the second
@@ -718,12 +704,12 @@ constexpr int FW_MAXH = 256, FW_SLOTS = 4;
 int fw_hp(int H) { return (H + 63) & ~63; }
 int fw_smem(int H) { return 1024 + 4 * GU_A_BYTES + FW_SLOTS * H * 128 + 4 * (128 + 3 * FW_MAXH) + 128; }
 
-// W1p[3][H][64], W2p[hp / 64][H][64] and, when wanted, W2T (row h_in, column h_out) BF16, rows of 128
+// W1p[3][H][64], W2p[hp / 64][H][64] and W2T (row h_in, column h_out) BF16, rows of 128
 // bytes swizzled as st_chunk does, zero beyond K
 __global__ void k_pack_weights(const float *__restrict__ W1, const float *__restrict__ W2, int H, int hp, uint8_t *W1p,
                                uint8_t *W2p, uint8_t *W2T)
 {
-    const int n1 = 3 * H * 8, n2 = hp / 64 * H * 8, n3 = W2T ? n2 : 0;
+    const int n1 = 3 * H * 8, n2 = hp / 64 * H * 8, n3 = n2;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 + n2 + n3; e += gridDim.x * blockDim.x) {
         float x[8];
         if (e < n1 + n2) {
@@ -740,6 +726,39 @@ __global__ void k_pack_weights(const float *__restrict__ W1, const float *__rest
             for (int k = 0; k < 8; k++) x[k] = k0 + k < H ? W2[(long long)(k0 + k) * H + r] : 0.f;
             st_chunk(W2T + (size_t)kb * H * 128, r, j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
         }
+    }
+}
+
+// entry (r, k) of such blocks
+__device__ __forceinline__ void st_packed(uint8_t *blocks, int H, int r, int k, float x)
+{
+    *reinterpret_cast<__nv_bfloat16 *>(blocks + (size_t)(k >> 6) * H * 128 + r * 128 + ((((k >> 3) & 7) ^ (r & 7)) << 4) +
+                                       2 * (k & 7)) = __float2bfloat16_rn(x);
+}
+
+// Adam with bias correction on every parameter.  Where the fused passes are used it
+// writes W1 and W2 into their BF16 blocks too, so that these always hold the parameters,
+// also when launches are replayed from a graph.
+__global__ void k_adam(float *p, float *m, float *v, const float *__restrict__ g, long long total, float lr, float b1,
+                       float b2, float eps, float c1, float c2, int H, long long oW2, uint8_t *W1p, uint8_t *W2p, uint8_t *W2T)
+{
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const float gg = g[e];
+    const float mm = b1 * m[e] + (1.f - b1) * gg;
+    const float vv = b2 * v[e] + (1.f - b2) * gg * gg;
+    m[e] = mm;
+    v[e] = vv;
+    const float x = p[e] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+    p[e] = x;
+    if (!W1p) return;
+    if (e < (long long)H * KIN) { // W1 comes first
+        const int r = (int)e / KIN;
+        st_packed(W1p, H, r, (int)e - r * KIN, x);
+    } else if (e >= oW2 && e < oW2 + (long long)H * H) {
+        const int q = (int)(e - oW2), r = q / H, c = q - r * H;
+        st_packed(W2p, H, r, c, x);
+        st_packed(W2T, H, c, r, x);
     }
 }
 
@@ -1308,7 +1327,6 @@ struct bc_mlp_s {
     int xb_cap = 0;
     float *loss = nullptr;
     uint8_t *wp = nullptr;        // BF16 weights in the fused forward pass's layout (hidden <= FW_MAXH)
-    int packed = 0;               // which hold the current parameters: 1 W1 and W2, 2 W2 transposed too
     int rotated_moments = 0;      // the ligand features are the moments of the rotated ligand (bc_mlp_set_features)
 };
 
@@ -1370,30 +1388,52 @@ bc_status ensure_batch(bc_mlp_t net, int n)
     return BC_OK;
 }
 
-// The BF16 weight blocks of the fused passes, once per parameter change.
-bc_status pack_weights(bc_mlp_t net, int want, cudaStream_t s)
+// The BF16 weight blocks of the fused passes, in one buffer.
+struct Packed {
+    uint8_t *W1 = nullptr, *W2 = nullptr, *W2T = nullptr;
+    explicit Packed(bc_mlp_t net)
+    {
+        if (!net->wp) return;
+        const size_t H = net->H, hp = fw_hp(net->H);
+        W1 = net->wp;
+        W2 = W1 + 3 * H * 128;
+        W2T = W2 + hp / 64 * H * 128;
+    }
+};
+
+// All of them from the parameters.
+cudaError_t pack_weights(bc_mlp_t net, cudaStream_t s)
 {
-    if (net->packed >= want) return BC_OK;
-    const int H = net->H, hp = fw_hp(H);
-    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128, *W2T = W2p + (size_t)hp / 64 * H * 128;
-    const int items = (3 + (want > 1 ? 2 : 1) * hp / 64) * H * 8;
-    k_pack_weights<<<(items + 255) / 256, 256, 0, s>>>(net->p + net->off.W1, net->p + net->off.W2, H, hp, W1p, W2p,
-                                                       want > 1 ? W2T : nullptr);
-    MCK(cudaGetLastError());
-    net->packed = want;
-    return BC_OK;
+    if (!net->wp) return cudaSuccess;
+    const int H = net->H, hp = fw_hp(H), items = (3 + 2 * hp / 64) * H * 8;
+    const Packed w(net);
+    k_pack_weights<<<(items + 255) / 256, 256, 0, s>>>(net->p + net->off.W1, net->p + net->off.W2, H, hp, w.W1, w.W2, w.W2T);
+    return cudaGetLastError();
+}
+
+// One Adam step with the gradients in net->g.
+cudaError_t adam(bc_mlp_t net, float lr, cudaStream_t s)
+{
+    net->step++;
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
+    const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
+    const long long total = net->off.total;
+    const Packed w(net);
+    k_adam<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(net->p, net->m, net->v, net->g, total, lr, b1, b2, eps, c1, c2,
+                                                          net->H, net->off.W2, w.W1, w.W2, w.W2T);
+    return cudaGetLastError();
 }
 
 // The fused forward pass: y of n rows.
 bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, cudaStream_t s)
 {
-    if (bc_status st = pack_weights(net, 1, s)) return st;
     const int H = net->H, hp = fw_hp(H);
     const Offsets &o = net->off;
-    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128;
+    const Packed w(net);
     int tcols = 32; // two accumulators of H columns
     while (tcols < 2 * H) tcols <<= 1;
-    k_mlp_forward<<<(n + 127) / 128, GU_THREADS, fw_smem(H), s>>>(X, n, H, hp, tcols, W1p, W2p, net->p + o.b1, net->p + o.b2,
+    k_mlp_forward<<<(n + 127) / 128, GU_THREADS, fw_smem(H), s>>>(X, n, H, hp, tcols, w.W1, w.W2, net->p + o.b1, net->p + o.b2,
                                                                   net->p + o.w3, net->p + o.b3, y, ctx_err(net->ctx));
     MCK(cudaGetLastError());
     return BC_OK;
@@ -1402,11 +1442,10 @@ bc_status fused_forward(bc_mlp_t net, const float *X, int n, float *y, cudaStrea
 // The fused training pass: y, the gradients into g and the loss (may be null).
 bc_status fused_train(bc_mlp_t net, const float *X, const float *t, int n, float *g, float *loss, cudaStream_t s)
 {
-    if (bc_status st = pack_weights(net, 2, s)) return st;
     const int H = net->H, hp = fw_hp(H), blocks = (n + 127) / 128;
     const Offsets &o = net->off;
-    uint8_t *W1p = net->wp, *W2p = W1p + (size_t)3 * H * 128, *W2T = W2p + (size_t)hp / 64 * H * 128;
-    k_mlp_train<<<blocks, GU_THREADS, tr_smem(H), s>>>(X, t, n, H, hp, 512, W1p, W2p, W2T, net->p + o.b1, net->p + o.b2,
+    const Packed w(net);
+    k_mlp_train<<<blocks, GU_THREADS, tr_smem(H), s>>>(X, t, n, H, hp, 512, w.W1, w.W2, w.W2T, net->p + o.b1, net->p + o.b2,
                                                        net->p + o.w3, net->p + o.b3, net->y, net->part, ctx_err(net->ctx));
     MCK(cudaGetLastError());
     const long long total = (long long)H * H + 144LL * H + 2 * H + 2;
@@ -1727,7 +1766,6 @@ void bc::mlp_orphan(bc_mlp_s *net)
     net->p = net->m = net->v = net->g = net->h1 = net->h2 = net->y = net->gy = net->dh2 = net->dh1 = net->loss = nullptr;
     net->part = net->xb = net->tb = nullptr;
     net->wp = nullptr;
-    net->packed = 0;
     net->cap = net->ycap = net->xb_cap = 0;
     net->part_floats = 0;
     net->ctx = nullptr;
@@ -1770,7 +1808,7 @@ bc_status bc_mlp_create(bc_ctx_t ctx, int hidden, const float *init, bc_mlp_t *o
         }
         if ((e = cudaMemcpyAsync(net->p, init, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(net->m, 0, bytes, s)) != cudaSuccess || (e = cudaMemsetAsync(net->v, 0, bytes, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess) {
+            (e = pack_weights(net, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) {
             bc_mlp_destroy(net);
             return mcuda(e, "bc_mlp_create: upload");
         }
@@ -1860,15 +1898,7 @@ bc_status bc_mlp_train_step(bc_mlp_t net, const float *X, const float *t, int n,
     try {
         if (!net || !X || !t || n < 1 || !(lr > 0.f)) return mfail(BC_ERR_ARG, "bc_mlp_train_step: bad arguments");
         if (bc_status st = bc_mlp_grads(net, X, t, n, nullptr, loss)) return st;
-        net->step++;
-        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
-        const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
-        const long long total = net->off.total;
-        k_adam<<<(unsigned)((total + 255) / 256), 256, 0, ctx_stream(net->ctx)>>>(net->p, net->m, net->v, net->g, total, lr,
-                                                                                 b1, b2, eps, c1, c2);
-        MCK(cudaGetLastError());
-        net->packed = 0;
+        MCK(adam(net, lr, ctx_stream(net->ctx)));
         return BC_OK;
     } catch (...) {
         return mfail(BC_ERR_INTERNAL, "bc_mlp_train_step: unexpected exception");
@@ -1918,8 +1948,6 @@ bc_status bc_mlp_train(bc_mlp_t net, const float *X, const float *t, int n, int 
             MCK(cudaMalloc(&net->tb, sizeof(float) * (size_t)batch));
             net->xb_cap = batch;
         }
-        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        const long long total = net->off.total;
         const int steps = n / batch;
         const bool x16 = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
         for (int e = 0; e < epochs; e++) {
@@ -1939,13 +1967,7 @@ bc_status bc_mlp_train(bc_mlp_t net, const float *X, const float *t, int n, int 
                 }
                 MCK(cudaGetLastError());
                 if (bc_status r = forward_backward(net, net->xb, net->tb, batch, nullptr, nullptr, s)) return r;
-                net->step++;
-                const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
-                const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
-                k_adam<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(net->p, net->m, net->v, net->g, total, lr_e, b1,
-                                                                      b2, eps, c1, c2);
-                MCK(cudaGetLastError());
-                net->packed = 0;
+                MCK(adam(net, lr_e, s));
             }
         }
         if (loss) {
@@ -1970,7 +1992,7 @@ bc_status bc_mlp_state(bc_mlp_t net, float *params, float *m, float *v, long lon
         if (!host[i]) continue;
         if (get) MCK(cudaMemcpyAsync(host[i], dev[i], bytes, cudaMemcpyDeviceToHost, s));
         else MCK(cudaMemcpyAsync(dev[i], host[i], bytes, cudaMemcpyHostToDevice, s));
-        if (!get && i == 0) net->packed = 0;
+        if (!get && i == 0) MCK(pack_weights(net, s));
     }
     MCK(cudaStreamSynchronize(s));
     if (step) {

@@ -73,3 +73,36 @@ def test_forward_and_gradients(bc, H, n):
     assert np.array_equal(net.predict(Xd).cpu().numpy(), y)
     net.close()
     ctx.close()
+
+
+# A recorded forward pass follows the weights, and a recorded Adam step leaves them usable by later calls.
+@pytest.mark.parametrize("H", [48, 256])
+def test_recorded_passes_follow_the_weights(bc, H):
+    n, s = 200, torch.cuda.Stream()
+    rng = np.random.default_rng(H)
+    with torch.cuda.stream(s):
+        X = torch.zeros((n, 144), device="cuda")
+        X[:, :132] = torch.tensor(rng.uniform(-1, 1, (n, 132)), device="cuda")
+        t = torch.tensor(rng.normal(0, 1, n).astype(np.float32), device="cuda")
+        y = torch.empty(n, device="cuda")
+        ctx = bc.Context(32, 6, synth.RADII_2, stream=s)
+        net = bc.MLP(ctx, H, synth.mlp_init(H, H))
+        net.train_step(X, t, 1e-2)  # buffers exist, the forward pass has run
+        net.predict(X)
+    s.synchronize()
+    forward, step = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(forward, stream=s):
+        bc.bc_mlp_predict(net.handle, X, n, y)
+    with torch.cuda.graph(step, stream=s):
+        net.train_step(X, t, 1e-2)
+    Xh = X[:, :132].double().cpu().numpy()
+    for _ in range(2):
+        with torch.cuda.stream(s):
+            step.replay()
+            forward.replay()
+            eager = net.predict(X)
+        s.synchronize()
+        yo, _ = M.forward(split(net.state()["params"], H), Xh, bf=True)
+        assert rel(y.cpu().numpy(), yo) < 1e-3 and torch.equal(y, eager)
+    net.close()
+    ctx.close()
