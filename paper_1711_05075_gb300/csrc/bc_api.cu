@@ -639,15 +639,26 @@ bc_status bc_selftest_wait(bc_ctx_t c)
     CK(cudaStreamSynchronize(c->stream));
     if (c->ws.sync.ensure(sizeof(unsigned), false, c->stream) != cudaSuccess)
         return fail(BC_ERR_OOM, "bc_selftest_wait: counter");
+    struct Scratch {
+        DevBuf b;
+        ~Scratch() { b.release(); }
+    } scratch;
+    if (scratch.b.ensure(xw_selftest_bytes(), true, c->stream) != cudaSuccess)
+        return fail(BC_ERR_OOM, "bc_selftest_wait: scratch");
+    CK(launch_xw_selftest(scratch.b.p, c->err_dev, c->stream));
+    CK(cudaMemcpyAsync(c->pin, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    const bool xw_reported = c->pin[0] & 8;
+    CK(cudaMemset(c->err_dev, 0, sizeof(int)));
     CK(launch_wait_selftest(c->err_dev, c->stream));
     CK(launch_queue_wait_selftest((unsigned *)c->ws.sync.p, c->err_dev, c->stream));
     CK(cudaMemcpyAsync(c->pin, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     const int herr = c->pin[0];
     CK(cudaMemset(c->err_dev, 0, sizeof(int)));
-    if ((herr & 8) && (herr & 16))
-        return fail(BC_ERR_TIMEOUT, "both self-test waits expired and reported it (the tensor-core mbarrier wait and "
-                                    "the persistent launch's dependency wait)");
+    if (xw_reported && (herr & 8) && (herr & 16))
+        return fail(BC_ERR_TIMEOUT, "every self-test wait expired and reported it (one warp's of the x pass, the "
+                                    "tensor-core mbarrier wait and the persistent launch's dependency wait)");
     return fail(BC_ERR_INTERNAL, "a self-test wait did not report its expiry");
 }
 

@@ -101,6 +101,9 @@ cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float 
 cudaError_t launch_xw(const Geometry &g, const Tables &t, const InstDesc *inst, const InstPlan *plan,
                       const PairDesc *pairs, int npairs, const float2 *y1, const float2 *fa_cache, float2 *fa_out,
                       float2 *h, int cap, int *err, int nsm, cudaStream_t s);
+// k_xw where one warp's wait expires (zeroed: xw_selftest_bytes() bytes): sets bit 8 of *err.
+size_t xw_selftest_bytes();
+cudaError_t launch_xw_selftest(void *zeroed, int *err, cudaStream_t s);
 cudaError_t launch_iyz(const Geometry &g, const Tables &t, const PairDesc *pairs, int npairs, const float2 *h,
                        float *out, unsigned long long *keys, int nsm, cudaStream_t s);
 // Binned spreading (bc_binned.cu).  cur[b] = first slot of bin b (the

@@ -48,7 +48,11 @@ cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float 
 // stage inputs of the inverse transform, so the conjugate product needs no
 // exchange.  With pr.a < 0 the spectrum of A comes from fa (layout
 // [m_z][j_y][j_x]); with pr.b < 0 it is written there and nothing else happens.
-// Output h[k_x][m_z][j_y].  Every wait is bounded (bit 8 of the error word).
+// Output h[k_x][m_z][j_y].  Every wait is bounded (bit 8 of the error word).  A warp
+// whose wait expired takes part in the block's barriers to the end: it waits no more,
+// reads whatever its stages hold (in bounds) and its results are not meant to be used;
+// thread 0 issues no further copies.  EXPIRE (the self-test): the second phase's wait
+// of warp 0 counts as expired.
 // Bound by instructions and latency (issue 57%, 128 registers).  20,000 + 20,000
 // balls, N = 128, L = 4: 37.3 us (k_fft_x 38.7 us); the walk's state in every thread's
 // registers instead of shared memory 44.5 us.  Items of 8 lines, not 16: the same time
@@ -84,7 +88,7 @@ struct XwCopies {
     bool done;
 };
 
-template <int NF, int LW>
+template <int NF, int LW, bool EXPIRE = false>
 __global__ void __launch_bounds__(XW<NF, LW>::THREADS, 512 / XW<NF, LW>::THREADS)
 k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *__restrict__ plan,
      const PairDesc *__restrict__ pairs, int npairs, const float2 *__restrict__ y1, const float2 *__restrict__ fa_cache,
@@ -184,7 +188,7 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
     int used = 0, st = 0, par = 0;
     bool ok = true;
     RotStart rs;
-    for (int pi = 0; pi < npairs && ok; pi++) {
+    for (int pi = 0; pi < npairs; pi++) {
         const PairDesc pr = pairs[pi];
         for (int it = rs.first(); it < items; it += gridDim.x) {
             const int mz = it / nch, ch = it - mz * nch, jy = ch * XL + c, my = mode_of(jy, N);
@@ -199,10 +203,18 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
 #pragma unroll
                 for (int r = 0; r < 8; r++) S[r] = make_float2(0.f, 0.f);
                 for (int l = 0; l < L; l++, used++) {
-                    if (threadIdx.x == 0) issue(used);
+                    if (threadIdx.x == 0 && ok) issue(used);
                     __syncwarp();
-                    ok = __all_sync(0xffffffffu, umma_wait(FULL + 8 * st, par, stop, err, XW_ERR));
-                    if (!ok) break;
+                    ok = ok && __all_sync(0xffffffffu, umma_wait(FULL + 8 * st, par, stop, err, XW_ERR));
+                    if constexpr (EXPIRE) {
+                        if (warp == 0 && used == 1) {
+                            ok = false;
+                            if (lane == 0) {
+                                atomicOr(err, XW_ERR);
+                                *stop = 1;
+                            }
+                        }
+                    }
                     const float *wt = reinterpret_cast<const float *>(ring + st * sbytes) + c * A;
                     const float2 *T = reinterpret_cast<const float2 *>(ring + st * sbytes + X::WBYTES);
                     wf_first_any<NF, LW>(E, lane, qx, [&](int sl, int ix, bool inside) {
@@ -218,13 +230,12 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
                         S[r] = make_float2(fmaf(m, v.x, S[r].x), fmaf(m, v.y, S[r].y));
                     }
                     __syncwarp(); // every lane has read the stage and E
-                    if (lane == 0) mbar_arrive(EMPTY + 8 * st);
+                    if (lane == 0 && ok) mbar_arrive(EMPTY + 8 * st); // (a stage is handed on by waits that held)
                     if (++st == XW_STAGES) {
                         st = 0;
                         par ^= 1;
                     }
                 }
-                if (!ok) break;
                 // this instance's level sum is complete: the box origins' phase
                 const int px = p->pos0[0], base = (my + NF) * p->pos0[1] + mz * p->pos0[2];
 #pragma unroll
@@ -235,7 +246,6 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
                     else FA[r] = v;
                 }
             }
-            if (!ok) break;
             if (pr.b < 0) {
                 if (live) {
 #pragma unroll
@@ -461,6 +471,33 @@ cudaError_t launch_xw(const Geometry &g, const Tables &t, const InstDesc *inst, 
     case 256: return xw_t<256, wf_full(256)>(g, t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, cap, err, nsm, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// One pair of empty shapes at N = 32 whose first warp gives up at its second phase:
+// the kernel ends by itself and sets bit 8 of *err.
+size_t xw_selftest_bytes() { return 1024 + sizeof(float2) * 32 * 32 * 16; }
+
+cudaError_t launch_xw_selftest(void *zeroed, int *err, cudaStream_t s)
+{
+    constexpr int NF = 64, LW = 2;
+    using X = XW<NF, LW>;
+    char *p = (char *)zeroed; // two instances, plans and a pair, all zero; tables and output
+    static_assert(2 * sizeof(InstDesc) + 2 * sizeof(InstPlan) + sizeof(PairDesc) <= 1024, "descriptors");
+    const InstDesc *inst = (const InstDesc *)p;
+    const InstPlan *plan = (const InstPlan *)(inst + 2);
+    const PairDesc *pair = (const PairDesc *)(plan + 2);
+    float2 *rest = (float2 *)(p + 1024);
+    Geometry g{};
+    g.N = 32, g.n = 64, g.H = 16, g.L = 2;
+    Tables t{};
+    t.tw_n = t.tw_N = rest;
+    t.wl = (const float *)rest; // (N/2) (N/8) L 8 (N/2 + 1) floats: less than the output
+    static_assert(sizeof(float) * 16 * 4 * 2 * 8 * 17 <= sizeof(float2) * 32 * 32 * 16, "level weights");
+    const size_t smem = X::smem(0);
+    cudaError_t e = set_smem(k_xw<NF, LW, true>, smem);
+    if (e != cudaSuccess) return e;
+    k_xw<NF, LW, true><<<2, X::THREADS, smem, s>>>(g, t, inst, plan, pair, 1, nullptr, nullptr, nullptr, rest, err, 0);
+    return cudaGetLastError();
 }
 
 template <int NI>
