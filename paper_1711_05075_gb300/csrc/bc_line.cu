@@ -48,11 +48,10 @@ cudaError_t launch_build_wl(const Geometry &g, const float *deconv, const float 
 // stage inputs of the inverse transform, so the conjugate product needs no
 // exchange.  With pr.a < 0 the spectrum of A comes from fa (layout
 // [m_z][j_y][j_x]); with pr.b < 0 it is written there and nothing else happens.
-// Output h[k_x][m_z][j_y].  Every wait is bounded (bit 8 of the error word).  A warp
-// whose wait expired takes part in the block's barriers to the end: it waits no more,
-// reads whatever its stages hold (in bounds) and its results are not meant to be used;
-// thread 0 issues no further copies.  EXPIRE (the self-test): the second phase's wait
-// of warp 0 counts as expired.
+// Output h[k_x][m_z][j_y].  Every wait is bounded (bit 8 of the error word); a warp
+// whose wait expired leaves the walk, but takes part in the block's barriers of the
+// rest of it (going on through the walk instead cost a percent of every call).
+// EXPIRE (the self-test): the second phase's wait of warp 0 counts as expired.
 // Bound by instructions and latency (issue 57%, 128 registers).  20,000 + 20,000
 // balls, N = 128, L = 4: 37.3 us (k_fft_x 38.7 us); the walk's state in every thread's
 // registers instead of shared memory 44.5 us.  Items of 8 lines, not 16: the same time
@@ -185,12 +184,12 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
         next_source();
         issue(0);
     }
-    int used = 0, st = 0, par = 0;
+    int used = 0, st = 0, par = 0, pi = 0, it = 0;
     bool ok = true;
     RotStart rs;
-    for (int pi = 0; pi < npairs; pi++) {
+    for (; pi < npairs; pi++) {
         const PairDesc pr = pairs[pi];
-        for (int it = rs.first(); it < items; it += gridDim.x) {
+        for (it = rs.first(); it < items; it += gridDim.x) {
             const int mz = it / nch, ch = it - mz * nch, jy = ch * XL + c, my = mode_of(jy, N);
             float2 FA[8], S[8];
             if (pr.a < 0) {
@@ -203,9 +202,9 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
 #pragma unroll
                 for (int r = 0; r < 8; r++) S[r] = make_float2(0.f, 0.f);
                 for (int l = 0; l < L; l++, used++) {
-                    if (threadIdx.x == 0 && ok) issue(used);
+                    if (threadIdx.x == 0) issue(used);
                     __syncwarp();
-                    ok = ok && __all_sync(0xffffffffu, umma_wait(FULL + 8 * st, par, stop, err, XW_ERR));
+                    ok = __all_sync(0xffffffffu, umma_wait(FULL + 8 * st, par, stop, err, XW_ERR));
                     if constexpr (EXPIRE) {
                         if (warp == 0 && used == 1) {
                             ok = false;
@@ -215,6 +214,7 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
                             }
                         }
                     }
+                    if (!ok) break;
                     const float *wt = reinterpret_cast<const float *>(ring + st * sbytes) + c * A;
                     const float2 *T = reinterpret_cast<const float2 *>(ring + st * sbytes + X::WBYTES);
                     wf_first_any<NF, LW>(E, lane, qx, [&](int sl, int ix, bool inside) {
@@ -230,12 +230,13 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
                         S[r] = make_float2(fmaf(m, v.x, S[r].x), fmaf(m, v.y, S[r].y));
                     }
                     __syncwarp(); // every lane has read the stage and E
-                    if (lane == 0 && ok) mbar_arrive(EMPTY + 8 * st); // (a stage is handed on by waits that held)
+                    if (lane == 0) mbar_arrive(EMPTY + 8 * st);
                     if (++st == XW_STAGES) {
                         st = 0;
                         par ^= 1;
                     }
                 }
+                if (!ok) break;
                 // this instance's level sum is complete: the box origins' phase
                 const int px = p->pos0[0], base = (my + NF) * p->pos0[1] + mz * p->pos0[2];
 #pragma unroll
@@ -246,6 +247,7 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
                     else FA[r] = v;
                 }
             }
+            if (!ok) break;
             if (pr.b < 0) {
                 if (live) {
 #pragma unroll
@@ -291,7 +293,16 @@ k_xw(Geometry g, Tables tb, const InstDesc *__restrict__ inst, const InstPlan *_
             }
             __syncthreads();
         }
+        if (!ok) break;
         rs.rot += items;
+    }
+    if (!ok) { // the walk from this item on, three barriers per item with an output (matched by number)
+        for (bool here = true; pi < npairs; pi++, here = false) {
+            if (!here) it = rs.first();
+            for (const bool barriers = pairs[pi].b >= 0; it < items; it += gridDim.x)
+                for (int k = 0; barriers && k < 3; k++) asm volatile("barrier.cta.sync 0;" ::: "memory");
+            rs.rot += items;
+        }
     }
     // the copies in flight land before the block's shared memory goes (a wait that
     // expired leaves some; otherwise all are complete)
