@@ -210,10 +210,10 @@ cudaError_t back_t(const Geometry &g, const Tables &t, const InstDesc *inst, con
     // the x pass's shared-memory layout (level weights for as many levels as fit
     // at the kernel's blocks per SM); the inverse units reuse its tiles
     using XL = XSmem<NF, NI, SP, S>;
-    const size_t room = (NF <= 256 ? 228 * 1024 / 2 : 228 * 1024) - 1024 - 512 - XL::bytes(0);
-    const int G = (int)std::max<size_t>(1, std::min<size_t>((size_t)g.L, room / XL::per_level));
+    const size_t room = (NF <= 256 ? 228 * 1024 / 2 : 228 * 1024) - 1024 - 512;
+    const int G = XL::groups(g.L, room);
     const size_t smem = XL::bytes(G);
-    cudaError_t e = set_smem(k_back<NF, NI, SP, S>, smem);
+    cudaError_t e = set_smem(k_back<NF, NI, SP, S>, XL::bytes(XL::groups(BC_MAX_LEVELS, room)));
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(sync, 0, sizeof(unsigned) * back_sync_words(NI, npairs), s)) != cudaSuccess) return e;
     k_back<NF, NI, SP, S><<<resident_blocks(k_back<NF, NI, SP, S>, smem, nsm), TB, smem, s>>>(

@@ -122,6 +122,10 @@ static int resident_blocks(K kernel, size_t smem, int nsm, int threads = TB)
     return per * nsm;
 }
 
+// Lets a kernel take up to `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel, not to a launch, and a launch beyond it fails: where the amount depends on the
+// shapes, `bytes` is the largest of any call, so that a smaller call in another thread
+// does not lower it between this one's setting and launch.
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes)
 {

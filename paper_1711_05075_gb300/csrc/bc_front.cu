@@ -244,7 +244,7 @@ static cudaError_t zy_t(const Geometry &g, const Tables &t, const InstDesc *inst
         if ((long long)ninst * g.L * cap <= 2LL * nsm)
             return zy_t<NF, 2>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
     const size_t smem = zy_smem<NF, LW>(cap);
-    cudaError_t e = set_smem(k_zy<NF, LW>, smem);
+    cudaError_t e = set_smem(k_zy<NF, LW>, zy_smem<NF, LW>(NF)); // cap <= NF
     if (e != cudaSuccess) return e;
     return launch_k(k_zy<NF, LW>, resident_blocks(k_zy<NF, LW>, smem, nsm, ZY_WARPS * 32), ZY_WARPS * 32, smem, s,
                     g.pdl != 0, g, t, inst, ninst, plan, grid, y1, zy_ps(cap), clear);

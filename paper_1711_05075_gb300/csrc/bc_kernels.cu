@@ -1170,10 +1170,10 @@ static cudaError_t fft_x_t(const Geometry &g, const Tables &t, const InstDesc *i
     // level weights for as many levels as fit beside the tiles at the kernel's
     // blocks per SM (two up to NF = 256, else one): all of them in the usual cases
     using XL = XSmem<NF, NI, SP, S>;
-    const size_t room = (NF <= 256 ? 228 * 1024 / 2 : 228 * 1024) - 1024 - XL::bytes(0);
-    const int G = (int)std::max<size_t>(1, std::min<size_t>((size_t)g.L, room / XL::per_level));
+    const size_t room = (NF <= 256 ? 228 * 1024 / 2 : 228 * 1024) - 1024;
+    const int G = XL::groups(g.L, room);
     const size_t smem = XL::bytes(G);
-    cudaError_t e = set_smem(k_fft_x<NF, NI, SP, S>, smem);
+    cudaError_t e = set_smem(k_fft_x<NF, NI, SP, S>, XL::bytes(XL::groups(BC_MAX_LEVELS, room)));
     if (e != cudaSuccess) return e;
     return launch_k(k_fft_x<NF, NI, SP, S>, resident_blocks(k_fft_x<NF, NI, SP, S>, smem, nsm, tb_of(NF)), tb_of(NF), smem, s,
                     g.pdl != 0, g, t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, G);

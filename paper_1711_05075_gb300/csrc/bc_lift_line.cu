@@ -340,11 +340,13 @@ k_lx_rx(const float2 *__restrict__ XA, const float2 *__restrict__ XB, int bA, in
         }
 }
 
+constexpr size_t LX_SMEM = 220 * 1024; // of k_lx_rx, at most (lift4_line_fits)
+
 template <int NF>
 cudaError_t lx_x(const float2 *y1, int b0, int bR, const float2 *tw, float2 *X1, int *err, int nsm, cudaStream_t s)
 {
     const size_t smem = LX<NF>::smem(b0);
-    cudaError_t e = set_smem(k_lx_x<NF>, smem);
+    cudaError_t e = set_smem(k_lx_x<NF>, LX<NF>::smem(NF)); // b0 < NF
     if (e != cudaSuccess) return e;
     k_lx_x<NF><<<resident_blocks(k_lx_x<NF>, smem, nsm, LX<NF>::THREADS), LX<NF>::THREADS, smem, s>>>(y1, b0, bR, tw, X1, err);
     return cudaGetLastError();
@@ -355,7 +357,7 @@ cudaError_t lx_rx(const float2 *XA, const float2 *XB, int bA, int bB, int4 dlo, 
                   int nslices, double period_r, float scale, float2 *h, int *err, int nsm, cudaStream_t s)
 {
     const size_t smem = rx_smem(N, NRK, NS, bA, bB);
-    cudaError_t e = set_smem(k_lx_rx<N, NRK, NS>, smem);
+    cudaError_t e = set_smem(k_lx_rx<N, NRK, NS>, LX_SMEM);
     if (e != cudaSuccess) return e;
     k_lx_rx<N, NRK, NS><<<resident_blocks(k_lx_rx<N, NRK, NS>, smem, nsm, 2 * N), 2 * N, smem, s>>>(
         XA, XB, bA, bB, dlo, t.wts, slices, nslices, period_r, scale, t.tw_s, t.tw_r, h, err);
@@ -407,7 +409,7 @@ cudaError_t lift4_build_weights(const Lift4Tables &t, int N, int Nr, const float
 // Shared memory of the last pass: two stages of both shapes' planes of one (m_z, j_y).
 bool lift4_line_fits(int N, int Nr, int bA, int bB, int nslices)
 {
-    return rx_smem(N, Nr, nslices > 1 ? LX_NS : 1, bA, bB) <= 220 * 1024;
+    return rx_smem(N, Nr, nslices > 1 ? LX_NS : 1, bA, bB) <= LX_SMEM;
 }
 
 cudaError_t lift4_line_spectrum(const Lift4Tables &t, int N, int Nr, const float4 *knots, int n, const Lift4Rot &rot,

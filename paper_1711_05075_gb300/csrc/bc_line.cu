@@ -465,7 +465,7 @@ static cudaError_t xw_t(const Geometry &g, const Tables &t, const InstDesc *inst
             return xw_t<NF, 2>(g, t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, cap, err, nsm, s);
     using X = XW<NF, LW>;
     const size_t smem = X::smem(cap);
-    cudaError_t e = set_smem(k_xw<NF, LW>, smem);
+    cudaError_t e = set_smem(k_xw<NF, LW>, X::smem(NF)); // cap <= NF
     if (e != cudaSuccess) return e;
     return launch_k(k_xw<NF, LW>, resident_blocks(k_xw<NF, LW>, smem, nsm, X::THREADS), X::THREADS, smem, s, g.pdl != 0, g,
                     t, inst, plan, pairs, npairs, y1, fa_cache, fa_out, h, err, cap);

@@ -2,8 +2,10 @@
 // (bc_kernels.cu) and the persistent back-half kernel (bc_back.cu).  Not part
 // of the public interface.
 #pragma once
+#include <algorithm>
 #include <climits>
 
+#include "../../include/ballcorr.h"
 #include "bc_device.cuh"
 
 namespace bc {
@@ -170,6 +172,8 @@ struct XSmem {
                                  (size_t)NI * CL + 2 * (size_t)MAXR * CL;
     static constexpr size_t per_level = sizeof(float) * (NI / 2 + 1) * CL;
     static constexpr size_t bytes(int G) { return sizeof(float2) * f2 + per_level * (size_t)G; }
+    // weights of at most L levels in `room` bytes beside the tiles (one group at least)
+    static int groups(int L, size_t room) { return (int)std::max<size_t>(1, std::min<size_t>((size_t)L, (room - bytes(0)) / per_level)); }
     struct Ptr {
         float2 *twF, *twI, *S0, *S1, *FAt, *stg0, *stg1;
         float *Ts;

@@ -92,7 +92,7 @@ k_query_eval(const float2 *__restrict__ ghat, const int4 *__restrict__ modes, in
 // 4,096 modes and points, 14.4 with it, k_query_eval 31).  Bound by instruction
 // issue: one block of 16 warps per SM at 4,096 points.  The tables [axis][|m|][lane] hold the same
 // values as k_query_eval's; a negative component takes the conjugate.
-constexpr int QL_WARPS = 16, QL_RING = 4;
+constexpr int QL_WARPS = 16, QL_RING = 4, QL_MAX_M = 128; // N <= 256: components below 128
 
 __global__ void __launch_bounds__(QL_WARPS * 32)
 k_query_lines(const QlGroup *__restrict__ groups, int ngroups, int M, double inv_period, float scale,
@@ -172,8 +172,9 @@ k_query_lines(const QlGroup *__restrict__ groups, int ngroups, int M, double inv
 cudaError_t launch_query_lines(const QlGroup *groups, int ngroups, int M, double period, const float *t, int npts, float *g,
                                cudaStream_t s)
 {
-    const size_t smem = sizeof(QlGroup) * QL_WARPS * QL_RING + sizeof(float2) * 3 * (size_t)M * 32;
-    cudaError_t e = set_smem(k_query_lines, smem);
+    auto bytes = [](int m) { return sizeof(QlGroup) * QL_WARPS * QL_RING + sizeof(float2) * 3 * (size_t)m * 32; };
+    const size_t smem = bytes(M);
+    cudaError_t e = set_smem(k_query_lines, bytes(QL_MAX_M));
     if (e != cudaSuccess) return e;
     k_query_lines<<<(npts + 31) / 32, QL_WARPS * 32, smem, s>>>(groups, ngroups, M, 1.0 / period,
                                                                  (float)(1.0 / (period * period * period)), t, npts, g);
