@@ -334,10 +334,12 @@ bc_status bc_lift_destroy(bc_lift_t lift);
  * A new context starts with {0, 64, 1, 0, 1, 0, 1} (z_transform 0 where 1 is
  * not available).  Plans keep the choices in force when
  * they were made.  bc_autotune times the candidates on the given shapes --
- * bc_correlate of A with B (identity) for `spread`, `z_transform` and `persistent` (when rotations > 0,
- * `z_transform` is decided again on the sweep with the chosen batch); in FP32 contexts the
+ * bc_correlate of A with B (identity) for every combination of `spread`, `z_transform` and
+ * `persistent` (when rotations > 0, `z_transform` is decided again on the sweep with the chosen
+ * batch, and `persistent` with it where it was 1); in FP32 contexts the
  * per-stage times of profiled correlations under each schedule, pass by pass,
- * for `fft_schedule`; when rotations > 0, a sweep of that many fixed rotations
+ * for `fft_schedule`, which is left as it is where the chosen passes do not read it (see
+ * `z_transform`); when rotations > 0, a sweep of that many fixed rotations
  * of B for each sweep_batch in {16, 32, 64, 128, 256} not above it -- keeps
  * the fastest in the context and returns them in out (may be NULL).  It
  * synchronises the stream, grows the context's workspaces to the largest

@@ -1931,55 +1931,45 @@ bc_status bc_autotune(bc_ctx_t c, bc_shape_t A, bc_shape_t B, int rotations, bc_
         if ((e = c->tune.ensure(sizeof(float) * (size_t)std::max<long long>(N3, 2LL * rotations), false, c->stream)) != cudaSuccess)
             return cuda_fail(e, "bc_autotune: scratch");
         float *dout = (float *)c->tune.p;
-        // spreading: one correlation of A with B, unrotated
+        // spreading, z transform and back half together, on one correlation of A with B,
+        // unrotated: the passes of bc_front.cu stand for one combination of all three
+        // (chosen one after the other, they went untimed where another was set before)
         static const float ident[4] = {1.f, 0.f, 0.f, 0.f};
+        struct Choice {
+            int spread, z_tc, persistent;
+        };
+        auto take = [&](const Choice &x) { c->spread_mode = x.spread, c->z_tc = x.z_tc, c->persistent = x.persistent; };
+        auto fastest = [&](const std::vector<Choice> &all, int warm, int reps, auto pass) {
+            const Choice saved{c->spread_mode, c->z_tc, c->persistent};
+            Choice best_choice = saved;
+            float best_ms = 0.f;
+            for (size_t i = 0; i < all.size(); i++) {
+                take(all[i]);
+                float ms = 0.f;
+                if (bc_status s = time_median(c, pass, warm, reps, &ms)) {
+                    take(saved);
+                    return s;
+                }
+                if (i == 0 || ms < best_ms) {
+                    best_ms = ms;
+                    best_choice = all[i];
+                }
+            }
+            take(best_choice);
+            return BC_OK;
+        };
+        std::vector<Choice> choices;
+        for (int spread = 0; spread <= 1; spread++)
+            for (int z = 0; z <= (c->zdft && spread == 0 ? 1 : 0); z++) // z transform: FFT or tensor-core DFT product (spread 0 only)
+                for (int b = 0; b <= 1; b++) // back half: three launches or one persistent launch
+                    choices.push_back(Choice{spread, c->zdft && spread == 0 ? z : c->z_tc, b});
+        if (bc_status s = fastest(choices, 3, 7, [&]() { return bc_correlate(c, A, B, ident, 1, dout, 1); })) return s;
         float best = 0.f;
-        int best_mode = c->spread_mode;
-        for (int mode = 0; mode <= 1; mode++) {
-            c->spread_mode = mode;
-            float ms = 0.f;
-            bc_status s = time_median(c, [&]() { return bc_correlate(c, A, B, ident, 1, dout, 1); }, 3, 7, &ms);
-            if (s != BC_OK) {
-                c->spread_mode = best_mode;
-                return s;
-            }
-            if (mode == 0 || ms < best) {
-                best = ms;
-                best_mode = mode;
-            }
-        }
-        c->spread_mode = best_mode;
-        // z transform: FFT or tensor-core DFT product (spread 0 only)
-        if (c->zdft && c->spread_mode == 0) {
-            const int saved = c->z_tc;
-            float tz[2] = {0.f, 0.f};
-            for (int z = 0; z <= 1; z++) {
-                c->z_tc = z;
-                bc_status s = time_median(c, [&]() { return bc_correlate(c, A, B, ident, 1, dout, 1); }, 3, 7, &tz[z]);
-                if (s != BC_OK) {
-                    c->z_tc = saved;
-                    return s;
-                }
-            }
-            c->z_tc = tz[1] < tz[0] ? 1 : 0;
-        }
-        // back half: three launches or one persistent launch
-        {
-            const int saved = c->persistent;
-            float tb[2] = {0.f, 0.f};
-            for (int b = 0; b <= 1; b++) {
-                c->persistent = b;
-                bc_status s = time_median(c, [&]() { return bc_correlate(c, A, B, ident, 1, dout, 1); }, 3, 7, &tb[b]);
-                if (s != BC_OK) {
-                    c->persistent = saved;
-                    return s;
-                }
-            }
-            c->persistent = tb[1] < tb[0] ? 1 : 0;
-        }
         // radix schedule per forward pass (the split-precision passes have their own):
         // the stage times of profiled correlations under each schedule, pass by pass
-        if (c->g.prec == 0) {
+        // (where the passes read it: those of bc_front.cu have one each, and the
+        // schedule set before is kept for the shapes that do not take them)
+        if (c->g.prec == 0 && !front_ok(c, {A, B})) {
             double stage_ms[2][BC_NUM_STAGES] = {};
             const int saved = c->fft_sched;
             for (int sched = 0; sched <= 1; sched++) {
@@ -2034,21 +2024,15 @@ bc_status bc_autotune(bc_ctx_t c, bc_shape_t A, bc_shape_t B, int rotations, bc_
             }
             c->sweep_batch = best_batch;
             // the z transform again, on the sweep itself (its passes batch many
-            // rotations of the smaller shape, which can favour the other transform)
+            // rotations of the smaller shape, which can favour the other transform),
+            // with the tensor-core one also beside three back-half launches
             if (c->zdft && c->spread_mode == 0) {
-                const int saved = c->z_tc;
-                float tz[2] = {0.f, 0.f};
-                for (int z = 0; z <= 1; z++) {
-                    c->z_tc = z;
-                    bc_status s = time_median(
-                        c, [&]() { return sweep_impl(c, A, B, q.data(), nullptr, rotations, best_batch, dpeak, darg, 1); },
-                        1, 3, &tz[z]);
-                    if (s != BC_OK) {
-                        c->z_tc = saved;
-                        return s;
-                    }
-                }
-                c->z_tc = tz[1] < tz[0] ? 1 : 0;
+                std::vector<Choice> zs{Choice{0, 0, c->persistent}, Choice{0, 1, c->persistent}};
+                if (c->persistent) zs.push_back(Choice{0, 1, 0});
+                if (bc_status s = fastest(zs, 1, 3, [&]() {
+                        return sweep_impl(c, A, B, q.data(), nullptr, rotations, best_batch, dpeak, darg, 1);
+                    }))
+                    return s;
             }
         }
         if (out) bc_get_tuning(c, out);

@@ -1,0 +1,40 @@
+"""The autotuner times the passes for shapes inside one period whatever was set before, and leaves the radix
+schedule alone where they do not read it."""
+import numpy as np
+import pytest
+
+from paper_1711_05075_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def context(bc, N, semi=(0.5, 0.3, 0.35), n=3000):
+    ctx = bc.Context(N, 8, synth.RADII_4)
+    A = synth.ellipsoid_shape(n, 1, synth.RADII_4, synth.PROBS_4, semi)
+    B = synth.ellipsoid_shape(n, 2, synth.RADII_4, synth.PROBS_4)
+    return ctx, ctx.shape(A.xyz.astype(np.float32), A.level), ctx.shape(B.xyz.astype(np.float32), B.level)
+
+
+# At N = 64 these shapes take 43 us with the passes for shapes inside one period (spread 0, z_transform 1,
+# persistent 0) and 50 us or more with every other choice, and more so at N = 128 (99 against 130).
+@pytest.mark.parametrize("N", [64, 128])
+@pytest.mark.parametrize("before", [dict(persistent=1), dict(spread=1, z_transform=0), dict()])
+@pytest.mark.parametrize("rotations", [0, 16])
+def test_finds_the_fastest_combination_and_keeps_the_schedule(N, before, rotations):
+    import paper_1711_05075_gb300 as bc
+    ctx, a, b = context(bc, N)
+    ctx.set_tuning(fft_schedule=5, **before)
+    t = ctx.autotune(a, b, rotations)
+    assert (t["spread"], t["z_transform"], t["persistent"]) == (0, 1, 0), t
+    assert t["fft_schedule"] == 5 and t == ctx.tuning  # no pass that was timed reads it
+    ctx.close()
+
+
+def test_across_the_period_the_schedule_is_chosen():
+    import paper_1711_05075_gb300 as bc
+    ctx, a, b = context(bc, 128, (0.99, 0.3, 0.7))
+    ctx.set_tuning(fft_schedule=7)
+    t = ctx.autotune(a, b)
+    assert t["fft_schedule"] != 7 and t["graphs"] == 1, t  # schedule 1 of every pass at once is slower at n = 256
+    ctx.close()
