@@ -65,7 +65,7 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
 // The passes for boxes narrower than the period on every axis (bc_lift_line.cu).
 size_t lift4_weight_bytes(int N, int Nr);
 cudaError_t lift4_build_weights(const Lift4Tables &t, int N, int Nr, const float2 *cone, cudaStream_t s);
-bool lift4_line_fits(int N, int Nr, int bA, int bB, int nslices);
+bool lift4_line_fits(int N, int Nr, const Lift4Box &ba, const Lift4Box &bb, int nslices, int nsm);
 inline size_t lift4_cells(const Lift4Box &b) { return (size_t)b.b[3] * b.b[0] * b.b[1] * b.b[2]; }
 // x planes X1[m_z][j_y][i_r][j_x] of n knots; G: the box grid, whose first `clean` cells are
 // zero (with none, the passes leave the box's cells zero behind them; else they don't); y1: scratch

@@ -406,10 +406,26 @@ cudaError_t lift4_build_weights(const Lift4Tables &t, int N, int Nr, const float
     return cudaGetLastError();
 }
 
-// Shared memory of the last pass: two stages of both shapes' planes of one (m_z, j_y).
-bool lift4_line_fits(int N, int Nr, int bA, int bB, int nslices)
+// Whether boxes narrower than the period take these passes: the last one's shared memory
+// holds two stages of both shapes' planes of one (m_z, j_y), and the passes are the faster
+// ones.  They save on the transforms of the box (bX bY z lines, bX N/2 y lines and N N/2 x
+// lines per cell along r), but repeat the r transforms for every LX_NS sections.
+//  - Fewer items of the last pass than SMs (N = 32): a call waits for one block's chain,
+//    which grows with N_r and the repetitions.  300 + 300 knots: N_r = 16, 12 sections 215
+//    us (general passes 231), 16 sections 239 (243); N_r = 32, 4 sections 190 (221), 5
+//    sections 233 (224), 16 sections 341 (258); N_r = 64, 1 section 264 (223).
+//  - Otherwise the repetitions are weighed against the lines saved (measured at N = 64, 96
+//    and 128 on boxes of a ninth and half of the period, line form / general in ms at N =
+//    128, N_r = 64, half: 5 sections 2.30 / 3.03, 9 sections 3.17 / 3.42, 13 sections 4.05 /
+//    3.55; ninth: 4 sections 1.19 / 1.94, 5 sections 2.00 / 2.07, 9 sections 2.88 / 2.46; at
+//    N_r = 32, ninth, 16 sections 1.61 / 1.83).
+bool lift4_line_fits(int N, int Nr, const Lift4Box &ba, const Lift4Box &bb, int nslices, int nsm)
 {
-    return rx_smem(N, Nr, nslices > 1 ? LX_NS : 1, bA, bB) <= LX_SMEM;
+    if (rx_smem(N, Nr, nslices > 1 ? LX_NS : 1, ba.b[3], bb.b[3]) > LX_SMEM) return false;
+    const int turns = (nslices + LX_NS - 1) / LX_NS;
+    if (N / 2 * (N / XL) < nsm) return turns * Nr <= 48;
+    auto lines = [&](const Lift4Box &b) { return (double)b.b[0] * (b.b[1] + N / 2) + (double)N * (N / 2); };
+    return 0.5 * (lines(ba) + lines(bb)) >= (turns - 1) * (double)Nr * Nr / 4300.0 * N * N;
 }
 
 cudaError_t lift4_line_spectrum(const Lift4Tables &t, int N, int Nr, const float4 *knots, int n, const Lift4Rot &rot,

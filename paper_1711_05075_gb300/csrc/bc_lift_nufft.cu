@@ -458,7 +458,7 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
             even[k].b[a] = a == 1 || a == 2 ? (bx[k].b[a] + 1) & ~1 : bx[k].b[a];
             inside = inside && !whole;
         }
-    *line = inside && t.wts && lift4_line_fits(N, Nr, bx[0].b[3], bx[1].b[3], nslices);
+    *line = inside && t.wts && lift4_line_fits(N, Nr, bx[0], bx[1], nslices, nsm);
     if (*line) {
         // spectra in turn over the same grid and y planes; A's x planes have their own
         // place, B's take the grid's, which only A's passes have to leave clear
