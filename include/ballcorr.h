@@ -268,7 +268,9 @@ typedef struct {
                           knots onto the (2N)^3 x 2Nr grid, a 4D FFT keeping the modes
                           above, deconvolution, the collapse formed from the two
                           spectra directly (Nr >= 16; workspace 52 x 2Nr x N^3 bytes,
-                          a table of the modes' weights of about Nr x N^3 bytes) */
+                          and, from the first call whose shapes fit inside the period on
+                          all axes, a table of the modes' weights of about Nr x N^3 bytes;
+                          where it cannot be allocated the call goes without) */
 } bc_lift_params;
 bc_status bc_lift_create(const bc_lift_params *params, void *cuda_stream, bc_lift_t *out);
 bc_status bc_lift_correlate(bc_lift_t lift, const float *A, int nA, const float *B, int nB, const float *quat,

@@ -626,7 +626,6 @@ bc_status bc_lift_create(const bc_lift_params *p, void *cuda_stream, bc_lift_t *
         lf->t4.consts = f + N + Nr;
         lf->t4.dbox = (int *)(((uintptr_t)(lf->t4.consts + CONSTS_FLOATS) + 15) & ~(uintptr_t)15);
         if ((e = cudaMallocHost(&lf->t4.hbox, LIFT4_BOX_BYTES)) != cudaSuccess) return bail(e, "cudaMallocHost box");
-        if ((e = cudaMalloc(&lf->t4.wts, lift4_weight_bytes(N, Nr))) != cudaSuccess) return bail(e, "cudaMalloc mode weights");
         Geometry gs{}, gr{};
         gs.N = N, gs.n = 2 * N, gs.W = W, gs.L = 0;
         gr.N = Nr, gr.n = 2 * Nr, gr.W = W, gr.L = 0;
@@ -635,7 +634,6 @@ bc_status bc_lift_create(const bc_lift_params *p, void *cuda_stream, bc_lift_t *
             (e = launch_build_tables(gr, beta, lf->period_r, nullptr, lf->t4.deconv_r, nullptr, lf->t4.tw_r, twNr,
                                      lf->t4.consts, lf->stream)) != cudaSuccess)
             return bail(e, "bc_lift_create: NUFFT tables");
-        if ((e = lift4_build_weights(lf->t4, N, Nr, lf->cone, lf->stream)) != cudaSuccess) return bail(e, "bc_lift_create: mode weights");
     }
     if ((e = cudaStreamSynchronize(lf->stream)) != cudaSuccess) return bail(e, "bc_lift_create: sync");
     cudaFree(g);

@@ -42,7 +42,7 @@ struct Lift4Tables {
     // their plans and descriptors for k_zy -- and the page-locked host copy
     int *dbox = nullptr;
     int *hbox = nullptr;
-    float2 *wts = nullptr; // the last pass's mode weights (lift4_build_weights)
+    float2 *wts = nullptr; // the line passes' mode weights, built by the first call that takes them (lift4_pair)
 };
 constexpr size_t LIFT4_BOX_BYTES = 1024;
 
@@ -58,7 +58,7 @@ size_t lift4_ws_bytes(int N, int Nr);
 // lift4_boxes first: it enqueues the search for the two shapes' support boxes.
 cudaError_t lift4_boxes(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                         const double (&RB)[9], double period, double period_r, int nsm, cudaStream_t s);
-cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
+cudaError_t lift4_pair(Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                        const double (&RB)[9], double period, double period_r, const float2 *cone, const float *slices,
                        int nslices, float scale, void *ws, float2 *h, bool *line, int *err, int nsm, cudaStream_t s);
 

@@ -428,7 +428,7 @@ cudaError_t lift4_boxes(const Lift4Tables &t, int N, int Nr, const float4 *kA, i
     return cudaMemcpyAsync(t.hbox, t.dbox, 16 * sizeof(int), cudaMemcpyDeviceToHost, s);
 }
 
-cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
+cudaError_t lift4_pair(Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                        const double (&RB)[9], double period, double period_r, const float2 *cone, const float *slices,
                        int nslices, float scale, void *ws, float2 *h, bool *line, int *err, int nsm, cudaStream_t s)
 {
@@ -458,7 +458,17 @@ cudaError_t lift4_pair(const Lift4Tables &t, int N, int Nr, const float4 *kA, in
             even[k].b[a] = a == 1 || a == 2 ? (bx[k].b[a] + 1) & ~1 : bx[k].b[a];
             inside = inside && !whole;
         }
-    *line = inside && t.wts && lift4_line_fits(N, Nr, bx[0], bx[1], nslices, nsm);
+    *line = inside && lift4_line_fits(N, Nr, bx[0], bx[1], nslices, nsm);
+    if (*line && !t.wts) { // the handle's first call that reads the weights; without room for them, the general passes
+        float2 *w = nullptr;
+        if (cudaMalloc(&w, lift4_weight_bytes(N, Nr)) == cudaSuccess) {
+            t.wts = w;
+            if ((e = lift4_build_weights(t, N, Nr, cone, s)) != cudaSuccess) return e;
+        } else {
+            cudaGetLastError();
+            *line = false;
+        }
+    }
     if (*line) {
         // spectra in turn over the same grid and y planes; A's x planes have their own
         // place, B's take the grid's, which only A's passes have to leave clear
