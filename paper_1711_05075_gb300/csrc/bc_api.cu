@@ -212,15 +212,15 @@ struct bc_shape_s {
 struct bc_query_s {
     bc_ctx_t ctx = nullptr;
     int count = 0;          // m'
-    DevBuf modes, ghat, io; // int4 modes, their g^ values, staging for host points and results
+    DevBuf lists, ghat, io; // modes and groups; the modes' g^ values; staging for host points and results
+    int4 *modes = nullptr;  // (m_x, m_y, m_z, w)
     // the same modes by columns (m_x, m_y), four columns to a group, weighted (launch_query_lines)
-    DevBuf groups;
+    QlGroup *groups = nullptr;
     int ngroups = 0, top = 0; // components below top
     void release()
     {
-        modes.release();
+        lists.release();
         ghat.release();
-        groups.release();
         io.release();
     }
 };
@@ -2068,20 +2068,25 @@ static std::vector<std::array<int, 4>> query_modes(int N, int mprime)
         if ((long long)cand.size() >= mprime || R == h) break;
         R = R * 2;
     }
-    std::sort(cand.begin(), cand.end());
-    std::vector<std::array<int, 4>> out;
-    for (int i = 0; i < mprime && i < (int)cand.size(); i++)
-        out.push_back({cand[i][1], cand[i][2], cand[i][3], cand[i][0] == 0 ? 1 : 2});
+    // the candidates come in the order (m_x, m_y, m_z): what is left is a stable sort by |m|^2
+    std::vector<int> at((size_t)3 * R * R + 2, 0); // first place of each |m|^2
+    for (const auto &m : cand) at[(size_t)m[0] + 1]++;
+    for (size_t q = 1; q < at.size(); q++) at[q] += at[q - 1];
+    std::vector<std::array<int, 4>> out((size_t)std::min<long long>(mprime, (long long)cand.size()));
+    for (const auto &m : cand) {
+        const size_t i = (size_t)at[(size_t)m[0]]++;
+        if (i < out.size()) out[i] = {m[1], m[2], m[3], m[0] == 0 ? 1 : 2};
+    }
     return out;
 }
 
 // The modes by columns (m_x, m_y), longest first, in the records of
-// launch_query_lines: their heads, and for each of a record's 8-byte places the
-// mode whose weighted g^ belongs there (weight 0 where there is none).
+// launch_query_lines: their heads, and for each of a record's values the index of
+// its mode (-1 where there is none).
 static void query_columns(const std::vector<std::array<int, 4>> &modes, int N, std::vector<QlGroup> *heads,
-                          std::vector<std::array<int, 4>> *places, int *top)
+                          std::vector<int> *src, int *top)
 {
-    const int h = N / 2, per = (int)(sizeof(QlGroup) / sizeof(float2));
+    const int h = N / 2;
     std::vector<int> len((size_t)N * N, 0); // by column: highest m_z + 1
     *top = 1;
     for (const auto &m : modes) {
@@ -2107,12 +2112,13 @@ static void query_columns(const std::vector<std::array<int, 4>> &modes, int N, s
             }
             heads->push_back(g);
         }
-        for (size_t c = 0; c < 4 && q + c < order.size(); c++) first[order[q + c]] = g0 * per + QL_HEAD + (int)c;
+        for (size_t c = 0; c < 4 && q + c < order.size(); c++) first[order[q + c]] = g0 * QL_VALUES + (int)c;
     }
-    places->assign(heads->size() * (size_t)per, std::array<int, 4>{0, 0, 0, 0});
-    for (const auto &m : modes) {
-        const size_t at = first[(size_t)(m[0] + h) * N + m[1] + h] + (size_t)(m[2] / QL_ROWS) * per + 4 * (size_t)(m[2] % QL_ROWS);
-        (*places)[at] = m;
+    src->assign(heads->size() * (size_t)QL_VALUES, -1);
+    for (size_t i = 0; i < modes.size(); i++) {
+        const auto &m = modes[i];
+        const size_t at = first[(size_t)(m[0] + h) * N + m[1] + h] + (size_t)(m[2] / QL_ROWS) * QL_VALUES + 4 * (size_t)(m[2] % QL_ROWS);
+        (*src)[at] = (int)i;
     }
 }
 
@@ -2133,9 +2139,13 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
         const std::vector<std::array<int, 4>> modes = query_modes(N, mprime);
         if ((int)modes.size() != mprime) return fail(BC_ERR_INTERNAL, "bc_query_create: mode enumeration");
         std::vector<QlGroup> heads;
-        std::vector<std::array<int, 4>> places;
+        std::vector<int> src;
         int top = 1;
-        query_columns(modes, N, &heads, &places, &top);
+        query_columns(modes, N, &heads, &src, &top);
+        // the records' heads follow the indices: one upload
+        const size_t nsrc = src.size();
+        src.resize(nsrc + heads.size() * (QL_HEAD * 2));
+        for (size_t i = 0; i < heads.size(); i++) std::memcpy(&src[nsrc + i * QL_HEAD * 2], &heads[i], QL_HEAD * sizeof(float2));
         cudaStream_t st = c->stream;
         cudaError_t e;
         qo = new bc_query_s();
@@ -2149,21 +2159,18 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
             delete qo;
             return s;
         };
-        if ((e = qo->modes.ensure(sizeof(int4) * mprime, false, st)) != cudaSuccess ||
-            (e = qo->ghat.ensure(sizeof(float2) * mprime, false, st)) != cudaSuccess ||
-            (e = qo->io.ensure(spec, false, st)) != cudaSuccess ||
-            (e = qo->groups.ensure(sizeof(QlGroup) * heads.size(), false, st)) != cudaSuccess)
+        const size_t mode_bytes = (sizeof(int4) * (size_t)mprime + 511) & ~size_t(511);
+        if ((e = qo->lists.ensure(mode_bytes + sizeof(QlGroup) * heads.size(), false, st)) != cudaSuccess ||
+            (e = qo->ghat.ensure(sizeof(float2) * (size_t)mprime, false, st)) != cudaSuccess ||
+            (e = qo->io.ensure(spec + sizeof(int) * src.size(), false, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: buffers"));
-        if ((e = cudaMemcpyAsync(qo->modes.p, modes.data(), sizeof(int4) * mprime, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        qo->modes = (int4 *)qo->lists.p;
+        qo->groups = (QlGroup *)((char *)qo->lists.p + mode_bytes);
+        const float2 *fa = (const float2 *)qo->io.p;           // f^_A
+        const int *dsrc = (const int *)((char *)qo->io.p + spec); // needed only here
+        if ((e = cudaMemcpyAsync(qo->modes, modes.data(), sizeof(int4) * (size_t)mprime, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+            (e = cudaMemcpyAsync((void *)dsrc, src.data(), sizeof(int) * src.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: modes"));
-        DevBuf lm; // the columns' modes, needed only here
-        struct Drop {
-            DevBuf &b;
-            ~Drop() { b.release(); }
-        } drop{lm};
-        if ((e = lm.ensure(sizeof(int4) * places.size(), false, st)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(lm.p, places.data(), sizeof(int4) * places.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
-            return bail(cuda_fail(e, "bc_query_create: columns"));
         // f^_A into the workspace cache, kept in io; then f^_RB into the cache
         std::vector<PairDesc> pairs(1, PairDesc{0, -1, 0, 0, 0});
         if (bc_status s = enqueue(c, std::vector<bc_shape_t>(1, A), std::vector<const float *>(1, nullptr), pairs, true,
@@ -2175,12 +2182,9 @@ bc_status bc_query_create(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *q
         if (bc_status s = enqueue(c, std::vector<bc_shape_t>(1, B), std::vector<const float *>(1, quat), pairs, true,
                                   nullptr, nullptr))
             return bail(s);
-        if ((e = launch_query_gather((const float2 *)qo->io.p, (const float2 *)c->ws.fa.p, (const int4 *)qo->modes.p,
-                                     mprime, N, line_a, c->ws.fa_line, false, (float2 *)qo->ghat.p, st)) != cudaSuccess ||
-            (e = launch_query_gather((const float2 *)qo->io.p, (const float2 *)c->ws.fa.p, (const int4 *)lm.p, (int)places.size(),
-                                     N, line_a, c->ws.fa_line, true, (float2 *)qo->groups.p, st)) != cudaSuccess ||
-            (e = cudaMemcpy2DAsync(qo->groups.p, sizeof(QlGroup), heads.data(), sizeof(QlGroup), QL_HEAD * sizeof(float2),
-                                   heads.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        if ((e = launch_query_gather(fa, (const float2 *)c->ws.fa.p, qo->modes, mprime, N, line_a, c->ws.fa_line, (float2 *)qo->ghat.p, st)) !=
+                cudaSuccess ||
+            (e = launch_query_records((const float2 *)qo->ghat.p, qo->modes, dsrc, qo->ngroups, qo->groups, st)) != cudaSuccess)
             return bail(cuda_fail(e, "bc_query_create: gather"));
         if (bc_status s = bc_sync(c)) return bail(s);
         c->queries.insert(qo);
@@ -2221,9 +2225,8 @@ bc_status bc_query_eval(bc_query_t q, const float *t, int npts, float *g, int on
         // at 2,048, 31 at 4,096, 121 at 20,000) and k_query_lines (14.4, 14.4, 45 us) is
         // the faster one, at any number of modes (64 .. 100,000 measured)
         e = npts > 8 * c->nsm
-                ? launch_query_lines((const QlGroup *)q->groups.p, q->ngroups, q->top, c->period, dt, npts, dg, st)
-                : launch_query_eval((const float2 *)q->ghat.p, (const int4 *)q->modes.p, q->count, c->g.N, c->period, dt, npts,
-                                    dg, st);
+                ? launch_query_lines(q->groups, q->ngroups, q->top, c->period, dt, npts, dg, st)
+                : launch_query_eval((const float2 *)q->ghat.p, q->modes, q->count, c->g.N, c->period, dt, npts, dg, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "bc_query_eval: launch");
         if (!on_device) {

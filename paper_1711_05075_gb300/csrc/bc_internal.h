@@ -191,7 +191,7 @@ void mlp_orphan(bc_mlp_s *net); // bc_mlp.cu
 // Single-configuration queries (bc_query.cu).  modes[i] = (m_x, m_y, m_z, w).
 // line_a, line_b: the spectrum is laid out [m_z][j_y][j_x] instead of [j_x][j_y][m_z].
 cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, bool line_a,
-                                bool line_b, bool weighted, float2 *ghat, cudaStream_t s);
+                                bool line_b, float2 *ghat, cudaStream_t s);
 // Many points: the modes by columns (m_x, m_y), four columns and up to QL_ROWS
 // consecutive m_z from z0 to a record; v: weighted g^ (zero where a column has none).
 constexpr int QL_ROWS = 15;
@@ -201,7 +201,10 @@ struct alignas(16) QlGroup {
     float2 v[QL_ROWS][4];
 };
 static_assert(sizeof(QlGroup) == 512, "one 16-byte copy per lane");
-constexpr int QL_HEAD = 4; // values (of 8 bytes) before v
+constexpr int QL_HEAD = 4, QL_VALUES = 4 * QL_ROWS; // values (of 8 bytes) before v, and of v
+// src: for each record's values the index of the mode, or -1; then the records' heads
+cudaError_t launch_query_records(const float2 *ghat, const int4 *modes, const int *src, int ngroups, QlGroup *out,
+                                 cudaStream_t s);
 // all components below M
 cudaError_t launch_query_lines(const QlGroup *groups, int ngroups, int M, double period, const float *t, int npts, float *g,
                                cudaStream_t s);

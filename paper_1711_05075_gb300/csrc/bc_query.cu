@@ -4,6 +4,7 @@
 // with g^(m) = f^_A(m) conj(f^_RB(m)) (Eq. (ccghat)), M' the first m' modes of
 // the canonical half space ordered outward from the origin, and w_m = 1 for
 // m = 0, 2 otherwise (each mode stands for itself and its conjugate -m).
+#include <algorithm>
 #include <cstdint>
 
 #include "bc_passes.cuh"
@@ -11,10 +12,9 @@
 namespace bc {
 
 // g^ at the listed modes from two half spectra F[jx][jy][mz] (line: F[mz][jy][jx];
-// jx, jy in FFT order, mz in [0, N/2)), times w when weighted; mode i =
-// (m_x, m_y, m_z, w).
+// jx, jy in FFT order, mz in [0, N/2)); mode i = (m_x, m_y, m_z, w).
 __global__ void k_query_gather(const float2 *__restrict__ fa, const float2 *__restrict__ fb, const int4 *__restrict__ modes,
-                               int count, int N, bool line_a, bool line_b, bool weighted, float2 *ghat)
+                               int count, int N, bool line_a, bool line_b, float2 *ghat)
 {
     const int H = N / 2;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
@@ -22,18 +22,49 @@ __global__ void k_query_gather(const float2 *__restrict__ fa, const float2 *__re
         const int jx = m.x < 0 ? m.x + N : m.x, jy = m.y < 0 ? m.y + N : m.y;
         const long long o = ((long long)jx * N + jy) * H + m.z, ol = ((long long)m.z * N + jy) * N + jx;
         const float2 a = fa[line_a ? ol : o], b = fb[line_b ? ol : o];
-        const float2 v = cmulc(a, b);
-        ghat[i] = weighted ? make_float2((float)m.w * v.x, (float)m.w * v.y) : v;
+        ghat[i] = cmulc(a, b);
     }
 }
 
+// The records of k_query_lines: value e of all records is the weighted g^ of mode src[e]
+// (zero for -1); their heads follow the indices.
+__global__ void k_query_records(const float2 *__restrict__ ghat, const int4 *__restrict__ modes, const int *__restrict__ src,
+                                int ngroups, float2 *out)
+{
+    constexpr int PER = QL_HEAD + QL_VALUES;
+    const float2 *heads = reinterpret_cast<const float2 *>(src + (size_t)ngroups * QL_VALUES);
+    const int total = ngroups * PER;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int g = e / PER, k = e - g * PER;
+        float2 v;
+        if (k < QL_HEAD) {
+            v = heads[g * QL_HEAD + k];
+        } else {
+            const int i = src[g * QL_VALUES + k - QL_HEAD];
+            v = i < 0 ? make_float2(0.f, 0.f) : ghat[i];
+            const float w = i < 0 ? 0.f : (float)modes[i].w;
+            v = make_float2(w * v.x, w * v.y);
+        }
+        out[e] = v;
+    }
+}
+
+cudaError_t launch_query_records(const float2 *ghat, const int4 *modes, const int *src, int ngroups, QlGroup *out,
+                                 cudaStream_t s)
+{
+    if (ngroups <= 0) return cudaSuccess;
+    const int total = ngroups * (QL_HEAD + QL_VALUES);
+    k_query_records<<<std::min((total + 255) / 256, 4096), 256, 0, s>>>(ghat, modes, src, ngroups, reinterpret_cast<float2 *>(out));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_query_gather(const float2 *fa, const float2 *fb, const int4 *modes, int count, int N, bool line_a,
-                                bool line_b, bool weighted, float2 *ghat, cudaStream_t s)
+                                bool line_b, float2 *ghat, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
     int blocks = (count + 255) / 256;
     if (blocks > 4096) blocks = 4096;
-    k_query_gather<<<blocks, 256, 0, s>>>(fa, fb, modes, count, N, line_a, line_b, weighted, ghat);
+    k_query_gather<<<blocks, 256, 0, s>>>(fa, fb, modes, count, N, line_a, line_b, ghat);
     return cudaGetLastError();
 }
 
