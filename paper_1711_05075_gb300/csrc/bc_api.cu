@@ -176,6 +176,8 @@ struct bc_ctx_s {
     DevBuf score_ft;                   // shape-complementarity weights for (score_r0, score_lambda)
     DevBuf score_xw, score_wl;         // their x-pass level weights
     double score_r0 = -1.0, score_lambda = 0.0;
+    enum { SCORE_XW = 1, SCORE_WL = 2 };
+    int score_forms = 0;               // the forms of the level weights built for them
     std::set<bc_shape_s *> shapes; // live shapes; orphaned (device memory freed) by bc_destroy
     std::set<bc_mlp_s *> nets;     // live networks; orphaned the same way
     std::set<bc_query_s *> queries; // live single-configuration queries; orphaned the same way
@@ -1274,8 +1276,10 @@ bc_status bc_correlate(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *quat
 }
 
 // The complementarity weights for (r0, lambda), rebuilt on the context stream
-// when the parameters change (stream order keeps earlier calls on the old ones).
-static bc_status score_weights(bc_ctx_t c, double r0, double lambda, const char *who, Weights *w)
+// when the parameters change (stream order keeps earlier calls on the old ones);
+// of the two forms of the level weights the one that the passes over A and B read.
+// A build that is only being recorded does not count as done.
+static bc_status score_weights(bc_ctx_t c, bc_shape_t A, bc_shape_t B, double r0, double lambda, const char *who, Weights *w)
 {
     if (!(r0 >= 0) || !std::isfinite(r0) || !(lambda >= 0) || !std::isfinite(lambda))
         return fail(BC_ERR_ARG, std::string(who) + ": r0 and lambda must be finite and >= 0");
@@ -1285,15 +1289,26 @@ static bc_status score_weights(bc_ctx_t c, double r0, double lambda, const char 
     if ((e = c->score_ft.ensure(sizeof(float) * n, false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
     if ((e = c->score_xw.ensure(sizeof(float) * xw_floats(c->g), false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
     if (c->wl && (e = c->score_wl.ensure(sizeof(float) * wl_floats(c->g), false, c->stream)) != cudaSuccess) return cuda_fail(e, who);
-    if (c->score_ft.bytes != before || r0 != c->score_r0 || lambda != c->score_lambda) {
-        if ((e = launch_build_score_table(c->g, c->period, c->radii_dev, r0, lambda, (float *)c->score_ft.p, c->stream)) != cudaSuccess)
-            return cuda_fail(e, who);
-        if ((e = launch_build_xw(c->g, c->deconv, (const float *)c->score_ft.p, (float *)c->score_xw.p, c->stream)) != cudaSuccess)
-            return cuda_fail(e, who);
-        if (c->wl && (e = launch_build_wl(c->g, c->deconv, (const float *)c->score_ft.p, (float *)c->score_wl.p, c->stream)) != cudaSuccess)
-            return cuda_fail(e, who);
-        c->score_r0 = r0;
-        c->score_lambda = lambda;
+    const bool renew = c->score_ft.bytes != before || r0 != c->score_r0 || lambda != c->score_lambda;
+    const int form = A && B && front_ok(c, {A, B}) ? bc_ctx_s::SCORE_WL : bc_ctx_s::SCORE_XW;
+    if (renew || !(c->score_forms & form)) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if ((e = cudaStreamIsCapturing(c->stream, &capture)) != cudaSuccess) return cuda_fail(e, who);
+        const float *ft = (const float *)c->score_ft.p;
+        if (renew) {
+            c->score_forms = 0;
+            c->score_r0 = -1.0;
+            if ((e = launch_build_score_table(c->g, c->period, c->radii_dev, r0, lambda, (float *)c->score_ft.p, c->stream)) != cudaSuccess)
+                return cuda_fail(e, who);
+        }
+        e = form == bc_ctx_s::SCORE_WL ? launch_build_wl(c->g, c->deconv, ft, (float *)c->score_wl.p, c->stream)
+                             : launch_build_xw(c->g, c->deconv, ft, (float *)c->score_xw.p, c->stream);
+        if (e != cudaSuccess) return cuda_fail(e, who);
+        if (capture == cudaStreamCaptureStatusNone) {
+            c->score_forms |= form;
+            c->score_r0 = r0;
+            c->score_lambda = lambda;
+        }
     }
     w->ballft = (const float *)c->score_ft.p;
     w->xw = (const float *)c->score_xw.p;
@@ -1308,7 +1323,7 @@ bc_status bc_score(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *quats, i
     try {
         if (!c) return fail(BC_ERR_ARG, "bc_score: null context");
         Weights w;
-        if (bc_status s = score_weights(c, r0, lambda, "bc_score", &w)) return s;
+        if (bc_status s = score_weights(c, A, B, r0, lambda, "bc_score", &w)) return s;
         return correlate_impl(c, A, B, quats, k, out, out_on_device, w, "bc_score");
     } catch (...) {
         return fail(BC_ERR_INTERNAL, "bc_score: unexpected exception");
@@ -1406,7 +1421,7 @@ bc_status bc_score_sweep(bc_ctx_t c, bc_shape_t A, bc_shape_t B, const float *qu
         if (batch < 0 || batch > 65534) return fail(BC_ERR_ARG, "bc_score_sweep: batch must be in [0, 65534]");
         if (bc_status s = check_quats(quats, k, "bc_score_sweep")) return s;
         Weights w;
-        if (bc_status s = score_weights(c, r0, lambda, "bc_score_sweep", &w)) return s;
+        if (bc_status s = score_weights(c, A, B, r0, lambda, "bc_score_sweep", &w)) return s;
         return sweep_impl(c, A, B, quats, nullptr, k, batch, peak, argmax, out_on_device, w);
     } catch (...) {
         return fail(BC_ERR_INTERNAL, "bc_score_sweep: unexpected exception");
