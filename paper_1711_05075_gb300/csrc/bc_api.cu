@@ -804,7 +804,6 @@ static Job plan_job(bc_ctx_t c, const std::vector<bc_shape_t> &shapes, const std
         std::memset(&d, 0, sizeof(d));
         d.knot_off = j.koff;
         d.nknots = s->n;
-        d.src_off = 0;
         d.knots = s->knots;
         const int e = cap_extent(c, s->rmax);
         d.cap_e = e;

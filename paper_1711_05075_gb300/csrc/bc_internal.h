@@ -15,7 +15,7 @@ namespace bc {
 struct InstDesc {
     int knot_off;       // first knot of this instance in the prepared-knot array
     int nknots;         // knot count
-    int src_off;        // first knot of its shape in the shape's knot array (always 0)
+    int even;           // 1: the box's y and z extents are rounded up to even (row-pair boxes, bc_front.cu)
     int cap_e;          // per-axis capacity of the compact spreading box
     long long grid_off; // float offset of its spreading boxes (L boxes)
     long long z1_off;   // float2 offset of its z-transformed planes
@@ -23,7 +23,6 @@ struct InstDesc {
     float q[4];         // rotation (w, x, y, z), unit; identity for A
     const float4 *knots; // the shape's knots (x, y, z, level bits)
     const float *qdev;   // when not null: the rotation is read from this device address instead of q
-    int even, pad_;      // 1: the box's y and z extents are rounded up to even (row-pair boxes, bc_front.cu)
 };
 
 // Device-computed support box of one instance in fine-grid cells.

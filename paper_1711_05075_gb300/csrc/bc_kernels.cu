@@ -272,7 +272,7 @@ k_prepare(Geometry g, const InstDesc *__restrict__ inst, int ninst, float4 *ku, 
     const float nf = (float)g.n, halfW = 0.5f * (float)g.W;
     int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
     if (j < d.nknots) {
-        const float4 c = d.knots[d.src_off + j];
+        const float4 c = d.knots[j];
         float p[3];
         p[0] = fmaf(R00, c.x, fmaf(R01, c.y, R02 * c.z));
         p[1] = fmaf(R10, c.x, fmaf(R11, c.y, R12 * c.z));

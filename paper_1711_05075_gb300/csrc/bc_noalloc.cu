@@ -196,7 +196,6 @@ extern "C" bc_status bc_correlate_noalloc(const bc_params *p, const float *xyzA,
         for (int i = 0; i < 2; i++) {
             inst[i].knot_off = i == 0 ? 0 : nA;
             inst[i].nknots = i == 0 ? nA : nB;
-            inst[i].src_off = 0;
             inst[i].cap_e = kn;
             inst[i].grid_off = i * gstride;
             inst[i].z1_off = i * zstride;
