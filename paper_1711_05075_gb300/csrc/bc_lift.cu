@@ -856,9 +856,7 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
         return lift_cuda(e, "bc_lift_correlate: error word");
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return lift_cuda(e, "bc_lift_correlate: sync");
     const int herr = *perr;
-    if (herr) return lift_fail(BC_ERR_TIMEOUT, "bc_lift_correlate: tensor-core contraction stalled (waits " +
-                                                   std::to_string(herr) + ": 1 copy, 2 accumulator, 4 stage, 8 drain); "
-                                                   "the spectrum is incomplete");
+    if (herr) return lift_fail(BC_ERR_TIMEOUT, "bc_lift_correlate: " + lift_stall_message(herr));
     return BC_OK;
 }
 

@@ -2,11 +2,29 @@
 // correlation (bc_lift.cu).  Not part of the public interface.
 #pragma once
 #include <cstddef>
+#include <string>
 #include <cuda_runtime.h>
 
 #include "bc_internal.h"
 
 namespace bc {
+
+// Bits of a lifted call's error word: what a bounded wait that expired was for.
+enum {
+    // the tensor-core contraction (bc_lift_umma.cuh)
+    LIFT_ERR_COPY = 1,        // a free stage for the next copies
+    LIFT_ERR_ACCUMULATOR = 2, // a free accumulator
+    LIFT_ERR_STAGE = 4,       // a stage's copies
+    LIFT_ERR_DRAIN = 8,       // a unit's products
+    // the 4D NUFFT's line passes (bc_lift_line.cu)
+    LIFT_ERR_LINE = 16        // their copies
+};
+inline std::string lift_stall_message(int word)
+{
+    const std::string incomplete = "; the spectrum is incomplete";
+    if (word & LIFT_ERR_LINE) return "a pass of the 4D NUFFT stalled (a bounded wait for its copies expired)" + incomplete;
+    return "tensor-core contraction stalled (waits " + std::to_string(word) + ": 1 copy, 2 accumulator, 4 stage, 8 drain)" + incomplete;
+}
 
 struct Lift4Rot {
     double R[9];
@@ -54,7 +72,7 @@ size_t lift4_ws_bytes(int N, int Nr);
 // ((3 (N/2)^2 + 1) x N_r), slices = device sections, scale = P^-3 P_r^-1; ws of
 // lift4_ws_bytes(N, Nr) bytes.  Synchronises s once (to size the support boxes).
 // With *line set on return h is [s][k_x][m_z][j_y] instead, the inverse transform
-// along x done (what launch_iyz takes); *err gets bit 8 if a bounded wait expired.
+// along x done (what launch_iyz takes); *err gets LIFT_ERR_LINE if a bounded wait expired.
 // lift4_boxes first: it enqueues the search for the two shapes' support boxes.
 cudaError_t lift4_boxes(const Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, const float4 *kB, int nB,
                         const double (&RB)[9], double period, double period_r, int nsm, cudaStream_t s);

@@ -26,7 +26,6 @@ namespace bc {
 namespace {
 
 constexpr int LW8 = 8; // window width
-constexpr int LX_ERR = 8;
 
 // 4W window weights by the lanes; then a lane owns one 16-byte piece of the (y, z)
 // cross-section -- a row pair and two z cells -- for all W x W cells along r and x.
@@ -116,7 +115,7 @@ k_lx_x(const float2 *__restrict__ y1, int b0, int bR, const float2 *__restrict__
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         // the stage of the previous item is free (the barrier that ended it)
         if (threadIdx.x == 0) fetch(it + (STAGES - 1) * (int)gridDim.x, (st + STAGES - 1) % STAGES);
-        if (!__syncthreads_and(umma_wait(FULL + 8 * st, par, stop, err, LX_ERR))) break;
+        if (!__syncthreads_and(umma_wait(FULL + 8 * st, par, stop, err, LIFT_ERR_LINE))) break;
         const float2 *T = ring + (size_t)st * b0 * XL;
         const int ir = it / (H * nch), rem = it - ir * H * nch, mz = rem / nch, jy0 = (rem - mz * nch) * XL;
         wf_first_any<NF>(E, lane, qx, [&](int sl, int ix, bool inside) {
@@ -263,7 +262,7 @@ k_lx_rx(const float2 *__restrict__ XA, const float2 *__restrict__ XB, int bA, in
     for (int u = 0; u < total; u++) {
         const int it = blockIdx.x + (u / XL) * gridDim.x, mz = it / nch, c = u % XL, jy = (it - mz * nch) * XL + c;
         if (threadIdx.x == 0) fetch(u + 1); // its stage was read before the barrier inside unit u - 1
-        if (!__syncthreads_and(umma_wait(FULL + 8 * (u & 1), (u >> 1) & 1, stop, err, LX_ERR))) break;
+        if (!__syncthreads_and(umma_wait(FULL + 8 * (u & 1), (u >> 1) & 1, stop, err, LIFT_ERR_LINE))) break;
         const float2 *TA = stg + (size_t)(u & 1) * sf2 + jx, *TB_ = TA + bA * N;
         const int my = jy < H ? jy : jy - N;
         const float2 *wt = wts + ((long long)mz * A + (my < 0 ? -my : my)) * NRK * A + ax;

@@ -188,7 +188,7 @@ k_lift_gemm_umma(const float *__restrict__ ahi, const float *__restrict__ alo, c
                 for (int kb = w.kb0; kb < w.kb1 && ok; kb++)
                     for (int h = 0; h < 2; h++, it++) {
                         const int s = it & 1;
-                        if (!umma_wait(b0 + 16 + 8 * s, ((it >> 1) & 1) ^ 1, stop, err, 1)) {
+                        if (!umma_wait(b0 + 16 + 8 * s, ((it >> 1) & 1) ^ 1, stop, err, LIFT_ERR_COPY)) {
                             ok = false;
                             break;
                         }
@@ -221,8 +221,8 @@ k_lift_gemm_umma(const float *__restrict__ ahi, const float *__restrict__ alo, c
                 for (int kb = w.kb0; kb < w.kb1 && ok; kb++)
                     for (int h = 0; h < 2; h++, it++) {
                         const int s = it & 1;
-                        if (!umma_wait(b0 + 48 + 8 * s, ((it >> 1) & 1) ^ 1, stop, err, 2) ||
-                            !umma_wait(b0 + 8 * s, (it >> 1) & 1, stop, err, 4)) {
+                        if (!umma_wait(b0 + 48 + 8 * s, ((it >> 1) & 1) ^ 1, stop, err, LIFT_ERR_ACCUMULATOR) ||
+                            !umma_wait(b0 + 8 * s, (it >> 1) & 1, stop, err, LIFT_ERR_STAGE)) {
                             ok = false;
                             break;
                         }
@@ -262,7 +262,7 @@ k_lift_gemm_umma(const float *__restrict__ ahi, const float *__restrict__ alo, c
             for (int kb = w.kb0; kb < w.kb1 && ok; kb++)
                 for (int h = 0; h < 2; h++, it++) {
                     const int s = it & 1;
-                    ok = __all_sync(0xffffffffu, umma_wait(b0 + 32 + 8 * s, (it >> 1) & 1, stop, err, 8));
+                    ok = __all_sync(0xffffffffu, umma_wait(b0 + 32 + 8 * s, (it >> 1) & 1, stop, err, LIFT_ERR_DRAIN));
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll
