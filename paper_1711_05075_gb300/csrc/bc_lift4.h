@@ -38,14 +38,16 @@ struct Lift4Box {
 
 #ifdef __CUDACC__
 // Fine-grid coordinate of knot c on axis a (0, 1, 2: rotated x, y, z; 3: r,
-// mirrored for B), half a period on.
+// mirrored for B), half a period on.  Every product and sum is spelled out: the box
+// search and the spreading must get the same bits, or a knot on a cell's edge could lie
+// one cell outside its box (left to the compiler, each kernel contracts them its own way).
 __device__ __forceinline__ double lift4_coord(const float4 &c, int a, const double (&R)[9], int mirror, int ns, int nr,
                                               double inv_p, double inv_pr)
 {
     double v;
-    if (a < 3) v = (R[3 * a] * c.x + R[3 * a + 1] * c.y + R[3 * a + 2] * c.z) * inv_p + 0.5;
-    else v = (mirror ? -(double)c.w : (double)c.w) * inv_pr + 0.5;
-    return (v - floor(v)) * (a < 3 ? ns : nr);
+    if (a < 3) v = __fma_rn(__fma_rn(R[3 * a + 2], c.z, __fma_rn(R[3 * a + 1], c.y, __dmul_rn(R[3 * a], c.x))), inv_p, 0.5);
+    else v = __fma_rn(mirror ? -(double)c.w : (double)c.w, inv_pr, 0.5);
+    return __dmul_rn(__dsub_rn(v, floor(v)), a < 3 ? ns : nr);
 }
 #endif
 
