@@ -746,7 +746,7 @@ bc_status bc_lift_correlate(bc_lift_t lf, const float *A, int nA, const float *B
     const double R[9] = {1 - 2 * (qy * qy + qz * qz), 2 * (qx * qy - qw * qz), 2 * (qx * qz + qw * qy),
                          2 * (qx * qy + qw * qz), 1 - 2 * (qx * qx + qz * qz), 2 * (qy * qz - qw * qx),
                          2 * (qx * qz - qw * qy), 2 * (qy * qz + qw * qx), 1 - 2 * (qx * qx + qy * qy)};
-    // the boxes go first: the host waits for them, the copies that follow need not be waited for
+    // the boxes go first: the device searches them while the host enqueues the copies below (lift4_pair waits for all of it)
     if (lf->contraction == 3 && (e = lift4_boxes(lf->t4, N, Nr, kA, nA, kB, nB, R, lf->period, lf->period_r, lf->nsm, st)) !=
                                     cudaSuccess)
         return lift_cuda(e, "bc_lift_correlate: support boxes");
