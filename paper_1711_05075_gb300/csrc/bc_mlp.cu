@@ -1364,6 +1364,7 @@ bc_status ensure_batch(bc_mlp_t net, int n)
 {
     const size_t H = net->H, cap = (size_t)n + n / 4 + 64;
     const bool fused = net->wp && n <= TR_MAX_ROWS;
+    if (!net->g) MCK(cudaMalloc(&net->g, sizeof(float) * (size_t)net->off.total));
     if (n > net->ycap) {
         net->ycap = 0;
         MCK(regrow(net->y, cap));
@@ -1759,8 +1760,8 @@ cudaError_t bc::launch_axpby(float *y, const float *x, int n, float alpha, float
 
 void bc::mlp_orphan(bc_mlp_s *net)
 {
-    // p heads the allocation that also holds m, v, g, loss and wp
-    float *bufs[] = {net->p, net->h1, net->h2, net->y, net->gy, net->dh2, net->dh1, net->part, net->xb, net->tb};
+    // p heads the allocation that also holds m, loss that of wp
+    float *bufs[] = {net->p, net->v, net->g, net->loss, net->h1, net->h2, net->y, net->gy, net->dh2, net->dh1, net->part, net->xb, net->tb};
     for (float *b : bufs)
         if (b) cudaFree(b);
     net->p = net->m = net->v = net->g = net->h1 = net->h2 = net->y = net->gy = net->dh2 = net->dh1 = net->loss = nullptr;
@@ -1787,17 +1788,18 @@ bc_status bc_mlp_create(bc_ctx_t ctx, int hidden, const float *init, bc_mlp_t *o
         const size_t bytes = sizeof(float) * (size_t)net->off.total;
         cudaStream_t s = ctx_stream(ctx);
         cudaError_t e;
-        // one allocation: parameters, Adam moments, gradients, the loss word, BF16 weight blocks
+        // parameters and first moments; second moments; the loss word and the BF16 weight blocks.
+        // (At H = 256 these stay below the 2 MB that cudaMalloc maps at a time; with the
+        // gradients, which come with the first training pass, a network took 160 us, not 40.)
         const size_t row = (size_t)((net->off.total + 63) & ~63LL), fused = hidden <= FW_MAXH;
         const size_t wbytes = fused ? (size_t)(3 + 2 * (fw_hp(hidden) / 64)) * hidden * 128 : 0;
-        if ((e = cudaMalloc(&net->p, sizeof(float) * (4 * row + 64) + wbytes)) != cudaSuccess) {
+        if ((e = cudaMalloc(&net->p, sizeof(float) * 2 * row)) != cudaSuccess ||
+            (e = cudaMalloc(&net->v, bytes)) != cudaSuccess ||
+            (e = cudaMalloc(&net->loss, sizeof(float) * 64 + wbytes)) != cudaSuccess) {
             bc_mlp_destroy(net);
             return mcuda(e, "bc_mlp_create: cudaMalloc");
         }
         net->m = net->p + row;
-        net->v = net->m + row;
-        net->g = net->v + row;
-        net->loss = net->g + row;
         if (fused) {
             net->wp = reinterpret_cast<uint8_t *>(net->loss + 64);
             if ((e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fw_smem(FW_MAXH))) != cudaSuccess ||
