@@ -96,16 +96,19 @@ k_spread_rp(const float *__restrict__ consts, const InstDesc *__restrict__ inst,
 // Bound by instructions and the latency between them (issue 63%, 127 registers, two
 // blocks per SM).  20,000 + 20,000 balls, N = 128: 46.9 us against 39.9 + 31.5 us of
 // the tensor-core z pass and the staged y pass, whose rows crossed device memory
-// twice; with block barriers in place of the warps' own tiles 85 us.
+// twice; with block barriers in place of the warps' own tiles 85 us.  Two lines per warp
+// in place of all it can take, for grids whose planes are all resident at once, gain
+// nothing (128 + 128 balls at N = 32, two levels: a correlation 22.6 us either way) or
+// cost (2,000 + 2,000, one level: 22.6 against 20.7).
 constexpr int ZY_WARPS = 8;
 
-template <int NF, int LW>
+template <int NF>
 __global__ void __launch_bounds__(ZY_WARPS * 32, 2)
 k_zy(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const InstPlan *__restrict__ plan,
      float *grid, float2 *y1, int PS, bool clear)
 {
-    using F = WF<NF, LW>;
-    constexpr int R0 = F::R0, H = F::H, N = F::N;
+    using F = WF<NF>;
+    constexpr int R0 = F::R0, H = F::H, N = F::N, LW = F::LW;
     extern __shared__ float4 sm4[];
     float2 *P = reinterpret_cast<float2 *>(sm4); // [H][PS]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -128,12 +131,12 @@ k_zy(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const 
         for (int it = rs.first(); it < planes; it += gridDim.x) {
             float2 *G2 = reinterpret_cast<float2 *>(grid + d.grid_off) + (long long)it * np * bz;
             for (int q0 = warp * LW; q0 < np; q0 += ZY_WARPS * LW) {
-                wf_first_any<NF, LW>(E, lane, qz, [&](int sl, int iz, bool inside) {
+                wf_first_any<NF>(E, lane, qz, [&](int sl, int iz, bool inside) {
                     return (inside || iz < bz) && q0 + sl < np ? G2[(q0 + sl) * bz + iz] : make_float2(0.f, 0.f);
                 });
                 __syncwarp();
                 float2 o[16], m[4];
-                wf_last<NF, 15, LW>(E, lane, w, o);
+                wf_last<NF>(E, lane, w, o);
 #pragma unroll
                 for (int r = 0; r < 4; r++) {
                     m[r].x = __shfl_sync(0xffffffffu, o[15 - r].x, mate & 31);
@@ -162,12 +165,12 @@ k_zy(Geometry g, Tables tb, const InstDesc *__restrict__ inst, int ninst, const 
             const int l = it / b0, ix = it - l * b0;
             float2 *Y = y1 + d.y1_off + ((long long)l * H * (N / XL) * b0 + ix) * XL;
             for (int k0 = warp * LW; k0 < H; k0 += ZY_WARPS * LW) {
-                wf_first_any<NF, LW>(E, lane, qy, [&](int sl, int iy, bool inside) {
+                wf_first_any<NF>(E, lane, qy, [&](int sl, int iy, bool inside) {
                     return inside || iy < b1 ? P[(k0 + sl) * PS + iy] : make_float2(0.f, 0.f);
                 });
                 __syncwarp();
                 float2 o[16];
-                wf_last<NF, 15, LW>(E, lane, w, o);
+                wf_last<NF>(E, lane, w, o);
                 if (lane < F::LIVE) {
                     float2 *Yk = Y + (long long)(k0 + s) * N * b0;
 #pragma unroll
@@ -199,10 +202,10 @@ static int zy_ps(int cap)
     return 2 * (h | 1);
 }
 
-template <int NF, int LW>
+template <int NF>
 static size_t zy_smem(int cap)
 {
-    return sizeof(float2) * ((size_t)WF<NF>::H * zy_ps(cap) + (size_t)ZY_WARPS * WF<NF, LW>::EW);
+    return sizeof(float2) * ((size_t)WF<NF>::H * zy_ps(cap) + (size_t)ZY_WARPS * WF<NF>::EW);
 }
 
 bool front_fits(const Geometry &g, int cap) { return supported_front(g) && cap + 2 <= g.n; }
@@ -233,20 +236,14 @@ cudaError_t launch_spread_rp(const Geometry &g, const Tables &t, const InstDesc 
     }
 }
 
-template <int NF, int LW = wf_full(NF)>
+template <int NF>
 static cudaError_t zy_t(const Geometry &g, const Tables &t, const InstDesc *inst, int ninst, const InstPlan *plan,
                         float *grid, float2 *y1, int cap, int nsm, cudaStream_t s, bool clear)
 {
-    // where every plane may be resident at once, idle lanes cost nothing and the shorter
-    // steps of two lines per warp shorten the pass (128 + 128 balls at N = 32, whole
-    // correlation: 22.4 us, with eight lines 23.5)
-    if constexpr (LW > 2)
-        if ((long long)ninst * g.L * cap <= 2LL * nsm)
-            return zy_t<NF, 2>(g, t, inst, ninst, plan, grid, y1, cap, nsm, s, clear);
-    const size_t smem = zy_smem<NF, LW>(cap);
-    cudaError_t e = set_smem(k_zy<NF, LW>, zy_smem<NF, LW>(NF)); // cap <= NF
+    const size_t smem = zy_smem<NF>(cap);
+    cudaError_t e = set_smem(k_zy<NF>, zy_smem<NF>(NF)); // cap <= NF
     if (e != cudaSuccess) return e;
-    return launch_k(k_zy<NF, LW>, resident_blocks(k_zy<NF, LW>, smem, nsm, ZY_WARPS * 32), ZY_WARPS * 32, smem, s,
+    return launch_k(k_zy<NF>, resident_blocks(k_zy<NF>, smem, nsm, ZY_WARPS * 32), ZY_WARPS * 32, smem, s,
                     g.pdl != 0, g, t, inst, ninst, plan, grid, y1, zy_ps(cap), clear);
 }
 
