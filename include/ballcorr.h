@@ -214,8 +214,10 @@ bc_status bc_score_sweep(bc_ctx_t ctx, bc_shape_t A, bc_shape_t B, const float *
  * another context, m' outside [1, ((N-1)^3 + 1) / 2]), BC_ERR_OOM, BC_ERR_CUDA.
  * bc_query_eval: t = npts x 3 FP32 translations, g = npts FP32 results, both
  * device (on_device = 1, asynchronous on ctx's stream) or host (0,
- * synchronous) memory; any t is allowed (g' is P-periodic).  Errors:
- * BC_ERR_ARG (null pointer, npts outside [1, 2^26], context destroyed),
+ * synchronous) memory; any t is allowed (g' is P-periodic).  Calls of many
+ * points (beyond eight per multiprocessor) sum the modes in another order, so a
+ * point's result can differ in its last bits with the number of points beside it.
+ * Errors: BC_ERR_ARG (null pointer, npts outside [1, 2^26], context destroyed),
  * BC_ERR_CUDA.  bc_query_destroy waits for the context stream. */
 typedef struct bc_query_s *bc_query_t;
 bc_status bc_query_create(bc_ctx_t ctx, bc_shape_t A, bc_shape_t B, const float *quat, int mprime, bc_query_t *out);
@@ -311,9 +313,9 @@ bc_status bc_lift_destroy(bc_lift_t lift);
  *                in FP32 contexts with N <= 128 (BC_ERR_UNSUPPORTED otherwise);
  *                a stalled tensor-core wait is reported by bc_sync as
  *                BC_ERR_TIMEOUT.
- *                With spread 0 and persistent 0 and shapes that fit inside
- *                one period (no stencil wraps: 2 n |c|_max / P + W + 4 <= n),
- *                1 stands for a pass of four launches after the knots'
+ *                With spread 0 and persistent 0 and shapes that all (of the call)
+ *                fit inside one period (no stencil wraps: 2 n |c|_max / P + W + 4
+ *                <= n), 1 stands for a pass of four launches after the knots'
  *                preparation instead: spreading into row-pair boxes, the z and
  *                y transforms of each (level, x) plane in shared memory, the x
  *                pass, the inverse y and z transforms of whole planes

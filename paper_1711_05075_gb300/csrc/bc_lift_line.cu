@@ -10,8 +10,8 @@
 // whose spatial part the last pass applies per mode and whose r part is folded
 // into the sections' phases.  (The half-period shift of the coordinates cancels.)
 //
-// A call at N = 128, N_r = 32 with 5,000 + 5,000 knots: 0.71 ms, against
-// 1.82-1.95 ms of the passes in bc_lift_nufft.cu (spreading 33 us a shape, z and y
+// A call at N = 128, N_r = 32 with 5,000 + 5,000 knots: 0.74 ms, against
+// 1.95 ms of the passes in bc_lift_nufft.cu (spreading 33 us a shape, z and y
 // 108, x 55, the last pass 206: instruction bound).
 #include <algorithm>
 #include <climits>

@@ -472,7 +472,7 @@ cudaError_t lift4_pair(Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, 
     if (*line) {
         // spectra in turn over the same grid and y planes; A's x planes have their own
         // place, B's take the grid's, which only A's passes have to leave clear
-        // (with the boxes in one launch: 764 -> 706 us at N = 128, N_r = 32)
+        // (a launch and a wait per box and a second clear: 761 us at N = 128, N_r = 32, now 737)
         InstPlan *hp = (InstPlan *)(t.hbox + 16), *dp = (InstPlan *)(t.dbox + 16);
         const InstDesc *dd = (const InstDesc *)(dp + 2); // offsets zero
         static_assert(16 * sizeof(int) + 2 * sizeof(InstPlan) + 2 * sizeof(InstDesc) <= LIFT4_BOX_BYTES, "box words");

@@ -456,7 +456,8 @@ static cudaError_t xw_t(const Geometry &g, const Tables &t, const InstDesc *inst
                         float2 *h, int cap, int *err, int nsm, cudaStream_t s)
 {
     // where every item has an SM to itself, idle lanes cost nothing and the shorter steps
-    // of two lines per warp shorten the pass.  Up to four items per SM (256 or 448
+    // of two lines per warp shorten the pass (a pair at N = 32 22.6 us, with eight lines
+    // 25.3).  Up to four items per SM (256 or 448
     // items) the fewer warps are the faster ones: a score at N = 64 with 5 rotations 69.9
     // us with two lines per warp, 67.7 with four; 7 rotations at N = 32 32.5 and 31.0;
     // only a single pair at N = 64 (256 items) gains from two: 38.7 against 39.2

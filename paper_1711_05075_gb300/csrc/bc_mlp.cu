@@ -919,7 +919,7 @@ k_mlp_forward(const float *__restrict__ X, int n, int H, int hp, int tcols, cons
 // that are not in use: W1, then W2 around the dh2 tile, W2^T around the h1 tile
 // (its ReLU mask is kept as bits).  Before it took five products and five other
 // launches with every operand through FP32 device memory: 117.6 us for 8,192 rows,
-// H = 256, now 40.  What is left is the latency of one block's chain (five products,
+// H = 256, now 43.  What is left is the latency of one block's chain (five products,
 // five epilogues) on 64 of the 152 SMs.
 constexpr int TR_TILES = 11; // 16 KB tiles: X 0-2, h 3-6, d 7-10
 constexpr int TR_MAX_ROWS = 1 << 15; // partials of 400 KB per 128 rows at H = 256

@@ -10,8 +10,9 @@
 // (8 MiB), enough for N = 32, two radius levels and 8192 knots per shape.
 // Every GPU that loads the library holds that array until the process exits.
 //
-// The kernels are the ones bc_correlate launches; only their scratch pointers
-// differ.  All calls share the one array: two calls whose work overlaps on
+// The kernels are the general ones that bc_correlate launches for shapes that reach
+// across the period (the passes of bc_front.cu are not used); only their scratch
+// pointers differ.  All calls share the one array: two calls whose work overlaps on
 // the GPU (different streams, or different host threads) race on it and give
 // wrong results.  The parts that must start at a known state (the spreading
 // boxes, the support-box accumulators, the status words) are reset by every call.
