@@ -1940,6 +1940,7 @@ bc_status bc_autotune(bc_ctx_t c, bc_shape_t A, bc_shape_t B, int rotations, bc_
         if (A->ctx != c || B->ctx != c) return fail(BC_ERR_ARG, "bc_autotune: shapes belong to another context");
         if (rotations < 0 || rotations > 65534) return fail(BC_ERR_ARG, "bc_autotune: rotations must be in [0, 65534]");
         CK(cudaStreamSynchronize(c->stream));
+        prof_free(c); // a profiled pass is not the one that is timed
         const long long N3 = (long long)c->g.N * c->g.N * c->g.N;
         cudaError_t e;
         if ((e = c->tune.ensure(sizeof(float) * (size_t)std::max<long long>(N3, 2LL * rotations), false, c->stream)) != cudaSuccess)

@@ -31,6 +31,16 @@ def test_finds_the_fastest_combination_and_keeps_the_schedule(N, before, rotatio
     ctx.close()
 
 
+def test_profiling_ends():
+    import paper_1711_05075_gb300 as bc
+    ctx, a, b = context(bc, 32, n=100)
+    bc.bc_profile_begin(ctx.handle, 4)
+    ctx.autotune(a, b)
+    with pytest.raises(bc.BallCorrError):
+        bc.bc_profile_end(ctx.handle)
+    ctx.close()
+
+
 def test_across_the_period_the_schedule_is_chosen():
     import paper_1711_05075_gb300 as bc
     ctx, a, b = context(bc, 128, (0.99, 0.3, 0.7))
