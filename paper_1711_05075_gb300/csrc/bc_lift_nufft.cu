@@ -463,7 +463,11 @@ cudaError_t lift4_pair(Lift4Tables &t, int N, int Nr, const float4 *kA, int nA, 
         float2 *w = nullptr;
         if (cudaMalloc(&w, lift4_weight_bytes(N, Nr)) == cudaSuccess) {
             t.wts = w;
-            if ((e = lift4_build_weights(t, N, Nr, cone, s)) != cudaSuccess) return e;
+            if ((e = lift4_build_weights(t, N, Nr, cone, s)) != cudaSuccess) {
+                cudaFree(w);
+                t.wts = nullptr;
+                return e;
+            }
         } else {
             cudaGetLastError();
             *line = false;
